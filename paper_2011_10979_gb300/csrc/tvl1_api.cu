@@ -69,7 +69,8 @@ Plan make_plan(int H, int W, const of_params *p) {
         const Geom g{pl.H[l], pl.W[l], pl.P[l]};
         mb = std::max({mb, admm_fused_blocks(g, p->rows_per_warp != 0 ? 1 : 0), admm_plain_blocks(g),
                        pdr_plain_blocks(g, PARTIAL_ROWS_MIN), cp_blocks(g, PARTIAL_ROWS_MIN), energy_blocks(g),
-                       adapt_blocks(g), admm_tile2_blocks(g), pdr_tile_blocks(g), cp_tile_blocks(g)});
+                       adapt_blocks(g), admm_tile_blocks(admm_tile_plan(g, 0)),
+                       admm_tile_blocks(admm_tile_plan(g, TILE_ITERS)), pdr_tile_blocks(g), cp_tile_blocks(g)});
     }
     pl.max_blocks = mb;
     pl.partials = take(3 * (size_t)mb * sizeof(double));
@@ -285,21 +286,19 @@ bool pdr_tile_of(const of_params *p) {
 // 2.7 / 4.3 at 80x60, 4.3 / 4.3 at 120x90, 6.0 / 4.4 at 160x120).
 constexpr long PDR_TILE_RESIDENT_MAX_PX = 12000;
 
-// Whether a single pair's streamed ADMM level runs several iterations per launch (k_admm_tile.cu):
+// Whether a single pair's streamed ADMM level runs several iterations per launch (k_admm_tile.cuh):
 // the built-in strip rule (a pinned or autotuned height asks for the row-streaming kernel), at any
-// size.  Measured per iteration against the row-streaming kernel (2-row strips at 640x480 and
-// below, 8-row above): 320x240 2.34 against 3.99 us, 640x480 5.41 against 7.98, 1024x436 7.82
-// against 9.27, 1920x1080 35.2 against 39.9 (DRAM-bound: the state is read and written once per
-// three iterations); 1242x375 9.40 against 9.27 and 960x540 9.92 against 9.63 are the exceptions,
-// within 3%.
-// Iterations per launch (the last launch of a warp may run 2, or 1).  Measured per iteration at
-// 640x480 / 320x240: 7.86 / 3.21 us with 2, 6.72 / 2.78 with 3, 7.13 / 3.01 with 4 (a 41 x 41
-// frame: 64 registers and 108 KB of shared memory per block, and a third more halo work).
-constexpr int TILE_ITERS = 3;
-
-bool admm_tile2_of(const of_params *p, bool batched, Geom) {
+// size.
+bool admm_tile_of(const of_params *p, bool batched) {
     return !batched && (p->method == OF_PADMM_I || p->method == OF_PADMM_II) && p->rows_per_warp == 0 &&
            (p->engine == OF_ENGINE_FUSED || p->engine == OF_ENGINE_STREAM);
+}
+
+// Iterations per launch of the tile kernel for a warp of `iters` iterations: the level's choice
+// (admm_tile_plan; 0), or TILE_ITERS on the streaming engine, with the stopping test (every ten
+// iterations run as launches of 3, 3, 3 and 1) and for warps of up to ten iterations.
+int tile_iters_of(const of_params *p, int iters) {
+    return p->engine == OF_ENGINE_STREAM || p->tol > 0.0 || iters <= 10 ? TILE_ITERS : 0;
 }
 
 // Whether a single pair's streamed ALG1 level runs several iterations per launch (k_cp_tile.cu):
@@ -325,7 +324,7 @@ bool use_resident(const of_params *p, Geom g, bool batched = false) {
     if (p->engine == OF_ENGINE_RESIDENT) return true;
     if (p->engine != OF_ENGINE_FUSED && p->engine != OF_ENGINE_PERSISTENT) return false;
     if (pdr_tile_of(p)) return (long)g.H * g.W <= PDR_TILE_RESIDENT_MAX_PX;
-    if (admm_tile2_of(p, batched, g)) return (long)g.H * g.W <= TILE_RESIDENT_MAX_PX;
+    if (admm_tile_of(p, batched)) return (long)g.H * g.W <= TILE_RESIDENT_MAX_PX;
     if (cp_tile_of(p, batched)) return (long)g.H * g.W <= CP_TILE_RESIDENT_MAX_PX;
     return admm_resident_preferred(g, p->method);
 }
@@ -910,18 +909,27 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
             // the non-resident pairs (ALG1)
             const bool streamed = !persl && (batched ? ((cp || pdr) ? B.nres[l] < n : B.ntiles[l] > 0) : !res1);
             // single pair, ADMM or ALG1, the built-in strip rule or block height: several iterations
-            // per launch (k_admm_tile.cu, k_cp_tile.cu).  With the
+            // per launch (k_admm_tile.cuh, k_cp_tile.cu).  With the
             // stopping test every ten iterations run as launches of 3, 3, 3 and 1: the tested state
             // is a single-iteration launch's (its residual partials), an even number of launches
             // leaves it in bufs[start2] as on the one-launch-per-iteration path, and the warp's last
             // launch is a single iteration too, so the final residual sums the same partials
             // whether or not the test stopped the warp.
-            const bool tile2 = streamed && (admm_tile2_of(p, batched, geom_of(*pc[0].pl, l)) || cp_tile_of(p, batched));
+            const bool tile = streamed && admm_tile_of(p, batched), tile2 = tile || (streamed && cp_tile_of(p, batched));
+            TilePlan tp;
+            CUtensorMap maps[2][3];
+            if (tile) {
+                const PairCtx &c = pc[0];
+                const Geom g = geom_of(*c.pl, l);
+                tp = admm_tile_plan(g, tile_iters_of(p, rest));
+                for (int b = 0; b < 2 && tp.staged; ++b)
+                    tp.staged = tile_encode_maps(maps[b], bufs_of(c)[b], data_of(c)[0], data_of(c)[1], g, prec, pflow, has_w, tp.R);
+            }
             int par = start2, last_nb = 0;  // the several-iterations path's buffer parity and last block count
             for (int it = 0, step = 1; streamed && it < rest; it += step) {
                 step = 1;
                 if (tile2) {
-                    step = std::min(TILE_ITERS, rest - it);
+                    step = std::min(tile ? tp.ni : TILE_ITERS, rest - it);
                     if (p->tol > 0.0) {
                         step = std::min(step, 10 - it % 10);
                         if (step > 1 && it + step == rest) --step;
@@ -960,16 +968,22 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                             launch_cp(a, prec, pflow, s);
                             last_nb = blocks_of(g, l);
                         }
-                    } else if (step > 1) {
-                        launch_admm_tile2(a, step, prec, pflow, s);
-                        last_nb = admm_tile2_blocks(g);
+                    } else if (tile) {
+                        TileArgs t{};
+                        t.a = a;
+                        tile_set_plan(t, tp, step);
+                        t.vec = 1;
+                        t.timeout = &c.misc->timeout;
+                        if (tp.staged) memcpy(t.maps, maps[par ^ 1], sizeof(t.maps));  // par is the next launch's by now
+                        launch_admm_tile(t, prec, pflow, s);
+                        last_nb = admm_tile_blocks(tp);
                     } else {
                         if (plain) launch_admm_plain(a, s);
                         else launch_admm_fused(a, prec, pflow, s);
                         last_nb = blocks_of(g, l);
                     }
                     if (check) {
-                        const int nb = step > 1 ? (cp ? cp_tile_blocks(g) : admm_tile2_blocks(g)) : blocks_of(g, l);
+                        const int nb = tile ? admm_tile_blocks(tp) : cp && step > 1 ? cp_tile_blocks(g) : blocks_of(g, l);
                         const double rows = (double)g.H * g.W * (has_w ? 3.0 : 2.0);
                         launch_reduce_check(c.partials, nb, &c.misc->res_check, rows, p->tol, &c.misc->done,
                                             &c.misc->iters, 10, s);
@@ -1708,7 +1722,9 @@ of_status iterate_common(of_fields f, const float *Ix, const float *Iy, const fl
     const int mb = fields_partial_slots(H, pitch);
     const int nb_used = pdr ? pdr_plain_blocks(g)
                             : cp ? cp_blocks(g)
-                                 : (params->engine == OF_ENGINE_PLAIN ? admm_plain_blocks(g) : admm_fused_blocks(g));
+                                 : (params->engine == OF_ENGINE_PLAIN
+                                        ? admm_plain_blocks(g)
+                                        : admm_tile_blocks(admm_tile_plan(g, params->tol > 0.0 ? TILE_ITERS : 0)));
     if (nb_used > mb) return fail(OF_EINVAL, "internal: partial sums exceed the scratch layout");
     double *partials = (double *)(S + (NFIELDS + 6) * plane);
     Misc *misc = (Misc *)(S + (NFIELDS + 6) * plane + align_up((size_t)mb * sizeof(double), 256));
@@ -1722,18 +1738,40 @@ of_status iterate_common(of_fields f, const float *Ix, const float *Iy, const fl
     pp.a_tilde = xb ? 1.f : a_tilde;
     const Coefs k = coefs_of(&pp);
     const double rows = (double)H * W * (has_w ? 3.0 : 2.0);
-    for (int it = 0; it < iters; ++it) {
-        const bool check = params->tol > 0.0 && (it + 1) % 10 == 0;
+    // ADMM, fused engines: the tile kernel straight from the caller's planes (8-byte loads where every
+    // plane and row allows them), several iterations per launch
+    const bool tile = !xb && !plain;
+    TilePlan tp;
+    bool vec = W % 2 == 0 && pitch % 2 == 0;
+    if (tile) {
+        tp = admm_tile_plan(g, params->tol > 0.0 ? TILE_ITERS : 0);
+        for (int q = 0; q < NFIELDS; ++q) vec = vec && (uintptr_t)user.f[q] % 8 == 0;
+        vec = vec && (uintptr_t)Ix % 8 == 0 && (uintptr_t)Iy % 8 == 0 && (uintptr_t)It % 8 == 0 && (uintptr_t)scratch % 8 == 0;
+        tp.staged = false;
+    }
+    int launches = 0;
+    for (int it = 0, step = 1; it < iters; it += step, ++launches) {
+        step = 1;
+        if (tile) {
+            step = std::min(tp.ni, iters - it);
+            // an even number of launches leaves the state in the caller's planes
+            if (it + step == iters && step > 1 && launches % 2 == 0) --step;
+            if (params->tol > 0.0) {
+                step = std::min(step, 10 - it % 10);
+                if (step > 1 && it % 10 + step == 10) --step;
+            }
+        }
+        const bool check = params->tol > 0.0 && (it + step) % 10 == 0;
         IterArgs a{};
         a.g = g;
         a.k = k;
-        a.in = bufs[pingpong ? it & 1 : 0];
-        a.out = bufs[pingpong ? (it + 1) & 1 : 0];
+        a.in = bufs[pingpong ? launches & 1 : 0];
+        a.out = bufs[pingpong ? (launches + 1) & 1 : 0];
         a.Ix = Ix;
         a.Iy = Iy;
         a.It = It;
         a.ms_max = nullptr;
-        a.partials = (check || it == iters - 1) ? partials : nullptr;
+        a.partials = (check || it + step == iters) ? partials : nullptr;
         a.done = params->tol > 0.0 ? &misc->done : nullptr;
         a.tmp = tmp;
         if (pdr) {
@@ -1741,17 +1779,20 @@ of_status iterate_common(of_fields f, const float *Ix, const float *Iy, const fl
             else launch_pdr_fused(a, PREC_F32, PREC_F32, s);
         } else if (cp) {
             launch_cp(a, PREC_F32, PREC_F32, s);
+        } else if (plain) {
+            launch_admm_plain(a, s);
         } else {
-            if (plain) launch_admm_plain(a, s);
-            else launch_admm_fused(a, PREC_F32, PREC_F32, s);
+            TileArgs t{};
+            t.a = a;
+            tile_set_plan(t, tp, step);
+            t.vec = vec;
+            launch_admm_tile(t, PREC_F32, PREC_F32, s);
         }
-        const int nb = pdr ? pdr_plain_blocks(g) : cp ? cp_blocks(g) : (plain ? admm_plain_blocks(g) : admm_fused_blocks(g));
-        if (check) {
-            launch_reduce_check(partials, nb, &misc->res_check, rows, params->tol, &misc->done, &misc->iters, 10, s);
-        }
+        if (check)
+            launch_reduce_check(partials, nb_used, &misc->res_check, rows, params->tol, &misc->done, &misc->iters, 10, s);
     }
-    if (pingpong && (iters & 1)) {
-        // after an odd number of iterations the result sits in the scratch buffer; an early stop
+    if (pingpong && (launches & 1)) {
+        // after an odd number of launches the result sits in the scratch buffer; an early stop
         // (always after an even count) leaves it in the caller's planes.  Copy back unless stopped.
         Fields from = bufs[1], to = bufs[0];
         for (int q = 0; q < NFIELDS; ++q)
@@ -1759,8 +1800,7 @@ of_status iterate_common(of_fields f, const float *Ix, const float *Iy, const fl
         launch_parity_fix(from, to, g, PREC_F32, PREC_F32, params->tol > 0.0 ? &misc->done : nullptr, 0, s);
     }
     if (res2) {
-        const int nb = pdr ? pdr_plain_blocks(g) : cp ? cp_blocks(g) : (plain ? admm_plain_blocks(g) : admm_fused_blocks(g));
-        if (iters > 0) launch_sum(partials, nb, &misc->res_final, s);
+        if (iters > 0) launch_sum(partials, nb_used, &misc->res_final, s);
         Misc m;
         OF_CUDA(cudaMemcpyAsync(&m, misc, sizeof(Misc), cudaMemcpyDeviceToHost, s));
         OF_CUDA(cudaStreamSynchronize(s));

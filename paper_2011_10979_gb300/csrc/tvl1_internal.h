@@ -1,6 +1,7 @@
 // tvl1_internal.h -- internal declarations shared by the kernel translation units and the host
 // runtime of the GB300 TV-L1 library.  Not part of the public C ABI (include/tvl1flow.h).
 #pragma once
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -48,6 +49,7 @@ struct __align__(16) PairIter {
     const float *ms_max;
     const int *done;
     float *tmp;  // the pair's FP32 scratch planes (pDR engine)
+    const void *maps;  // tensor maps of the staged tile kernel: per buffer, flow, dual and data planes
 };
 
 // Device scalars of one pair in a batch, for the batched reductions: the partial sums of the
@@ -90,6 +92,31 @@ struct IterArgs {
     // pDR, gs_sweeps = 1: the one-launch tile kernel, reading `in` and writing `out` (batched:
     // buf[parity] -> buf[parity ^ 1]); 0: the per-kernel engine, in place in `in`
     int pdr_tile = 0;
+};
+
+// The several-iterations ADMM tile kernel (k_admm_tile.cuh): blocks of TILE_WARPS warps hold frames
+// of 64 x TILE_WARPS R pixels, at most one block per SM and TILE_MAX_ITERS iterations per launch.
+constexpr int TILE_WARPS = 12, TILE_SMS = 152, TILE_MAX_ITERS = 8;
+// Iterations per launch where the number is fixed (ALG1's tile kernel too).
+constexpr int TILE_ITERS = 3;
+
+// A level's tiling: ni iterations of halo around tiles of ow x oh pixels whose output starts offx
+// columns and offy rows into their frames; gx x gy tiles.
+struct TilePlan {
+    int R = 0, ni = 0, offx = 0, offy = 0, ow = 0, oh = 0, gx = 0, gy = 0;
+    bool staged = false;
+};
+
+// One launch: a.g / in / out / data of the single pair, or a.tiles / a.pairs / a.parity of a batch; ni
+// iterations (at most the plan's).
+struct TileArgs {
+    IterArgs a;
+    int R, ni, offx, offy, ow, oh;
+    int gx, ntiles;       // single pair: tiles per row; tiles in all
+    int staged;
+    int vec;              // every plane's rows start on an 8-byte boundary
+    int *timeout;         // set when a bounded wait ran out
+    CUtensorMap maps[3];  // staged form, single pair: flow, dual and data planes
 };
 
 // Geometry of the fused ADMM engine: each warp owns a strip of admm_fused_strip_w() output
@@ -241,13 +268,19 @@ void launch_parity_fix(const Fields &from, const Fields &to, Geom g, int prec, i
                        int want_done, cudaStream_t s);
 
 // ---------------------------------------------------------------- several iterations per launch (k_admm_tile.cu, k_cp_tile.cu)
-// Single pair: ni (2 or 3) consecutive iterations of the fused ADMM engine (ALG1: of k_cp) in one
-// launch over TT x TT tiles (*_tile_size: 32, or 16 on small levels), reading a.in and writing
+// The tiling of a single pair's level for launches of ni iterations (0: the rule's choice).
+TilePlan admm_tile_plan(Geom g, int ni);
+int admm_tile_blocks(const TilePlan &p);  // partial-sum slots of a launch
+void tile_set_plan(TileArgs &t, const TilePlan &p, int ni);
+// The staged form's tensor maps of a state buffer (its planes equally spaced) and the data planes;
+// false when the driver cannot encode them.
+bool tile_encode_maps(CUtensorMap maps[3], const Fields &f, const void *Ix, const void *Iy, Geom g, int prec,
+                      int prec_flow, bool has_w, int R);
+void launch_admm_tile(const TileArgs &a, int prec, int prec_flow, cudaStream_t s);
+// Single pair: ni (2 or 3) consecutive iterations of k_cp in one
+// launch over TT x TT tiles (cp_tile_size: 32, or 16 on small levels), reading a.in and writing
 // a.out, bitwise ni launches of the one-iteration kernel; partials (of the last iteration) in
-// *_tile_blocks(a.g) slots.
-int admm_tile2_size(Geom g);
-int admm_tile2_blocks(Geom g);
-void launch_admm_tile2(const IterArgs &a, int ni, int prec, int prec_flow, cudaStream_t s);
+// cp_tile_blocks(a.g) slots.
 int cp_tile_size(Geom g);
 int cp_tile_blocks(Geom g);
 void launch_cp_tile(const IterArgs &a, int ni, int prec, int prec_flow, cudaStream_t s);
