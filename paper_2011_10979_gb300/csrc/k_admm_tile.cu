@@ -60,6 +60,29 @@ TilePlan admm_tile_plan(Geom g, int ni) {
     return best;
 }
 
+// Batches run the staged form with four rows per warp; the iterations per launch that cost the least
+// over all pairs' tiles.
+TilePlan admm_tile_plan_batch(const Geom *g, int n, int ni) {
+    TilePlan best;
+    float us = 0.f;
+    for (int k = ni ? ni : 1; k <= (ni ? ni : TILE_MAX_ITERS); ++k) {
+        TilePlan p;
+        int tiles = 0;
+        for (int q = 0; q < n; ++q) {
+            p = plan_of(g[q], 4, k, true);
+            tiles += p.gx * p.gy;
+        }
+        p.gx = tiles;
+        p.gy = 1;
+        const float t = plan_us(p) / k;
+        if (us == 0.f || t < us) {
+            us = t;
+            best = p;
+        }
+    }
+    return best;
+}
+
 int admm_tile_blocks(const TilePlan &p) { return p.gx * p.gy; }
 
 void tile_set_plan(TileArgs &t, const TilePlan &p, int ni) {

@@ -101,6 +101,19 @@ Coefs coefs_of(const of_params *p) {
     return k;
 }
 
+int tile_iters_of(const of_params *p, int iters) {
+    return p->engine == OF_ENGINE_STREAM || p->tol > 0.0 || iters <= 10 ? TILE_ITERS : 0;
+}
+
+int tile_step(const of_params *p, int ni, int it, int iters) {
+    int step = std::min(ni, iters - it);
+    if (p->tol > 0.0) {
+        step = std::min(step, 10 - it % 10);
+        if (step > 1 && it + step == iters) --step;
+    }
+    return step;
+}
+
 Fields fields_at(char *base, size_t plane) {
     Fields f;
     for (int k = 0; k < NFIELDS; ++k) f.f[k] = base + (size_t)k * plane;
@@ -258,6 +271,10 @@ struct Batch {
     int res_nc[MAX_LEVELS] = {};  // CTAs per cluster of the level's resident launch
     // the other pairs, for the one-slice-per-pair batched kernels (ALG1)
     size_t streamlist_off[MAX_LEVELS] = {};
+    // the ADMM tile kernel's tiling of the streamed pairs per level (R = 0: the level runs on the
+    // row-streaming kernel), its work-list, and the pairs' tensor maps per precision
+    TilePlan tp[MAX_LEVELS];
+    size_t ttiles_off[MAX_LEVELS] = {}, maps_off[MAX_LEVELS][2] = {};
     size_t partials = 0, table_off = 0, table_bytes = 0, total = 0;
     // persistent ADMM engine per level (any n): the segment plan and the offsets (in the table
     // region) of its segments, warp lists, per-pair scalars, counters and partial sums
@@ -286,19 +303,12 @@ bool pdr_tile_of(const of_params *p) {
 // 2.7 / 4.3 at 80x60, 4.3 / 4.3 at 120x90, 6.0 / 4.4 at 160x120).
 constexpr long PDR_TILE_RESIDENT_MAX_PX = 12000;
 
-// Whether a single pair's streamed ADMM level runs several iterations per launch (k_admm_tile.cuh):
-// the built-in strip rule (a pinned or autotuned height asks for the row-streaming kernel), at any
-// size.
-bool admm_tile_of(const of_params *p, bool batched) {
-    return !batched && (p->method == OF_PADMM_I || p->method == OF_PADMM_II) && p->rows_per_warp == 0 &&
+// Whether streamed ADMM levels run several iterations per launch (k_admm_tile.cuh): the built-in
+// strip rule (a pinned or autotuned height asks for the row-streaming kernel), at any size, single
+// pairs and batches.
+bool admm_tile_of(const of_params *p) {
+    return (p->method == OF_PADMM_I || p->method == OF_PADMM_II) && p->rows_per_warp == 0 &&
            (p->engine == OF_ENGINE_FUSED || p->engine == OF_ENGINE_STREAM);
-}
-
-// Iterations per launch of the tile kernel for a warp of `iters` iterations: the level's choice
-// (admm_tile_plan; 0), or TILE_ITERS on the streaming engine, with the stopping test (every ten
-// iterations run as launches of 3, 3, 3 and 1) and for warps of up to ten iterations.
-int tile_iters_of(const of_params *p, int iters) {
-    return p->engine == OF_ENGINE_STREAM || p->tol > 0.0 || iters <= 10 ? TILE_ITERS : 0;
 }
 
 // Whether a single pair's streamed ALG1 level runs several iterations per launch (k_cp_tile.cu):
@@ -324,7 +334,7 @@ bool use_resident(const of_params *p, Geom g, bool batched = false) {
     if (p->engine == OF_ENGINE_RESIDENT) return true;
     if (p->engine != OF_ENGINE_FUSED && p->engine != OF_ENGINE_PERSISTENT) return false;
     if (pdr_tile_of(p)) return (long)g.H * g.W <= PDR_TILE_RESIDENT_MAX_PX;
-    if (admm_tile_of(p, batched)) return (long)g.H * g.W <= TILE_RESIDENT_MAX_PX;
+    if (admm_tile_of(p) && !batched) return (long)g.H * g.W <= TILE_RESIDENT_MAX_PX;
     if (cp_tile_of(p, batched)) return (long)g.H * g.W <= CP_TILE_RESIDENT_MAX_PX;
     return admm_resident_preferred(g, p->method);
 }
@@ -514,7 +524,19 @@ Batch make_batch(int n, const int *H, const int *W, const of_params *p) {
             t += align_up(sizeof(int) * n, 256);
             B.streamlist_off[l] = t;
             t += align_up(sizeof(int) * n, 256);
-            const size_t np = std::max({(size_t)nt, (size_t)n * pdr_plain_blocks(gm, PARTIAL_ROWS_MIN),
+            if (admm_tile_of(p) && B.nres[l] < n && l >= B.out_level) {
+                std::vector<Geom> gs;
+                for (int k = 0; k < n; ++k)
+                    if (!B.res[l][k]) gs.push_back(geom_of(B.pl[k], l));
+                B.tp[l] = admm_tile_plan_batch(gs.data(), (int)gs.size(), tile_iters_of(p, p->iters));
+                B.ttiles_off[l] = t;
+                t += align_up(sizeof(TileRef) * B.tp[l].gx, 256);
+                for (int v = 0; v < (l == 0 && B.pl[0].use32_last ? 2 : 1); ++v) {
+                    B.maps_off[l][v] = t;
+                    t += align_up(6 * sizeof(CUtensorMap) * n, 256);
+                }
+            }
+            const size_t np = std::max({(size_t)nt, (size_t)B.tp[l].gx, (size_t)n * pdr_plain_blocks(gm, PARTIAL_ROWS_MIN),
                                         (size_t)n * cp_blocks(gm, PARTIAL_ROWS_MIN)});
             maxpart = std::max(maxpart, np);
         }
@@ -588,6 +610,8 @@ of_status upload_tables(of_ctx *ctx, const Batch &B, const of_params *p) {
     const bool pdr = p->method == OF_PDR, cp = p->method == OF_CP;
     const bool xb = pdr || cp;  // one grid slice per pair (pDR, ALG1) instead of a tile work-list
     // the descriptors of pair k at level l, for its storage-precision and its FP32 buffers
+    const bool has_w = p->beta != 0.f;
+    bool maps_ok = true;
     auto pair_iter = [&](PairIter *pi0, PairIter *pi1, int k, int l) {
         const Plan &pl = B.pl[k];
         char *A = ctx->arena + B.base[k];
@@ -611,6 +635,16 @@ of_status upload_tables(of_ctx *ctx, const Batch &B, const of_params *p) {
             P.ms_max = &misc->ms_max;
             P.done = p->tol > 0.0 ? &misc->done : nullptr;
             P.tmp = (float *)(A + pl.tmp);
+            if (B.maps_off[l][v] > 0 && !B.res[l][k]) {
+                const size_t o = B.maps_off[l][v] + 6 * sizeof(CUtensorMap) * k;
+                P.maps = ctx->arena + B.table_off + o;
+                for (int b = 0; b < 2; ++b) {
+                    CUtensorMap m[3];  // aligned as the encoder asks for
+                    maps_ok = maps_ok && tile_encode_maps(m, P.buf[b], P.Ix, P.Iy, P.g, v ? PREC_F32 : pl.prec,
+                                                          v ? PREC_F32 : pl.pflow, has_w, B.tp[l].R);
+                    memcpy(img.data() + o + b * sizeof(m), m, sizeof(m));
+                }
+            }
         }
     };
     auto scalars = [&](PairScalars &ps, int k, int l) {
@@ -630,7 +664,9 @@ of_status upload_tables(of_ctx *ctx, const Batch &B, const of_params *p) {
         PairScalars *ps = (PairScalars *)(img.data() + B.scal_off[l]);
         int *rl = (int *)(img.data() + B.reslist_off[l]);
         int *sl = (int *)(img.data() + B.streamlist_off[l]);
-        int t = 0, r = 0, ns = 0;
+        int t = 0, r = 0, ns = 0, tt = 0;
+        const bool tile = B.tp[l].R > 0;
+        TileRef *ttr = (TileRef *)(img.data() + B.ttiles_off[l]);
         const int G = cp                ? cp_blocks(B.gmax[l], B.tile_h[l])
                       : pdr_tile_of(p) ? pdr_tile_blocks(B.gmax[l])
                                        : pdr_plain_blocks(B.gmax[l], B.tile_h[l]);
@@ -644,9 +680,13 @@ of_status upload_tables(of_ctx *ctx, const Batch &B, const of_params *p) {
             if (!B.res[l][k])
                 for (int ty = 0; ty < (g.H + rows - 1) / rows; ++ty)
                     for (int tx = 0; tx < (g.W + SWD - 1) / SWD; ++tx) tr[t++] = TileRef{k, tx, ty, 0};
+            const int tt0 = tt;
+            if (tile && !B.res[l][k])
+                for (int ty = 0; ty < tile_rows(B.tp[l], g); ++ty)
+                    for (int tx = 0; tx < tile_cols(B.tp[l], g); ++tx) ttr[tt++] = TileRef{k, tx, ty, 0};
             scalars(ps[k], k, l);
-            ps[k].part_begin = xb ? k * G : t0;
-            ps[k].part_end = xb ? (k + 1) * G : t;
+            ps[k].part_begin = xb ? k * G : tile ? tt0 : t0;
+            ps[k].part_end = xb ? (k + 1) * G : tile ? tt : t;
             ps[k].resident = B.res[l][k];
         }
     }
@@ -666,6 +706,7 @@ of_status upload_tables(of_ctx *ctx, const Batch &B, const of_params *p) {
             ps[k].resident = B.pbegin[l][k] == B.pend[l][k];  // not on this engine: skipped by the reductions
         }
     }
+    if (!maps_ok) return fail(OF_ECUDA, "cuTensorMapEncodeTiled failed");
     // work already queued on any stream may still read another layout's tables in this region
     OF_CUDA(cudaDeviceSynchronize());
     OF_CUDA(cudaMemcpy(ctx->arena + B.table_off, img.data(), img.size(), cudaMemcpyHostToDevice));
@@ -842,8 +883,28 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                 launch_count_iters(&c.misc->iters, nullptr, kw, s);
             }
             const int start2 = (start + kw) & 1;  // where the level's engine picks the state up
-            // level-resident engine: the single pair, or the batch's resident pairs, in one launch
+            // the streamed pairs' launches: how many iterations each takes.  ADMM and ALG1 by the built-in
+            // strip rule or block height run several per launch (k_admm_tile.cuh, k_cp_tile.cu).
             const bool res1 = !batched && use_resident(p, geom_of(*pc[0].pl, l));
+            const bool tile = !B.pers[l] && (batched ? B.tp[l].R > 0 : !res1 && admm_tile_of(p));
+            const bool tile2 = tile || (!B.pers[l] && !res1 && cp_tile_of(p, batched));
+            TilePlan tp = B.tp[l];
+            CUtensorMap maps[2][3];
+            if (tile && !batched) {
+                const PairCtx &c = pc[0];
+                const Geom g = geom_of(*c.pl, l);
+                tp = admm_tile_plan(g, tile_iters_of(p, rest));
+                for (int b = 0; b < 2 && tp.staged; ++b)
+                    tp.staged = tile_encode_maps(maps[b], bufs_of(c)[b], data_of(c)[0], data_of(c)[1], g, prec, pflow, has_w, tp.R);
+            }
+            std::vector<int> steps;
+            for (int it = 0, step = 1; it < rest; it += step) {
+                step = 1;
+                if (tile2) step = tile_step(p, tile ? tp.ni : TILE_ITERS, it, rest);
+                steps.push_back(step);
+            }
+            const int launches = (int)steps.size();
+            // level-resident engine: the single pair, or the batch's resident pairs, in one launch
             const bool resb = batched && B.nres[l] > 0;
             if (rest > 0 && (res1 || resb)) {
                 ResArgs r{};
@@ -853,7 +914,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                 r.final_res = last_warp;
                 r.tol = p->tol;
                 r.parity_in = start2;
-                r.parity_out = pingpong ? (start2 + rest) & 1 : start2;  // pDR works in place
+                r.parity_out = pingpong ? (start2 + launches) & 1 : start2;  // pDR works in place
                 if (res1) {
                     const PairCtx &c = pc[0];
                     const Geom g = geom_of(*c.pl, l);
@@ -908,33 +969,9 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
             // pairs left for one launch per iteration: the tile work-list (ADMM), all pairs (pDR),
             // the non-resident pairs (ALG1)
             const bool streamed = !persl && (batched ? ((cp || pdr) ? B.nres[l] < n : B.ntiles[l] > 0) : !res1);
-            // single pair, ADMM or ALG1, the built-in strip rule or block height: several iterations
-            // per launch (k_admm_tile.cuh, k_cp_tile.cu).  With the
-            // stopping test every ten iterations run as launches of 3, 3, 3 and 1: the tested state
-            // is a single-iteration launch's (its residual partials), an even number of launches
-            // leaves it in bufs[start2] as on the one-launch-per-iteration path, and the warp's last
-            // launch is a single iteration too, so the final residual sums the same partials
-            // whether or not the test stopped the warp.
-            const bool tile = streamed && admm_tile_of(p, batched), tile2 = tile || (streamed && cp_tile_of(p, batched));
-            TilePlan tp;
-            CUtensorMap maps[2][3];
-            if (tile) {
-                const PairCtx &c = pc[0];
-                const Geom g = geom_of(*c.pl, l);
-                tp = admm_tile_plan(g, tile_iters_of(p, rest));
-                for (int b = 0; b < 2 && tp.staged; ++b)
-                    tp.staged = tile_encode_maps(maps[b], bufs_of(c)[b], data_of(c)[0], data_of(c)[1], g, prec, pflow, has_w, tp.R);
-            }
-            int par = start2, last_nb = 0;  // the several-iterations path's buffer parity and last block count
-            for (int it = 0, step = 1; streamed && it < rest; it += step) {
-                step = 1;
-                if (tile2) {
-                    step = std::min(tile ? tp.ni : TILE_ITERS, rest - it);
-                    if (p->tol > 0.0) {
-                        step = std::min(step, 10 - it % 10);
-                        if (step > 1 && it + step == rest) --step;
-                    }
-                }
+            int par = start2, last_nb = 0;  // the buffer parity and the last launch's block count
+            for (int it = 0, q = 0, step = 1; streamed && it < rest; it += step) {
+                step = steps[q++];
                 const bool check = p->tol > 0.0 && (it + step) % 10 == 0;
                 const bool final_it = last_warp && it + step == rest;
                 IterArgs a{};
@@ -945,9 +982,8 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                     const Fields *bf = bufs_of(c);
                     const void *const *dat = data_of(c);
                     a.g = g;
-                    a.in = bf[tile2 ? par : pingpong ? (start2 + it) & 1 : start2];
-                    a.out = bf[tile2 ? par ^ 1 : pingpong ? (start2 + it + 1) & 1 : start2];
-                    par ^= 1;
+                    a.in = bf[pingpong ? par : start2];
+                    a.out = bf[pingpong ? par ^ 1 : start2];
                     a.Ix = dat[0];
                     a.Iy = dat[1];
                     a.It = dat[2];
@@ -974,7 +1010,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                         tile_set_plan(t, tp, step);
                         t.vec = 1;
                         t.timeout = &c.misc->timeout;
-                        if (tp.staged) memcpy(t.maps, maps[par ^ 1], sizeof(t.maps));  // par is the next launch's by now
+                        if (tp.staged) memcpy(t.maps, maps[par], sizeof(t.maps));
                         launch_admm_tile(t, prec, pflow, s);
                         last_nb = admm_tile_blocks(tp);
                     } else {
@@ -995,7 +1031,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                         a.g = B.gmax[l];
                         a.ntiles = n - B.nres[l];
                         a.plist = (const int *)(ctx->arena + B.table_off + B.streamlist_off[l]);
-                        a.parity = pdr_tile ? (start2 + it) & 1 : start2;
+                        a.parity = pdr_tile ? par : start2;
                         a.tile_h = B.tile_h[l];
                         a.pdr_tile = pdr_tile;
                         launch_pdr_fused(a, prec, pflow, s);
@@ -1003,20 +1039,30 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                         a.g = B.gmax[l];
                         a.ntiles = n - B.nres[l];
                         a.plist = (const int *)(ctx->arena + B.table_off + B.streamlist_off[l]);
-                        a.parity = (start2 + it) & 1;
+                        a.parity = par;
                         a.tile_h = B.tile_h[l];
                         launch_cp(a, prec, pflow, s);
+                    } else if (tile) {
+                        TileArgs t{};
+                        a.tiles = (const TileRef *)(ctx->arena + B.table_off + B.ttiles_off[l]);
+                        a.parity = par;
+                        t.a = a;
+                        tile_set_plan(t, tp, step);
+                        t.vec = 1;
+                        t.timeout = &pc[0].misc->timeout;
+                        launch_admm_tile(t, prec, pflow, s);
                     } else {
                         a.tiles = (const TileRef *)(ctx->arena + B.table_off + B.tiles_off[l]);
                         a.ntiles = B.ntiles[l];
                         a.tile_h = B.tile_h[l];
-                        a.parity = (start2 + it) & 1;
+                        a.parity = par;
                         launch_admm_fused(a, prec, pflow, s);
                     }
                     if (check)
                         launch_reduce_check_batched(bpart, (const PairScalars *)(ctx->arena + B.table_off + B.scal_off[l]),
                                                     n, p->tol, 10, 0, s);
                 }
+                par ^= 1;
             }
             const PairScalars *ps = batched ? (const PairScalars *)(ctx->arena + B.table_off + B.scal_off[l]) : nullptr;
             if (batched) {
@@ -1027,8 +1073,8 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                 else launch_count_iters(&m->iters, nullptr, rest, s);
             }
             if (pingpong) {
-                const int fin = tile2 ? par : (start + p->iters) & 1;
-                if (p->tol > 0.0 && (tile2 ? par != start2 : (rest & 1)))
+                const int fin = (start2 + launches) & 1;
+                if (p->tol > 0.0 && fin != start2)
                     for (int q = 0; q < n; ++q)
                         if (!(res1 || (batched && B.res[l][q])))  // the resident engine writes buf[fin] itself
                             launch_parity_fix(bufs_of(pc[q])[start2], bufs_of(pc[q])[fin], geom_of(*pc[q].pl, l),
@@ -1753,13 +1799,9 @@ of_status iterate_common(of_fields f, const float *Ix, const float *Iy, const fl
     for (int it = 0, step = 1; it < iters; it += step, ++launches) {
         step = 1;
         if (tile) {
-            step = std::min(tp.ni, iters - it);
+            step = tile_step(params, tp.ni, it, iters);
             // an even number of launches leaves the state in the caller's planes
             if (it + step == iters && step > 1 && launches % 2 == 0) --step;
-            if (params->tol > 0.0) {
-                step = std::min(step, 10 - it % 10);
-                if (step > 1 && it % 10 + step == 10) --step;
-            }
         }
         const bool check = params->tol > 0.0 && (it + step) % 10 == 0;
         IterArgs a{};

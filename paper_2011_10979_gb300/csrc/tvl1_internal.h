@@ -270,7 +270,12 @@ void launch_parity_fix(const Fields &from, const Fields &to, Geom g, int prec, i
 // ---------------------------------------------------------------- several iterations per launch (k_admm_tile.cu, k_cp_tile.cu)
 // The tiling of a single pair's level for launches of ni iterations (0: the rule's choice).
 TilePlan admm_tile_plan(Geom g, int ni);
+// The tiling of n pairs' levels in one batched launch (gx: tiles in all).
+TilePlan admm_tile_plan_batch(const Geom *g, int n, int ni);
 int admm_tile_blocks(const TilePlan &p);  // partial-sum slots of a launch
+// Tiles of one pair's level in a batched launch.
+inline int tile_cols(const TilePlan &p, Geom g) { return (g.W + p.ow - 1) / p.ow; }
+inline int tile_rows(const TilePlan &p, Geom g) { return (g.H + p.oh - 1) / p.oh; }
 void tile_set_plan(TileArgs &t, const TilePlan &p, int ni);
 // The staged form's tensor maps of a state buffer (its planes equally spaced) and the data planes;
 // false when the driver cannot encode them.

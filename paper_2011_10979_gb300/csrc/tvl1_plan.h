@@ -56,6 +56,18 @@ Plan make_plan(int H, int W, const of_params *p);
 // Kernel coefficients of the parameters.
 Coefs coefs_of(const of_params *p);
 
+// Iterations per launch of the ADMM tile kernel for a warp of `iters` iterations: the level's choice
+// (0; admm_tile_plan), or TILE_ITERS on the streaming engine, with the stopping test, and for warps of
+// up to ten iterations (such a warp takes four launches on every engine).
+int tile_iters_of(const of_params *p, int iters);
+
+// Iterations of the launch that starts after `it` of a warp's `iters` iterations, at most ni.  With the
+// stopping test every ten iterations run as launches of 3, 3, 3 and 1: an even number of launches
+// leaves the tested state in the buffer the warp started from, as on the one-launch-per-iteration
+// path, and the warp's last launch is a single iteration, so that the final residual sums the same
+// partials whether or not the test stopped the warp.
+int tile_step(const of_params *p, int ni, int it, int iters);
+
 // The 13 planes of a state buffer at `base`, `plane` bytes apart.
 Fields fields_at(char *base, size_t plane);
 

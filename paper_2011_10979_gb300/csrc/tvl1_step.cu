@@ -139,10 +139,21 @@ cudaError_t run_group(std::vector<StepPair *> &G, const of_params *p, StepTables
         const Geom g = geom_of(q->pl, q->l);
         ntiles += ((g.W + SWD - 1) / SWD) * ((g.H + rows - 1) / rows);
     }
+    // the ADMM tile kernel, several iterations per launch, by the built-in strip rule (as the whole
+    // solve; the launches of 3, 3, 3 and 1 per ten iterations with the stopping test)
+    const bool tile = !(pdr || cp) && p->rows_per_warp == 0 && (p->engine == OF_ENGINE_FUSED || p->engine == OF_ENGINE_STREAM);
+    TilePlan tp;
+    if (tile) {
+        std::vector<Geom> gs;
+        for (StepPair *q : G) gs.push_back(geom_of(q->pl, q->l));
+        tp = admm_tile_plan_batch(gs.data(), n, tile_iters_of(p, p->iters));
+        ntiles = tp.gx;
+    }
     const int Gb = cp ? cp_blocks(gmax) : pdr_plain_blocks(gmax);
     const size_t nparts = (pdr || cp) ? (size_t)n * Gb : (size_t)std::max(ntiles, 1);
-    // table layout: PairIter[n] | PairScalars[n] | plist[n] | TileRef[ntiles] | partials
-    const size_t o_pi = 0, o_ps = align_up(sizeof(PairIter) * n, 256);
+    // table layout: PairIter[n] | tensor maps | PairScalars[n] | plist[n] | TileRef[ntiles] | partials
+    const size_t o_pi = 0, o_tm = align_up(sizeof(PairIter) * n, 256);
+    const size_t o_ps = o_tm + (tile ? align_up(6 * sizeof(CUtensorMap) * n, 256) : 0);
     const size_t o_pl = o_ps + align_up(sizeof(PairScalars) * n, 256);
     const size_t o_tr = o_pl + align_up(sizeof(int) * n, 256);
     const size_t o_pa = o_tr + align_up(sizeof(TileRef) * (size_t)std::max(ntiles, 1), 256);
@@ -185,7 +196,16 @@ cudaError_t run_group(std::vector<StepPair *> &G, const of_params *p, StepTables
         P.tmp = (float *)(q.A + q.pl.tmp);
         pl[k] = k;
         const int t0 = t;
-        if (!(pdr || cp))
+        if (tile) {
+            P.maps = T.dev + o_tm + 6 * sizeof(CUtensorMap) * k;
+            for (int b = 0; b < 2; ++b) {
+                CUtensorMap m[3];  // aligned as the encoder asks for
+                if (!tile_encode_maps(m, P.buf[b], P.Ix, P.Iy, g, prec, pflow, has_w, tp.R)) return cudaErrorUnknown;
+                memcpy(h + o_tm + 6 * sizeof(CUtensorMap) * k + b * sizeof(m), m, sizeof(m));
+            }
+            for (int y = 0; y < tile_rows(tp, g); ++y)
+                for (int x = 0; x < tile_cols(tp, g); ++x) tr[t++] = TileRef{k, x, y, 0};
+        } else if (!(pdr || cp))
             for (int y = 0; y < (g.H + rows - 1) / rows; ++y)
                 for (int x = 0; x < (g.W + SWD - 1) / SWD; ++x) tr[t++] = TileRef{k, x, y, 0};
         ps[k].res_check = &m->res_check;
@@ -205,29 +225,37 @@ cudaError_t run_group(std::vector<StepPair *> &G, const of_params *p, StepTables
     const TileRef *dtr = (const TileRef *)(T.dev + o_tr);
     double *part = (double *)(T.dev + o_pa);
     const Coefs k = coefs_of(p);
-    for (int it = 0; it < p->iters; ++it) {
-        const bool check = p->tol > 0.0 && (it + 1) % 10 == 0;
+    int launches = 0;
+    for (int it = 0, step = 1; it < p->iters; it += step, ++launches) {
+        step = tile ? tile_step(p, tp.ni, it, p->iters) : 1;
+        const bool check = p->tol > 0.0 && (it + step) % 10 == 0;
         IterArgs a{};
         a.k = k;
         a.pairs = dpi;
-        a.partials = (check || it == p->iters - 1) ? part : nullptr;
+        a.partials = (check || it + step == p->iters) ? part : nullptr;
+        a.parity = pdr ? 0 : launches & 1;
         if (pdr) {
             a.g = gmax;
             a.ntiles = n;
             a.plist = dpl;
-            a.parity = 0;
             launch_pdr_fused(a, prec, pflow, s);
         } else if (cp) {
             a.g = gmax;
             a.ntiles = n;
             a.plist = dpl;
-            a.parity = it & 1;
             launch_cp(a, prec, pflow, s);
+        } else if (tile) {
+            TileArgs ta{};
+            a.tiles = dtr;
+            ta.a = a;
+            tile_set_plan(ta, tp, step);
+            ta.vec = 1;
+            ta.timeout = &misc_of(*G[0])->timeout;
+            launch_admm_tile(ta, prec, pflow, s);
         } else {
             a.tiles = dtr;
             a.ntiles = ntiles;
             a.tile_h = ty;
-            a.parity = it & 1;
             launch_admm_fused(a, prec, pflow, s);
         }
         if (check) launch_reduce_check_batched(part, dps, n, p->tol, 10, 0, s);
@@ -236,10 +264,10 @@ cudaError_t run_group(std::vector<StepPair *> &G, const of_params *p, StepTables
         launch_count_iters_batched(dps, n, p->tol > 0.0 ? p->iters % 10 : p->iters, p->tol > 0.0, s);
         launch_reduce_check_batched(part, dps, n, 0.0, 0, 1, s);  // residual of the stage's last iteration
     }
-    // the state after the stage: buffer cur ^ (iters & 1) for the ping-pong engines, unless the pair
+    // the state after the stage: buffer cur ^ (launches & 1) for the ping-pong engines, unless the pair
     // stopped (always after an even count), which leaves it in buffer cur: copy it over then
     for (StepPair *q : G) {
-        if (!pingpong || !(p->iters & 1)) continue;
+        if (!pingpong || !(launches & 1)) continue;
         const Bufs bf = bufs_of(*q);
         if (p->tol > 0.0)
             launch_parity_fix(bf.st[q->cur], bf.st[q->cur ^ 1], geom_of(q->pl, q->l), cp ? pflow : prec, pflow,
