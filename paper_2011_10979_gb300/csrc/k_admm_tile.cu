@@ -14,8 +14,8 @@ void tile_launch_bf16(const TileArgs &a, bool flow32, cudaStream_t s);
 
 namespace {
 
-// The tiling of a level into frames of 64 x TILE_WARPS R with ni iterations of halo.  Staged frames
-// start at multiples of 4 columns (16-byte aligned copies), the others at even ones.
+// The tiling of a level into frames of 64 x TILE_WARPS R (staged: 64 x 48) with ni iterations of halo.
+// Staged frames start at multiples of 4 columns (16-byte aligned copies), the others at even ones.
 TilePlan plan_of(Geom g, int R, int ni, bool staged) {
     TilePlan p;
     p.R = R;
@@ -25,32 +25,31 @@ TilePlan plan_of(Geom g, int R, int ni, bool staged) {
     p.offx = (ni + 1 + al - 1) / al * al;
     p.offy = ni + 1;
     p.ow = (64 - p.offx - ni) / al * al;
-    p.oh = TILE_WARPS * R - 2 * ni - 1;
+    p.oh = (staged ? TILE_STAGED_HEIGHT : TILE_WARPS * R) - 2 * ni - 1;
     p.gx = (g.W + p.ow - 1) / p.ow;
     p.gy = (g.H + p.oh - 1) / p.oh;
     return p;
 }
 
-// Microseconds of one launch of the plan.
+// Microseconds of one launch of the plan, fitted to launches inside a CUDA graph (per round of tiles
+// over the SMs: a part per tile and one per iteration; FP32, beta > 0).  Measured against it: 320x240,
+// R = 2, five iterations 8.4 us; 640x480, R = 4, three 10.6 and R = 3, six 20.7; 1024x436 staged, six
+// 27.1 and R = 3, three 14.5; 3840x2160 staged, four 239.
 float plan_us(const TilePlan &p) {
-    static const float per_iter[5] = {0.f, 0.f, 0.8f, 1.05f, 1.2f}, per_tile[5] = {0.f, 0.f, 2.5f, 3.5f, 4.4f};
+    static const float per_iter[5] = {0.f, 0.f, 0.95f, 1.2f, 1.7f}, per_tile[5] = {0.f, 0.f, 3.2f, 3.7f, 4.9f};
     const int n = p.gx * p.gy, rounds = (n + TILE_SMS - 1) / TILE_SMS;
-    return 2.5f + rounds * (per_tile[p.R] + p.ni * per_iter[p.R]);
+    return p.staged ? 3.4f + rounds * (3.8f + 1.25f * p.ni) : 0.4f + rounds * (per_tile[p.R] + p.ni * per_iter[p.R]);
 }
 
 }  // namespace
 
-TilePlan admm_tile_plan(Geom g, int ni) {
+TilePlan admm_tile_plan(Geom g, int ni, bool direct) {
     TilePlan best;
     float us = 0.f;
-    for (int R = 2; R <= 4; ++R)
-        for (int k = ni ? ni : 1; k <= (ni ? ni : TILE_MAX_ITERS); ++k) {
-            TilePlan p = plan_of(g, R, k, false);
+    for (int k = ni ? ni : 1; k <= (ni ? ni : TILE_MAX_ITERS); ++k)
+        for (int R = 2; R <= (direct ? 4 : 5); ++R) {  // 5: staged
+            const TilePlan p = plan_of(g, R, k, R == 5);
             if (p.oh < 1) continue;
-            if (p.gx * p.gy > TILE_SMS) {
-                if (R < 4) continue;
-                p = plan_of(g, R, k, true);
-            }
             const float t = plan_us(p) / k;
             if (us == 0.f || t < us) {
                 us = t;
@@ -60,8 +59,7 @@ TilePlan admm_tile_plan(Geom g, int ni) {
     return best;
 }
 
-// Batches run the staged form with four rows per warp; the iterations per launch that cost the least
-// over all pairs' tiles.
+// Batches run the staged form; the iterations per launch that cost the least over all pairs' tiles.
 TilePlan admm_tile_plan_batch(const Geom *g, int n, int ni) {
     TilePlan best;
     float us = 0.f;
@@ -69,7 +67,7 @@ TilePlan admm_tile_plan_batch(const Geom *g, int n, int ni) {
         TilePlan p;
         int tiles = 0;
         for (int q = 0; q < n; ++q) {
-            p = plan_of(g[q], 4, k, true);
+            p = plan_of(g[q], 5, k, true);
             tiles += p.gx * p.gy;
         }
         p.gx = tiles;
@@ -98,7 +96,7 @@ void tile_set_plan(TileArgs &t, const TilePlan &p, int ni) {
 }
 
 bool tile_encode_maps(CUtensorMap maps[3], const Fields &f, const void *Ix, const void *Iy, Geom g, int prec,
-                      int prec_flow, bool has_w, int R) {
+                      int prec_flow, bool has_w) {
     static const PFN_cuTensorMapEncodeTiled_v12000 enc = [] {
         void *fn = nullptr;
         cudaDriverEntryPointQueryResult q;
@@ -113,7 +111,7 @@ bool tile_encode_maps(CUtensorMap maps[3], const Fields &f, const void *Ix, cons
         const int eb = (int)prec_bytes(pr);
         const cuuint64_t dim[3] = {(cuuint64_t)g.W, (cuuint64_t)g.H, (cuuint64_t)n};
         const cuuint64_t stride[2] = {(cuuint64_t)g.pitch * eb, (cuuint64_t)plane};
-        const cuuint32_t box[3] = {eb == 4 ? 64u : 72u, (cuuint32_t)(TILE_WARPS * R), (cuuint32_t)n}, es[3] = {1, 1, 1};
+        const cuuint32_t box[3] = {eb == 4 ? 64u : 72u, (cuuint32_t)TILE_STAGED_HEIGHT, (cuuint32_t)n}, es[3] = {1, 1, 1};
         const CUtensorMapDataType dt = pr == PREC_F32   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                        : pr == PREC_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                                         : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;

@@ -109,6 +109,12 @@ template <> __device__ __forceinline__ void st_pair<__nv_bfloat16>(void *base, s
     *reinterpret_cast<__nv_bfloat162 *>(reinterpret_cast<__nv_bfloat16 *>(base) + o) = __floats2bfloat162_rn(a, b);
 }
 
+// Arrival at, and wait on, a named barrier of this block that `n` threads take part in (whole
+// warps): the arriving warps do not wait, and their earlier shared-memory writes are visible to
+// the waiting ones.
+__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_wait(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
 // 1 / max(1, sqrt(n2)) per half: rsqrt.approx of max(n2, 1), which is exactly 1 inside the ball and
 // the value of rsqrtf(n2) outside (n2 > 1 is a normal number, where the flushing and the
 // non-flushing instruction agree).  A NaN n2 gives 1, as the comparison n2 > 1 does.

@@ -69,8 +69,8 @@ Plan make_plan(int H, int W, const of_params *p) {
         const Geom g{pl.H[l], pl.W[l], pl.P[l]};
         mb = std::max({mb, admm_fused_blocks(g, p->rows_per_warp != 0 ? 1 : 0), admm_plain_blocks(g),
                        pdr_plain_blocks(g, PARTIAL_ROWS_MIN), cp_blocks(g, PARTIAL_ROWS_MIN), energy_blocks(g),
-                       adapt_blocks(g), admm_tile_blocks(admm_tile_plan(g, 0)),
-                       admm_tile_blocks(admm_tile_plan(g, TILE_ITERS)), pdr_tile_blocks(g), cp_tile_blocks(g)});
+                       adapt_blocks(g), pdr_tile_blocks(g), cp_tile_blocks(g)});
+        for (int q = 0; q < 4; ++q) mb = std::max(mb, admm_tile_blocks(admm_tile_plan(g, q & 1 ? TILE_ITERS : 0, q & 2)));
     }
     pl.max_blocks = mb;
     pl.partials = take(3 * (size_t)mb * sizeof(double));
@@ -524,7 +524,7 @@ Batch make_batch(int n, const int *H, const int *W, const of_params *p) {
             t += align_up(sizeof(int) * n, 256);
             B.streamlist_off[l] = t;
             t += align_up(sizeof(int) * n, 256);
-            if (admm_tile_of(p) && B.nres[l] < n && l >= B.out_level) {
+            if (admm_tile_of(p) && p->a_tilde_mode == 0 && B.nres[l] < n && l >= B.out_level) {
                 std::vector<Geom> gs;
                 for (int k = 0; k < n; ++k)
                     if (!B.res[l][k]) gs.push_back(geom_of(B.pl[k], l));
@@ -641,7 +641,7 @@ of_status upload_tables(of_ctx *ctx, const Batch &B, const of_params *p) {
                 for (int b = 0; b < 2; ++b) {
                     CUtensorMap m[3];  // aligned as the encoder asks for
                     maps_ok = maps_ok && tile_encode_maps(m, P.buf[b], P.Ix, P.Iy, P.g, v ? PREC_F32 : pl.prec,
-                                                          v ? PREC_F32 : pl.pflow, has_w, B.tp[l].R);
+                                                          v ? PREC_F32 : pl.pflow, has_w);
                     memcpy(img.data() + o + b * sizeof(m), m, sizeof(m));
                 }
             }
@@ -894,8 +894,10 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                 const PairCtx &c = pc[0];
                 const Geom g = geom_of(*c.pl, l);
                 tp = admm_tile_plan(g, tile_iters_of(p, rest));
+                bool ok = true;
                 for (int b = 0; b < 2 && tp.staged; ++b)
-                    tp.staged = tile_encode_maps(maps[b], bufs_of(c)[b], data_of(c)[0], data_of(c)[1], g, prec, pflow, has_w, tp.R);
+                    ok = ok && tile_encode_maps(maps[b], bufs_of(c)[b], data_of(c)[0], data_of(c)[1], g, prec, pflow, has_w);
+                if (!ok) tp = admm_tile_plan(g, tile_iters_of(p, rest), true);
             }
             std::vector<int> steps;
             for (int it = 0, step = 1; it < rest; it += step) {
@@ -1770,7 +1772,7 @@ of_status iterate_common(of_fields f, const float *Ix, const float *Iy, const fl
                             : cp ? cp_blocks(g)
                                  : (params->engine == OF_ENGINE_PLAIN
                                         ? admm_plain_blocks(g)
-                                        : admm_tile_blocks(admm_tile_plan(g, params->tol > 0.0 ? TILE_ITERS : 0)));
+                                        : admm_tile_blocks(admm_tile_plan(g, params->tol > 0.0 ? TILE_ITERS : 0, true)));
     if (nb_used > mb) return fail(OF_EINVAL, "internal: partial sums exceed the scratch layout");
     double *partials = (double *)(S + (NFIELDS + 6) * plane);
     Misc *misc = (Misc *)(S + (NFIELDS + 6) * plane + align_up((size_t)mb * sizeof(double), 256));
@@ -1790,10 +1792,9 @@ of_status iterate_common(of_fields f, const float *Ix, const float *Iy, const fl
     TilePlan tp;
     bool vec = W % 2 == 0 && pitch % 2 == 0;
     if (tile) {
-        tp = admm_tile_plan(g, params->tol > 0.0 ? TILE_ITERS : 0);
+        tp = admm_tile_plan(g, params->tol > 0.0 ? TILE_ITERS : 0, true);
         for (int q = 0; q < NFIELDS; ++q) vec = vec && (uintptr_t)user.f[q] % 8 == 0;
         vec = vec && (uintptr_t)Ix % 8 == 0 && (uintptr_t)Iy % 8 == 0 && (uintptr_t)It % 8 == 0 && (uintptr_t)scratch % 8 == 0;
-        tp.staged = false;
     }
     int launches = 0;
     for (int it = 0, step = 1; it < iters; it += step, ++launches) {

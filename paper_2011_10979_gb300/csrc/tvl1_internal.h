@@ -97,6 +97,8 @@ struct IterArgs {
 // The several-iterations ADMM tile kernel (k_admm_tile.cuh): blocks of TILE_WARPS warps hold frames
 // of 64 x TILE_WARPS R pixels, at most one block per SM and TILE_MAX_ITERS iterations per launch.
 constexpr int TILE_WARPS = 12, TILE_SMS = 152, TILE_MAX_ITERS = 8;
+// Rows of the staged form's frames (R is then ignored).
+constexpr int TILE_STAGED_HEIGHT = 48;
 // Iterations per launch where the number is fixed (ALG1's tile kernel too).
 constexpr int TILE_ITERS = 3;
 
@@ -268,8 +270,9 @@ void launch_parity_fix(const Fields &from, const Fields &to, Geom g, int prec, i
                        int want_done, cudaStream_t s);
 
 // ---------------------------------------------------------------- several iterations per launch (k_admm_tile.cu, k_cp_tile.cu)
-// The tiling of a single pair's level for launches of ni iterations (0: the rule's choice).
-TilePlan admm_tile_plan(Geom g, int ni);
+// The tiling of a single pair's level for launches of ni iterations (0: the rule's choice); direct:
+// without the staged form, which needs the library's own planes.
+TilePlan admm_tile_plan(Geom g, int ni, bool direct = false);
 // The tiling of n pairs' levels in one batched launch (gx: tiles in all).
 TilePlan admm_tile_plan_batch(const Geom *g, int n, int ni);
 int admm_tile_blocks(const TilePlan &p);  // partial-sum slots of a launch
@@ -280,7 +283,7 @@ void tile_set_plan(TileArgs &t, const TilePlan &p, int ni);
 // The staged form's tensor maps of a state buffer (its planes equally spaced) and the data planes;
 // false when the driver cannot encode them.
 bool tile_encode_maps(CUtensorMap maps[3], const Fields &f, const void *Ix, const void *Iy, Geom g, int prec,
-                      int prec_flow, bool has_w, int R);
+                      int prec_flow, bool has_w);
 void launch_admm_tile(const TileArgs &a, int prec, int prec_flow, cudaStream_t s);
 // Single pair: ni (2 or 3) consecutive iterations of k_cp in one
 // launch over TT x TT tiles (cp_tile_size: 32, or 16 on small levels), reading a.in and writing

@@ -141,7 +141,7 @@ cudaError_t run_group(std::vector<StepPair *> &G, const of_params *p, StepTables
     }
     // the ADMM tile kernel, several iterations per launch, by the built-in strip rule (as the whole
     // solve; the launches of 3, 3, 3 and 1 per ten iterations with the stopping test)
-    const bool tile = !(pdr || cp) && p->rows_per_warp == 0 && (p->engine == OF_ENGINE_FUSED || p->engine == OF_ENGINE_STREAM);
+    const bool tile = !(pdr || cp) && p->rows_per_warp == 0 && p->a_tilde_mode == 0 && (p->engine == OF_ENGINE_FUSED || p->engine == OF_ENGINE_STREAM);
     TilePlan tp;
     if (tile) {
         std::vector<Geom> gs;
@@ -200,7 +200,7 @@ cudaError_t run_group(std::vector<StepPair *> &G, const of_params *p, StepTables
             P.maps = T.dev + o_tm + 6 * sizeof(CUtensorMap) * k;
             for (int b = 0; b < 2; ++b) {
                 CUtensorMap m[3];  // aligned as the encoder asks for
-                if (!tile_encode_maps(m, P.buf[b], P.Ix, P.Iy, g, prec, pflow, has_w, tp.R)) return cudaErrorUnknown;
+                if (!tile_encode_maps(m, P.buf[b], P.Ix, P.Iy, g, prec, pflow, has_w)) return cudaErrorUnknown;
                 memcpy(h + o_tm + 6 * sizeof(CUtensorMap) * k + b * sizeof(m), m, sizeof(m));
             }
             for (int y = 0; y < tile_rows(tp, g); ++y)
