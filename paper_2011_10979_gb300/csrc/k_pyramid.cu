@@ -114,13 +114,80 @@ __global__ void k_derivatives(const float *__restrict__ I, Geom g, float *__rest
     Iy[o] = 0.5f * (__ldg(I + (size_t)id * g.pitch + j) - __ldg(I + (size_t)iu * g.pitch + j));
 }
 
+// ---- twofold FP32: a value as an unevaluated sum h + l of two FP32 numbers (about 48 bits), from the
+// error-free transformations of sums (Knuth's TwoSum) and products (by FMA).  The warping needs more
+// than FP32 (see k_warp) and FP64 runs at 1/64 of the FP32 rate here.
+struct F2 {
+    float h, l;
+};
+// a - b exactly
+__device__ __forceinline__ F2 two_diff(float a, float b) {
+    const float s = __fsub_rn(a, b), t = __fsub_rn(s, a);
+    return {s, __fsub_rn(__fsub_rn(a, __fsub_rn(s, t)), __fadd_rn(b, t))};
+}
+// a + b exactly
+__device__ __forceinline__ F2 two_sum(float a, float b) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+// h + l with l at most half an ulp of h
+__device__ __forceinline__ F2 renorm(float h, float l) {
+    const float s = __fadd_rn(h, l);
+    return {s, __fsub_rn(l, __fsub_rn(s, h))};
+}
+// p + w (q - p)
+__device__ __forceinline__ F2 lerp2(F2 p, F2 q, float w) {
+    const F2 d = two_diff(q.h, p.h);
+    const float e = __fadd_rn(d.l, __fsub_rn(q.l, p.l)), m = __fmul_rn(w, d.h);
+    const float ml = __fmaf_rn(w, e, __fmaf_rn(w, d.h, -m));
+    const F2 s = two_sum(p.h, m);
+    return {s.h, __fadd_rn(s.l, __fadd_rn(p.l, ml))};
+}
+// acc - g u, acc and g twofold
+__device__ __forceinline__ F2 sub_mul(F2 acc, F2 g, float u) {
+    const float m = __fmul_rn(g.h, u), ml = __fmaf_rn(g.l, u, __fmaf_rn(g.h, u, -m));
+    const F2 d = two_diff(acc.h, m);
+    return {d.h, __fadd_rn(d.l, __fsub_rn(acc.l, ml))};
+}
+// Rounds v, known to within `err`, to FP32; false when the interval straddles two FP32 numbers (Ziv's
+// rounding test), or when v is not finite.
+__device__ __forceinline__ bool round_safe(F2 v, float err, float &out) {
+    const F2 r = renorm(v.h, v.l);
+    out = __fadd_rn(r.h, __fadd_rn(r.l, err));
+    return out == __fadd_rn(r.h, __fsub_rn(r.l, err));
+}
+
+// The sample position j + d clamped to [0, n - 1] as a base index p, its neighbour q and the weight
+// w of q, an exact FP32 number: for d >= 0 the base is the pixel below the position and w its
+// fraction; for d < 0 the base is the pixel above and w the fraction of |d| (1 - fraction would
+// need more than 24 bits).
+__device__ __forceinline__ void split_pos(int j, float d, int n, int &p, int &q, float &w) {
+    w = 0.f;
+    if (!(d > (float)-j)) {  // at or below 0; also catches NaN
+        p = 0;
+    } else if (d >= (float)(n - 1 - j)) {
+        p = n - 1;
+    } else {
+        const float t = truncf(d);  // towards zero
+        w = fabsf(d - t);
+        p = j + (int)t;
+    }
+    // inside the image, 0 < j + d < n - 1, the neighbour is too; weight 0: the one FP64 would read
+    q = w != 0.f && d < 0.f ? p - 1 : min(p + 1, n - 1);
+}
+
 // Warp I1 and its derivatives to (x + u0, y + v0) (clamped), linearise around d0:
 // It = I1w - I0 - Ix u0 - Iy v0, so that rho(w, d) = Ix u + Iy v + beta w + It.
 // The block max of M_s = beta^2 + Ix^2 + Iy^2 (of the stored, rounded values) raises *ms_max.
-// The interpolation and It run in FP64 and are rounded once, when stored: It is a small difference
-// of terms up to |grad I| |d0|, and the L1 data term puts the flow of weakly textured pixels on the
-// line Ix u + Iy v + It = 0, so an FP32 It moved those pixels by up to a few 1e-3 px over a whole
-// schedule (measured against the FP64 oracle).  The kernel runs once per warp; FP64 costs little.
+// The results are those of the interpolation and It in FP64, rounded once when stored: It is a small
+// difference of terms up to |grad I| |d0|, and the L1 data term puts the flow of weakly textured
+// pixels on the line Ix u + Iy v + It = 0, so an FP32 It moved those pixels by up to a few 1e-3 px
+// over a whole schedule (measured against the FP64 oracle).  FP64 bounded the kernel (33 operations
+// of 64 cycles each per 32 pixels and SM quarter).  So the values are formed in twofold FP32, with an
+// error of some 2^-45 of the terms' magnitude, and rounded when an error of 2^-41 cannot change the
+// rounding; where it could (about one pixel in ten thousand, exact ties, non-finite values) the pixel
+// takes the FP64 path, so that every result is the FP64 path's, bit for bit.  Measured at 1920x1080:
+// 36 us against 233 all in FP64 (640x480 10 against 37).
 template <typename T, typename TF>
 __global__ void k_warp(const float *__restrict__ I0, const float *__restrict__ I1, const float *__restrict__ I1x,
                        const float *__restrict__ I1y, const TF *__restrict__ u0, const TF *__restrict__ v0, Geom g,
@@ -130,18 +197,48 @@ __global__ void k_warp(const float *__restrict__ I0, const float *__restrict__ I
     float ms = 0.f;
     if (i < g.H && j < g.W) {
         const size_t o = (size_t)i * g.pitch + j;
-        const float uu = Store<TF>::ld(u0 + o), vv = Store<TF>::ld(v0 + o);
-        int x0, y0;
-        double fx, fy;
-        split_pos_f64(j, uu, g.W, x0, fx);
-        split_pos_f64(i, vv, g.H, y0, fy);
-        const double w1 = bilinear_split_f64(I1, g.H, g.W, g.pitch, x0, fx, y0, fy);
-        const double gx = bilinear_split_f64(I1x, g.H, g.W, g.pitch, x0, fx, y0, fy);
-        const double gy = bilinear_split_f64(I1y, g.H, g.W, g.pitch, x0, fx, y0, fy);
-        Store<T>::st(Ix + o, (float)gx);
-        Store<T>::st(Iy + o, (float)gy);
-        Store<T>::st(It + o, (float)(w1 - (double)__ldg(I0 + o) - gx * (double)uu - gy * (double)vv));
-        const float gxr = Store<T>::ld(Ix + o), gyr = Store<T>::ld(Iy + o);
+        const float uu = Store<TF>::ld(u0 + o), vv = Store<TF>::ld(v0 + o), i0 = __ldg(I0 + o);
+        int xp, xq, yp, yq;
+        float wx, wy;
+        split_pos(j, uu, g.W, xp, xq, wx);
+        split_pos(i, vv, g.H, yp, yq, wy);
+        const size_t rp = (size_t)yp * g.pitch, rq = (size_t)yq * g.pitch;
+        float mag;  // sum of the magnitudes of the last interpolation's samples
+        auto sample = [&](const float *f) -> F2 {
+            const float a = __ldg(f + rp + xp), b = __ldg(f + rp + xq), c = __ldg(f + rq + xp), d = __ldg(f + rq + xq);
+            mag = fabsf(a) + fabsf(b) + (fabsf(c) + fabsf(d));
+            return lerp2(lerp2(F2{a, 0.f}, F2{b, 0.f}, wx), lerp2(F2{c, 0.f}, F2{d, 0.f}, wx), wy);
+        };
+        constexpr float EPS = 0x1p-41f, TINY = 1e-36f;  // TINY: products that underflow
+        auto bound = [&](float m) { return m > 0.f ? fmaf(m, EPS, TINY) : 0.f; };
+        const F2 w1 = sample(I1);
+        const float m1 = mag;
+        const F2 gx = sample(I1x);
+        const float mx = mag;
+        const F2 gy = sample(I1y);
+        const float my = mag;
+        float ix, iy, it;
+        F2 t = two_diff(w1.h, i0);
+        t.l = __fadd_rn(t.l, w1.l);
+        t = sub_mul(sub_mul(t, gx, uu), gy, vv);
+        const float mt = m1 + fabsf(i0) + mx * fabsf(uu) + my * fabsf(vv);
+        const bool okx = round_safe(gx, bound(mx), ix), oky = round_safe(gy, bound(my), iy);
+        if (!(round_safe(t, bound(mt), it) && okx && oky)) {
+            int x0, y0;
+            double fx, fy;
+            split_pos_f64(j, uu, g.W, x0, fx);
+            split_pos_f64(i, vv, g.H, y0, fy);
+            const double w1d = bilinear_split_f64(I1, g.H, g.W, g.pitch, x0, fx, y0, fy);
+            const double gxd = bilinear_split_f64(I1x, g.H, g.W, g.pitch, x0, fx, y0, fy);
+            const double gyd = bilinear_split_f64(I1y, g.H, g.W, g.pitch, x0, fx, y0, fy);
+            ix = (float)gxd;
+            iy = (float)gyd;
+            it = (float)(w1d - (double)i0 - gxd * (double)uu - gyd * (double)vv);
+        }
+        Store<T>::st(Ix + o, ix);
+        Store<T>::st(Iy + o, iy);
+        Store<T>::st(It + o, it);
+        const float gxr = storage_round<T>(ix), gyr = storage_round<T>(iy);
         ms = beta * beta + gxr * gxr + gyr * gyr;
     }
 #pragma unroll
