@@ -4,6 +4,8 @@
 // images, warping + linearisation with the per-warp max of M_s, and precision conversion.
 #include <math.h>
 
+#include <algorithm>
+
 #include "tvl1_device.cuh"
 
 namespace tvl1 {
@@ -188,11 +190,16 @@ __device__ __forceinline__ void split_pos(int j, float d, int n, int &p, int &q,
 // rounding; where it could (about one pixel in ten thousand, exact ties, non-finite values) the pixel
 // takes the FP64 path, so that every result is the FP64 path's, bit for bit.  Measured at 1920x1080:
 // 36 us against 233 all in FP64 (640x480 10 against 37).
-template <typename T, typename TF>
-__global__ void k_warp(const float *__restrict__ I0, const float *__restrict__ I1, const float *__restrict__ I1x,
-                       const float *__restrict__ I1y, const TF *__restrict__ u0, const TF *__restrict__ v0, Geom g,
-                       float beta, T *__restrict__ Ix, T *__restrict__ Iy, T *__restrict__ It, float *ms_max) {
+template <typename T, typename TF> __global__ void k_warp(const __grid_constant__ PairSet A, int cur, float beta) {
     __shared__ float red[B2X * B2Y / 32];
+    const PairIter &P = A.pairs ? A.pairs[blockIdx.z] : A.one;
+    const Geom g = P.g;
+    if (blockIdx.x * B2X >= g.W || blockIdx.y * B2Y >= g.H) return;  // beyond a smaller pair of the batch
+    const float *__restrict__ I0 = P.I0, *__restrict__ I1 = P.I1, *__restrict__ I1x = P.I1x, *__restrict__ I1y = P.I1y;
+    const TF *__restrict__ u0 = reinterpret_cast<const TF *>(P.buf[cur].f[F_U]);
+    const TF *__restrict__ v0 = reinterpret_cast<const TF *>(P.buf[cur].f[F_V]);
+    T *__restrict__ Ix = (T *)P.Ix, *__restrict__ Iy = (T *)P.Iy, *__restrict__ It = (T *)P.It;
+    float *ms_max = const_cast<float *>(P.ms_max);
     const int j = blockIdx.x * B2X + threadIdx.x, i = blockIdx.y * B2Y + threadIdx.y;
     float ms = 0.f;
     if (i < g.H && j < g.W) {
@@ -254,19 +261,127 @@ __global__ void k_warp(const float *__restrict__ I0, const float *__restrict__ I
     }
 }
 
-template <typename S, typename D>
-__global__ void k_convert(const S *__restrict__ src, D *__restrict__ dst, Geom g) {
+__global__ void k_warp_reset(const __grid_constant__ PairSet A) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= A.n) return;
+    float *m = const_cast<float *>(A.pairs[k].ms_max);
+    m[0] = 0.f;
+    reinterpret_cast<int *>(m)[1] = 0;  // the stop flag
+}
+
+// Everything a level starts with, one pixel per thread: the planes were filled, upsampled and
+// differentiated by up to 17 launches of a microsecond or two each, most of it launch and drain.
+template <typename TD, typename TF> __global__ void k_level_begin(const __grid_constant__ LevelArgs A) {
+    const PairIter &P = A.fine.pairs ? A.fine.pairs[blockIdx.z] : A.fine.one;
+    const Geom g = P.g;
     const int j = blockIdx.x * B2X + threadIdx.x, i = blockIdx.y * B2Y + threadIdx.y;
     if (i >= g.H || j >= g.W) return;
     const size_t o = (size_t)i * g.pitch + j;
-    Store<D>::st(dst + o, Store<S>::ld(src + o));
+    const Fields &to = P.buf[A.to];
+    float x[3] = {0.f, 0.f, 0.f};
+    if (!A.first) {
+        // fine pixel centre -> coarse x = (j + 0.5) * Wc / Wf - 0.5, clamped, as k_upsample
+        const PairIter &C = A.coarse.pairs ? A.coarse.pairs[blockIdx.z] : A.coarse.one;
+        const Geom gc = C.g;
+        const float sx = (float)gc.W / (float)g.W, sy = (float)gc.H / (float)g.H;
+        const float xc = clampf((j + 0.5f) * sx - 0.5f, 0.f, (float)(gc.W - 1));
+        const float yc = clampf((i + 0.5f) * sy - 0.5f, 0.f, (float)(gc.H - 1));
+        const float scale[3] = {1.f, (float)g.W / (float)gc.W, (float)g.H / (float)gc.H};
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            if (c > 0 || A.has_w)
+                x[c] = scale[c] * bilinear<TF>(reinterpret_cast<const TF *>(C.buf[A.from].f[F_W + c]), gc.H, gc.W, gc.pitch, xc, yc);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        stT<TF>(to.f[F_W + c], o, x[c]);
+        if (A.xbar) stT<TF>(to.f[F_WB + c], o, x[c]);
+    }
+#pragma unroll
+    for (int k = F_P1; k <= F_S; ++k) stT<TD>(to.f[k], o, 0.f);
+    const int jl = max(j - 1, 0), jr = min(j + 1, g.W - 1), iu = max(i - 1, 0), id = min(i + 1, g.H - 1);
+    const float *__restrict__ I = P.I1;
+    P.I1x[o] = 0.5f * (__ldg(I + (size_t)i * g.pitch + jr) - __ldg(I + (size_t)i * g.pitch + jl));
+    P.I1y[o] = 0.5f * (__ldg(I + (size_t)id * g.pitch + j) - __ldg(I + (size_t)iu * g.pitch + j));
 }
 
-template <typename T>
-__global__ void k_fill(T *__restrict__ dst, Geom g, float value) {
+template <typename TD, typename TF>
+__global__ void k_state_to_f32(const __grid_constant__ PairSet A, const __grid_constant__ PairSet B, int cur, int xbar) {
+    const PairIter &P = A.pairs ? A.pairs[blockIdx.z] : A.one, &Q = B.pairs ? B.pairs[blockIdx.z] : B.one;
+    const Geom g = P.g;
     const int j = blockIdx.x * B2X + threadIdx.x, i = blockIdx.y * B2Y + threadIdx.y;
     if (i >= g.H || j >= g.W) return;
-    Store<T>::st(dst + (size_t)i * g.pitch + j, value);
+    const size_t o = (size_t)i * g.pitch + j;
+    const Fields &f = P.buf[cur], &t = Q.buf[0];
+#pragma unroll
+    for (int k = 0; k < NFIELDS; ++k)
+        if (xbar || k < F_WB) stT<float>(t.f[k], o, is_flow_field(k) ? ldT<TF>(f.f[k], o) : ldT<TD>(f.f[k], o));
+}
+
+template <typename TF> __global__ void k_output(Fields f, Geom g, float *u, float *v, float *w) {
+    const int j = blockIdx.x * B2X + threadIdx.x, i = blockIdx.y * B2Y + threadIdx.y;
+    if (i >= g.H || j >= g.W) return;
+    const size_t o = (size_t)i * g.pitch + j;
+    u[o] = ldT<TF>(f.f[F_U], o);
+    v[o] = ldT<TF>(f.f[F_V], o);
+    w[o] = ldT<TF>(f.f[F_W], o);
+}
+
+// One pyramid step in one launch: a block stages the fine pixels its coarse tile needs (with the
+// blur's margin, mirrored at the border), blurs their rows in shared memory, and forms each coarse
+// pixel from the column blurs at its four fine neighbours.  The sums run in the order of k_blur_rows,
+// k_blur_cols and k_resample, so the results are theirs bit for bit; those pass two fine planes
+// through memory and took 45 us at 1920x1080.
+constexpr int PDX = 32, PDY = 16;
+struct PyrArgs {
+    const float *fine[2];
+    float *coarse[2];
+    Geom gf, gc;
+    GaussTaps t;
+    int nx, ny;  // fine columns and rows of a tile, at most
+};
+__global__ void __launch_bounds__(256) k_pyr_down(const __grid_constant__ PyrArgs A) {
+    extern __shared__ float sm[];
+    const int R = A.t.R, Hf = A.gf.H, Wf = A.gf.W, Hc = A.gc.H, Wc = A.gc.W;
+    const float *__restrict__ in = A.fine[blockIdx.z];
+    const float sx = (float)Wf / (float)Wc, sy = (float)Hf / (float)Hc;
+    auto px = [&](int j) { return clampf((j + 0.5f) * sx - 0.5f, 0.f, (float)(Wf - 1)); };
+    auto py = [&](int i) { return clampf((i + 0.5f) * sy - 0.5f, 0.f, (float)(Hf - 1)); };
+    const int j0 = blockIdx.x * PDX, i0 = blockIdx.y * PDY;
+    const int x0 = (int)floorf(px(j0)), y0 = (int)floorf(py(i0));
+    const int x1 = min((int)floorf(px(min(j0 + PDX, Wc) - 1)) + 1, Wf - 1), y1 = min((int)floorf(py(min(i0 + PDY, Hc) - 1)) + 1, Hf - 1);
+    const int nx = x1 - x0 + 1, ny = y1 - y0 + 1, aw = A.nx + 2 * R;
+    float *a = sm, *b = sm + (A.ny + 2 * R) * aw;  // the fine pixels; their rows blurred (pitch A.nx)
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    for (int r = ty; r < ny + 2 * R; r += 8) {
+        const float *row = in + (size_t)reflect_index(y0 - R + r, Hf) * A.gf.pitch;
+        for (int c = tx; c < nx + 2 * R; c += 32) a[r * aw + c] = __ldg(row + reflect_index(x0 - R + c, Wf));
+    }
+    __syncthreads();
+    for (int r = ty; r < ny + 2 * R; r += 8)
+        for (int c = tx; c < nx; c += 32) {
+            float acc = 0.f;
+            for (int k = 0; k <= 2 * R; ++k) acc += A.t.w[k] * a[r * aw + c + k];
+            b[r * A.nx + c] = acc;
+        }
+    __syncthreads();
+    const int j = j0 + tx;
+    if (j >= Wc) return;
+    const float x = px(j), xf = floorf(x), fx = x - xf;
+    const int xa = (int)xf - x0, xb = min((int)xf + 1, Wf - 1) - x0;
+    for (int i = i0 + ty; i < min(i0 + PDY, Hc); i += 8) {
+        const float y = py(i), yf = floorf(y), fy = y - yf;
+        const int ya = (int)yf - y0, yb = min((int)yf + 1, Hf - 1) - y0;
+        auto blur = [&](int yy, int xx) {
+            float acc = 0.f;
+            for (int k = 0; k <= 2 * R; ++k) acc += A.t.w[k] * b[(yy + k) * A.nx + xx];
+            return acc;
+        };
+        const float va = blur(ya, xa), vb = blur(ya, xb), vc = blur(yb, xa), vd = blur(yb, xb);
+        const float top = (1.f - fx) * va + fx * vb;
+        const float bot = (1.f - fx) * vc + fx * vd;
+        A.coarse[blockIdx.z][(size_t)i * A.gc.pitch + j] = (1.f - fy) * top + fy * bot;
+    }
 }
 
 dim3 grid2(int H, int W) { return dim3((W + B2X - 1) / B2X, (H + B2Y - 1) / B2Y); }
@@ -290,19 +405,32 @@ GaussTaps gauss_taps(float eta) {
     return t;
 }
 
-void launch_pyr_down(const float *fine, Geom gf, float *coarse, Geom gc, const GaussTaps &taps, float *scratch,
-                     cudaStream_t s) {
-    // scratch holds two Hf x pitch planes: rows-blurred and fully blurred
-    float *t1 = scratch, *t2 = scratch + (size_t)gf.H * gf.pitch;
-    k_blur_rows<<<grid2(gf.H, gf.W), dim3(B2X, B2Y), 0, s>>>(fine, t1, gf, taps);
-    k_blur_cols<<<grid2(gf.H, gf.W), dim3(B2X, B2Y), 0, s>>>(t1, t2, gf, taps);
-    k_resample<<<grid2(gc.H, gc.W), dim3(B2X, B2Y), 0, s>>>(t2, gf, coarse, gc);
-}
-
-void launch_upsample(const void *coarse, Geom gc, void *fine, Geom gf, float scale, int prec, cudaStream_t s) {
-    TVL1_DISPATCH_PREC(prec, T,
-                       k_upsample<T><<<grid2(gf.H, gf.W), dim3(B2X, B2Y), 0, s>>>(
-                           (const T *)coarse, gc, (T *)fine, gf, scale));
+void launch_pyr_down(const float *const *fine, Geom gf, float *const *coarse, Geom gc, int n, const GaussTaps &taps,
+                     float *scratch, cudaStream_t s) {
+    PyrArgs a{};
+    a.gf = gf;
+    a.gc = gc;
+    a.t = taps;
+    // fine pixels between the first and the last coarse centre of a tile, and the neighbours
+    a.nx = std::min(gf.W, (int)ceilf((PDX - 1) * ((float)gf.W / (float)gc.W)) + 3);
+    a.ny = std::min(gf.H, (int)ceilf((PDY - 1) * ((float)gf.H / (float)gc.H)) + 3);
+    const size_t rows = (size_t)a.ny + 2 * taps.R, smem = rows * (2 * (size_t)a.nx + 2 * taps.R) * sizeof(float);
+    if (smem <= 48 * 1024) {
+        for (int q = 0; q < n; ++q) {
+            a.fine[q] = fine[q];
+            a.coarse[q] = coarse[q];
+        }
+        const dim3 grid((gc.W + PDX - 1) / PDX, (gc.H + PDY - 1) / PDY, n);
+        k_pyr_down<<<grid, 256, smem, s>>>(a);
+        return;
+    }
+    for (int q = 0; q < n; ++q) {
+        // scratch holds two Hf x pitch planes: rows-blurred and fully blurred
+        float *t1 = scratch, *t2 = scratch + (size_t)gf.H * gf.pitch;
+        k_blur_rows<<<grid2(gf.H, gf.W), dim3(B2X, B2Y), 0, s>>>(fine[q], t1, gf, taps);
+        k_blur_cols<<<grid2(gf.H, gf.W), dim3(B2X, B2Y), 0, s>>>(t1, t2, gf, taps);
+        k_resample<<<grid2(gc.H, gc.W), dim3(B2X, B2Y), 0, s>>>(t2, gf, coarse[q], gc);
+    }
 }
 
 void launch_upsample_f32(const float *coarse, Geom gc, float *fine, Geom gf, float scale, cudaStream_t s) {
@@ -313,35 +441,40 @@ void launch_derivatives(const float *I, Geom g, float *Ix, float *Iy, cudaStream
     k_derivatives<<<grid2(g.H, g.W), dim3(B2X, B2Y), 0, s>>>(I, g, Ix, Iy);
 }
 
-void launch_warp(const float *I0, const float *I1, const float *I1x, const float *I1y, const void *u0,
-                 const void *v0, Geom g, float beta, void *Ix, void *Iy, void *It, float *ms_max, int prec,
-                 int prec_flow, cudaStream_t s) {
+namespace {
+
+dim3 grid_of(const PairSet &a) {
+    dim3 d = grid2(a.pairs ? a.grid.H : a.one.g.H, a.pairs ? a.grid.W : a.one.g.W);
+    d.z = a.pairs ? a.n : 1;
+    return d;
+}
+
+}  // namespace
+
+void launch_level_begin(const LevelArgs &a, int prec_dual, int prec_flow, cudaStream_t s) {
+    TVL1_DISPATCH_PREC(prec_dual, TD, TVL1_DISPATCH_PREC(prec_flow, TF,
+                       k_level_begin<TD, TF><<<grid_of(a.fine), dim3(B2X, B2Y), 0, s>>>(a)));
+}
+
+void launch_warp(const PairSet &a, int cur, float beta, int prec, int prec_flow, cudaStream_t s) {
     TVL1_DISPATCH_PREC(prec, T, TVL1_DISPATCH_PREC(prec_flow, TF,
-                       k_warp<T, TF><<<grid2(g.H, g.W), dim3(B2X, B2Y), 0, s>>>(
-                           I0, I1, I1x, I1y, (const TF *)u0, (const TF *)v0, g, beta, (T *)Ix, (T *)Iy, (T *)It,
-                           ms_max)));
+                       k_warp<T, TF><<<grid_of(a), dim3(B2X, B2Y), 0, s>>>(a, cur, beta)));
 }
 
-void launch_convert(const void *const *src, int src_prec, void *const *dst, int dst_prec, int nplanes, Geom g,
-                    cudaStream_t s) {
-    for (int k = 0; k < nplanes; ++k) {
-        if (!src[k] || !dst[k]) continue;
-        TVL1_DISPATCH_PREC(src_prec, S,
-                           TVL1_DISPATCH_PREC(dst_prec, D,
-                                              k_convert<S, D><<<grid2(g.H, g.W), dim3(B2X, B2Y), 0, s>>>(
-                                                  (const S *)src[k], (D *)dst[k], g)));
-    }
+void launch_warp_reset(const PairSet &a, cudaStream_t s) {
+    // one pair: ms_max and the stop flag are adjacent
+    if (!a.pairs) cudaMemsetAsync(const_cast<float *>(a.one.ms_max), 0, sizeof(float) + sizeof(int), s);
+    else k_warp_reset<<<(a.n + 127) / 128, 128, 0, s>>>(a);
 }
 
-void launch_fill(void *const *dst, int prec, int nplanes, Geom g, float value, cudaStream_t s) {
-    for (int k = 0; k < nplanes; ++k) {
-        if (!dst[k]) continue;
-        TVL1_DISPATCH_PREC(prec, T, k_fill<T><<<grid2(g.H, g.W), dim3(B2X, B2Y), 0, s>>>((T *)dst[k], g, value));
-    }
+void launch_state_to_f32(const PairSet &from, const PairSet &to, int cur, int xbar, int prec_dual, int prec_flow,
+                         cudaStream_t s) {
+    TVL1_DISPATCH_PREC(prec_dual, TD, TVL1_DISPATCH_PREC(prec_flow, TF,
+                       k_state_to_f32<TD, TF><<<grid_of(from), dim3(B2X, B2Y), 0, s>>>(from, to, cur, xbar)));
 }
 
-void launch_copy_planes(const void *const *src, void *const *dst, int nplanes, Geom g, int prec, cudaStream_t s) {
-    launch_convert(src, prec, dst, prec, nplanes, g, s);
+void launch_output(const Fields &f, Geom g, float *u, float *v, float *w, int prec_flow, cudaStream_t s) {
+    TVL1_DISPATCH_PREC(prec_flow, TF, k_output<TF><<<grid2(g.H, g.W), dim3(B2X, B2Y), 0, s>>>(f, g, u, v, w));
 }
 
 }  // namespace tvl1

@@ -28,12 +28,13 @@ __global__ void k_reduce_check(const double *partials, int n, double *out, doubl
     }
 }
 
-__global__ void k_sum(const double *partials, int n, double *out) {
+__global__ void k_sum(const double *p0, const double *p1, int n, double *out0, double *out1) {
     __shared__ double red[32];
+    const double *partials = blockIdx.x ? p1 : p0;
     double v = 0.0;
     for (int k = threadIdx.x; k < n; k += blockDim.x) v += partials[k];
     const double tot = block_sum(v, red);
-    if (threadIdx.x == 0) out[0] = tot;
+    if (threadIdx.x == 0) *(blockIdx.x ? out1 : out0) = tot;
 }
 
 __global__ void k_count_iters(long long *counter, const int *done, int n) {
@@ -129,7 +130,12 @@ void launch_reduce_check(const double *partials, int n, double *out, double rows
     k_reduce_check<<<1, 1024, 0, s>>>(partials, n, out, rows, tol, done, iters_counter, add_iters);
 }
 
-void launch_sum(const double *partials, int n, double *out, cudaStream_t s) { k_sum<<<1, 1024, 0, s>>>(partials, n, out); }
+void launch_sum(const double *partials, int n, double *out, cudaStream_t s) {
+    k_sum<<<1, 1024, 0, s>>>(partials, partials, n, out, out);
+}
+void launch_sum2(const double *p0, const double *p1, int n, double *out0, double *out1, cudaStream_t s) {
+    k_sum<<<2, 1024, 0, s>>>(p0, p1, n, out0, out1);
+}
 
 void launch_count_iters(long long *counter, const int *done, int n, cudaStream_t s) {
     k_count_iters<<<1, 1, 0, s>>>(counter, done, n);

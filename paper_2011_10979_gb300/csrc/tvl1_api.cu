@@ -635,6 +635,10 @@ of_status upload_tables(of_ctx *ctx, const Batch &B, const of_params *p) {
             P.ms_max = &misc->ms_max;
             P.done = p->tol > 0.0 ? &misc->done : nullptr;
             P.tmp = (float *)(A + pl.tmp);
+            P.I0 = (const float *)(A + pl.img0[l]);
+            P.I1 = (const float *)(A + pl.img1[l]);
+            P.I1x = (float *)(A + pl.I1x);
+            P.I1y = (float *)(A + pl.I1y);
             if (B.maps_off[l][v] > 0 && !B.res[l][k]) {
                 const size_t o = B.maps_off[l][v] + 6 * sizeof(CUtensorMap) * k;
                 P.maps = ctx->arena + B.table_off + o;
@@ -762,10 +766,9 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
         cudaMemsetAsync(c.misc, 0, sizeof(Misc), s);
         if (p->c_adapt_iters > 0) launch_c_init(&c.misc->c_cur, pdr ? 1.f : p->c, s);  // pDR: theta
         for (int l = 1; l < L; ++l) {
-            launch_pyr_down((float *)(c.A + pl.img0[l - 1]), geom_of(pl, l - 1), (float *)(c.A + pl.img0[l]),
-                            geom_of(pl, l), taps, (float *)(c.A + pl.blur), s);
-            launch_pyr_down((float *)(c.A + pl.img1[l - 1]), geom_of(pl, l - 1), (float *)(c.A + pl.img1[l]),
-                            geom_of(pl, l), taps, (float *)(c.A + pl.blur), s);
+            const float *fine[2] = {(float *)(c.A + pl.img0[l - 1]), (float *)(c.A + pl.img1[l - 1])};
+            float *coarse[2] = {(float *)(c.A + pl.img0[l]), (float *)(c.A + pl.img1[l])};
+            launch_pyr_down(fine, geom_of(pl, l - 1), coarse, geom_of(pl, l), 2, taps, (float *)(c.A + pl.blur), s);
         }
     }
 
@@ -774,62 +777,58 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
     auto bufs_of = [&](const PairCtx &c) { return in32 ? c.buf32 : c.buf; };
     auto data_of = [&](const PairCtx &c) { return in32 ? c.data32 : c.data; };
 
-    for (int l = L - 1; l >= B.out_level; --l) {
-        for (int q = 0; q < n; ++q) {
-            const PairCtx &c = pc[q];
-            const Plan &pl = *c.pl;
-            const Geom g = geom_of(pl, l);
-            const Fields *bf = bufs_of(c);
-            if (l == L - 1) {
-                launch_fill(bf[cur].f + F_W, pflow, 3, g, 0.f, s);
-            } else {
-                const Geom gc = geom_of(pl, l + 1);
-                const int nxt = cur ^ 1;
-                launch_upsample(bf[cur].f[F_W], gc, bf[nxt].f[F_W], g, 1.f, pflow, s);
-                launch_upsample(bf[cur].f[F_U], gc, bf[nxt].f[F_U], g, (float)g.W / (float)gc.W, pflow, s);
-                launch_upsample(bf[cur].f[F_V], gc, bf[nxt].f[F_V], g, (float)g.H / (float)gc.H, pflow, s);
-            }
-            const int now = l == L - 1 ? cur : cur ^ 1;
-            // duals p, q, s restart at 0 (ALG1 keeps its dual in the flow fields' type)
-            launch_fill(bf[now].f + F_P1, cp ? pflow : prec, F_S - F_P1 + 1, g, 0.f, s);
-            if (!has_w) launch_fill(bf[now].f + F_W, pflow, 1, g, 0.f, s);
-            if (pdr || cp) {  // pDR: Xbar = X; ALG1: the extrapolated point starts at X
-                const void *src[3] = {bf[now].f[F_W], bf[now].f[F_U], bf[now].f[F_V]};
-                void *dst[3] = {bf[now].f[F_WB], bf[now].f[F_UB], bf[now].f[F_VB]};
-                launch_copy_planes(src, dst, 3, g, pflow, s);
-            }
-            launch_derivatives((float *)(c.A + pl.img1[l]), g, (float *)(c.A + pl.I1x), (float *)(c.A + pl.I1y), s);
+    // the pairs' planes at level l, in the storage precision (v = 0) or the FP32 last warp's (v = 1)
+    auto set_of = [&](int l, int v) {
+        PairSet a;
+        if (batched) {
+            a.pairs = (const PairIter *)(ctx->arena + B.table_off + B.pairs_off[l][v]);
+            a.n = n;
+            a.grid = B.gmax[l];
+            return a;
         }
-        if (l != L - 1) cur ^= 1;
+        const PairCtx &c = pc[0];
+        const Plan &pl = *c.pl;
+        const void *const *dat = v ? c.data32 : c.data;
+        a.one.g = geom_of(pl, l);
+        for (int b = 0; b < 2; ++b) a.one.buf[b] = v ? c.buf32[b] : c.buf[b];
+        a.one.Ix = dat[0];
+        a.one.Iy = dat[1];
+        a.one.It = dat[2];
+        a.one.ms_max = &c.misc->ms_max;
+        a.one.I0 = (const float *)(c.A + pl.img0[l]);
+        a.one.I1 = (const float *)(c.A + pl.img1[l]);
+        a.one.I1x = (float *)(c.A + pl.I1x);
+        a.one.I1y = (float *)(c.A + pl.I1y);
+        return a;
+    };
+    for (int l = L - 1; l >= B.out_level; --l) {
+        // level transfer; the duals restart at 0 (ALG1 keeps its dual in the flow fields' type); pDR: Xbar
+        // = X; ALG1: the extrapolated point starts at X
+        LevelArgs la;
+        la.fine = set_of(l, 0);
+        la.first = l == L - 1;
+        la.from = cur;
+        if (!la.first) {
+            la.coarse = set_of(l + 1, 0);
+            cur ^= 1;
+        }
+        la.to = cur;
+        la.has_w = has_w;
+        la.xbar = pdr || cp;
+        launch_level_begin(la, cp ? pflow : prec, pflow, s);
         for (int wp = 0; wp < p->warps; ++wp) {
             const bool last_warp = (l == B.out_level) && (wp == p->warps - 1);
             const bool switch32 = B.pl[0].use32_last && l == 0 && wp == p->warps - 1;
-            for (int q = 0; q < n; ++q) {
-                const PairCtx &c = pc[q];
-                const Plan &pl = *c.pl;
-                const Geom g = geom_of(pl, l);
-                if (switch32) {
-                    // precision policy: the finest level's last warp runs with FP32 storage
-                    launch_convert(c.buf[cur].f + F_W, pflow, c.buf32[0].f + F_W, PREC_F32, 3, g, s);
-                    launch_convert(c.buf[cur].f + F_P1, cp ? pflow : prec, c.buf32[0].f + F_P1, PREC_F32,
-                                   F_S - F_P1 + 1, g, s);
-                    launch_convert(c.buf[cur].f + F_WB, pflow, c.buf32[0].f + F_WB, PREC_F32, 3, g, s);
-                }
-                const Fields *bf = switch32 ? c.buf32 : bufs_of(c);
-                const int cc = switch32 ? 0 : cur;
-                const void *const *dat = switch32 ? c.data32 : data_of(c);
-                const int pw = switch32 ? PREC_F32 : prec, pwf = switch32 ? PREC_F32 : pflow;
-                cudaMemsetAsync(&c.misc->ms_max, 0, sizeof(float) + sizeof(int), s);  // ms_max and done
-                launch_warp((float *)(c.A + pl.img0[l]), (float *)(c.A + pl.img1[l]), (float *)(c.A + pl.I1x),
-                            (float *)(c.A + pl.I1y), bf[cc].f[F_U], bf[cc].f[F_V], g, p->beta, (void *)dat[0],
-                            (void *)dat[1], (void *)dat[2], &c.misc->ms_max, pw, pwf, s);
-            }
+            // precision policy: the finest level's last warp runs with FP32 storage
+            if (switch32) launch_state_to_f32(set_of(l, 0), set_of(l, 1), cur, pdr || cp, cp ? pflow : prec, pflow, s);
             if (switch32) {
                 in32 = true;
                 cur = 0;
                 prec = PREC_F32;
                 pflow = PREC_F32;
             }
+            launch_warp_reset(set_of(l, in32), s);
+            launch_warp(set_of(l, in32), cur, p->beta, prec, pflow, s);
             const int start = cur;
             // adaptive steps (single pair; ADMM: c, pDR: sigma and tau with sigma tau fixed): the
             // level's first warp runs its first c_adapt_iters iterations one per-iteration launch
@@ -1110,13 +1109,10 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                 if (!has_w) fe.f[F_W] = nullptr;
                 const void *const *dat = data_of(c);
                 launch_energy(fe, dat[0], dat[1], dat[2], g, p->beta, p->lambda, prec, pflow, pe, pd, s);
-                launch_sum(pe, energy_blocks(g), &c.misc->energy, s);
-                launch_sum(pd, energy_blocks(g), &c.misc->dual, s);
+                launch_sum2(pe, pd, energy_blocks(g), &c.misc->energy, &c.misc->dual, s);
                 float *out = (float *)(c.A + pl.out);
                 const size_t on = (size_t)pl.H[pl.out_level] * pl.P[pl.out_level];
-                const void *src[3] = {bufs_of(c)[cur].f[F_U], bufs_of(c)[cur].f[F_V], bufs_of(c)[cur].f[F_W]};
-                void *dst[3] = {out, out + on, out + 2 * on};
-                launch_convert(src, pflow, dst, PREC_F32, 3, g, s);
+                launch_output(bufs_of(c)[cur], g, out, out + on, out + 2 * on, pflow, s);
             }
         }
     }
@@ -1666,7 +1662,7 @@ of_status of_pyr_down(const float *fine, int Hf, int Wf, int pf, float *coarse, 
     if (!(eta > 0.f && eta < 1.f)) return fail(OF_EINVAL, "eta must lie in (0, 1)");
     GaussTaps t = gauss_taps(eta);
     if (t.R < 0) return fail(OF_EINVAL, "eta too small");
-    launch_pyr_down(fine, Geom{Hf, Wf, pf}, coarse, Geom{Hc, Wc, pc}, t, scratch, (cudaStream_t)stream);
+    launch_pyr_down(&fine, Geom{Hf, Wf, pf}, &coarse, Geom{Hc, Wc, pc}, 1, t, scratch, (cudaStream_t)stream);
     OF_CUDA(cudaGetLastError());
     return OF_OK;
 }
@@ -1693,7 +1689,19 @@ of_status of_warp_linearise(const float *I0, const float *I1, const float *I1x, 
                             float *ms_max, void *stream) {
     if (!I0 || !I1 || !I1x || !I1y || !u0 || !v0 || !Ix || !Iy || !It || !ms_max) return fail(OF_EINVAL, "NULL pointer");
     if (H < 1 || W < 1 || pitch < W) return fail(OF_EINVAL, "bad sizes or pitch");
-    launch_warp(I0, I1, I1x, I1y, u0, v0, Geom{H, W, pitch}, beta, Ix, Iy, It, ms_max, PREC_F32, PREC_F32, (cudaStream_t)stream);
+    PairSet a;
+    a.one.g = Geom{H, W, pitch};
+    a.one.I0 = I0;
+    a.one.I1 = I1;
+    a.one.I1x = const_cast<float *>(I1x);
+    a.one.I1y = const_cast<float *>(I1y);
+    a.one.buf[0].f[F_U] = const_cast<float *>(u0);
+    a.one.buf[0].f[F_V] = const_cast<float *>(v0);
+    a.one.Ix = Ix;
+    a.one.Iy = Iy;
+    a.one.It = It;
+    a.one.ms_max = ms_max;
+    launch_warp(a, 0, beta, PREC_F32, PREC_F32, (cudaStream_t)stream);
     OF_CUDA(cudaGetLastError());
     return OF_OK;
 }
@@ -1888,8 +1896,7 @@ of_status of_energy(const float *w, const float *u, const float *v, const float 
     f.f[F_V] = (void *)v;
     f.f[F_S] = (void *)s;
     launch_energy(f, Ix, Iy, It, g, beta, lambda, PREC_F32, PREC_F32, buf, buf + nb, st);
-    launch_sum(buf, nb, buf + 2 * nb, st);
-    launch_sum(buf + nb, nb, buf + 2 * nb + 1, st);
+    launch_sum2(buf, buf + nb, nb, buf + 2 * nb, buf + 2 * nb + 1, st);
     double h[2];
     cudaError_t e = cudaMemcpyAsync(h, buf + 2 * nb, sizeof(h), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -50,6 +50,8 @@ struct __align__(16) PairIter {
     const int *done;
     float *tmp;  // the pair's FP32 scratch planes (pDR engine)
     const void *maps;  // tensor maps of the staged tile kernel: per buffer, flow, dual and data planes
+    const float *I0, *I1;  // the level's images
+    float *I1x, *I1y;      // the derivatives of I1
 };
 
 // Device scalars of one pair in a batch, for the batched reductions: the partial sums of the
@@ -199,20 +201,38 @@ struct GaussTaps {
     int R;
 };
 GaussTaps gauss_taps(float eta);
-void launch_pyr_down(const float *fine, Geom gf, float *coarse, Geom gc, const GaussTaps &taps,
+// One pyramid step of n (1 or 2) images of one geometry.  scratch: two planes of the fine geometry per
+// image, used only where a tile's fine pixels do not fit in shared memory (eta far below 1/2).
+void launch_pyr_down(const float *const *fine, Geom gf, float *const *coarse, Geom gc, int n, const GaussTaps &taps,
                      float *scratch, cudaStream_t s);
-void launch_upsample(const void *coarse, Geom gc, void *fine, Geom gf, float scale, int prec, cudaStream_t s);
 void launch_upsample_f32(const float *coarse, Geom gc, float *fine, Geom gf, float scale, cudaStream_t s);
 void launch_derivatives(const float *I, Geom g, float *Ix, float *Iy, cudaStream_t s);
-// u0, v0 in precision `prec_flow`, the outputs Ix, Iy, It in `prec`; ms_max raised with atomicMax.
-void launch_warp(const float *I0, const float *I1, const float *I1x, const float *I1y, const void *u0,
-                 const void *v0, Geom g, float beta, void *Ix, void *Iy, void *It, float *ms_max,
-                 int prec, int prec_flow, cudaStream_t s);
-// Element-wise precision conversion of `nplanes` planes (same geometry).
-void launch_convert(const void *const *src, int src_prec, void *const *dst, int dst_prec, int nplanes,
-                    Geom g, cudaStream_t s);
-void launch_fill(void *const *dst, int prec, int nplanes, Geom g, float value, cudaStream_t s);
-void launch_copy_planes(const void *const *src, void *const *dst, int nplanes, Geom g, int prec, cudaStream_t s);
+
+// The pairs a launch of the kernels below covers: one, passed by value (pairs == nullptr), or pairs[0 .. n)
+// of a table, `grid` the largest geometry.
+struct PairSet {
+    PairIter one{};
+    const PairIter *pairs = nullptr;
+    int n = 1;
+    Geom grid{};
+};
+// The start of a level: w, u, v upsampled from the coarser level's buffer `from` (from_set empty: zero)
+// into this level's buffer `to`, zero w when beta = 0, the duals zero (in prec_dual), with xbar the
+// barred copies of w, u, v, and the derivatives of I1.
+struct LevelArgs {
+    PairSet fine, coarse;
+    int first = 0, from = 0, to = 0, has_w = 1, xbar = 0;
+};
+void launch_level_begin(const LevelArgs &a, int prec_dual, int prec_flow, cudaStream_t s);
+// Warping and linearisation around the flow (u, v) of buffer `cur` (prec_flow), outputs Ix, Iy, It in
+// `prec`; ms_max raised with atomicMax (it and the stop flag behind it are zeroed by launch_warp_reset).
+void launch_warp(const PairSet &a, int cur, float beta, int prec, int prec_flow, cudaStream_t s);
+void launch_warp_reset(const PairSet &a, cudaStream_t s);
+// The state of buffer `cur` of `from` (duals in prec_dual, the rest in prec_flow) as FP32 in buffer 0 of `to`.
+void launch_state_to_f32(const PairSet &from, const PairSet &to, int cur, int xbar, int prec_dual, int prec_flow,
+                         cudaStream_t s);
+// u, v, w (prec_flow) as FP32.
+void launch_output(const Fields &f, Geom g, float *u, float *v, float *w, int prec_flow, cudaStream_t s);
 
 // ---------------------------------------------------------------- ADMM (k_admm.cu)
 // Fused engine: one kernel per iteration, reads args.in, writes args.out.  The multipliers
@@ -257,6 +277,8 @@ int energy_blocks(Geom g);
 void launch_energy(const Fields &f, const void *Ix, const void *Iy, const void *It, Geom g, float beta,
                    float lambda, int prec, int prec_flow, double *partials_e, double *partials_d, cudaStream_t s);
 void launch_sum(const double *partials, int n, double *out, cudaStream_t s);
+// The same for two arrays at once.
+void launch_sum2(const double *p0, const double *p1, int n, double *out0, double *out1, cudaStream_t s);
 // Adds `n` to *counter unless *done is set.
 void launch_count_iters(long long *counter, const int *done, int n, cudaStream_t s);
 // Batched forms over `npairs` pairs (one block per pair): the stopping test on each pair's

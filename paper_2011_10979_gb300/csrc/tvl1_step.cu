@@ -85,10 +85,9 @@ void step_pair_start(StepPair &q, const float *I0, const float *I1, const of_par
     cudaMemsetAsync(misc_of(q), 0, sizeof(Misc), s);
     const GaussTaps taps = gauss_taps(p->eta);
     for (int l = 1; l < pl.L; ++l) {
-        launch_pyr_down((float *)(q.A + pl.img0[l - 1]), geom_of(pl, l - 1), (float *)(q.A + pl.img0[l]),
-                        geom_of(pl, l), taps, (float *)(q.A + pl.blur), s);
-        launch_pyr_down((float *)(q.A + pl.img1[l - 1]), geom_of(pl, l - 1), (float *)(q.A + pl.img1[l]),
-                        geom_of(pl, l), taps, (float *)(q.A + pl.blur), s);
+        const float *fine[2] = {(float *)(q.A + pl.img0[l - 1]), (float *)(q.A + pl.img1[l - 1])};
+        float *coarse[2] = {(float *)(q.A + pl.img0[l]), (float *)(q.A + pl.img1[l])};
+        launch_pyr_down(fine, geom_of(pl, l - 1), coarse, geom_of(pl, l), 2, taps, (float *)(q.A + pl.blur), s);
     }
 }
 
@@ -194,6 +193,10 @@ cudaError_t run_group(std::vector<StepPair *> &G, const of_params *p, StepTables
         P.ms_max = &m->ms_max;
         P.done = p->tol > 0.0 ? &m->done : nullptr;
         P.tmp = (float *)(q.A + q.pl.tmp);
+        P.I0 = (const float *)(q.A + q.pl.img0[q.l]);
+        P.I1 = (const float *)(q.A + q.pl.img1[q.l]);
+        P.I1x = (float *)(q.A + q.pl.I1x);
+        P.I1y = (float *)(q.A + q.pl.I1y);
         pl[k] = k;
         const int t0 = t;
         if (tile) {
@@ -225,6 +228,13 @@ cudaError_t run_group(std::vector<StepPair *> &G, const of_params *p, StepTables
     const TileRef *dtr = (const TileRef *)(T.dev + o_tr);
     double *part = (double *)(T.dev + o_pa);
     const Coefs k = coefs_of(p);
+    // the warping of every pair around its current flow
+    PairSet ws;
+    ws.pairs = dpi;
+    ws.n = n;
+    ws.grid = gmax;
+    launch_warp_reset(ws, s);
+    launch_warp(ws, 0, p->beta, prec, pflow, s);
     int launches = 0;
     for (int it = 0, step = 1; it < p->iters; it += step, ++launches) {
         step = tile ? tile_step(p, tp.ni, it, p->iters) : 1;
@@ -283,49 +293,44 @@ cudaError_t step_run(std::vector<StepPair *> &act, const of_params *p, StepTable
     const bool pdr = p->method == OF_PDR, cp = p->method == OF_CP;
     const bool has_w = p->beta != 0.f;
     std::vector<StepPair *> g16, g32;
-    // stage set-up of every pair: level transfer at a level's first warp, then the warping
+    // stage set-up of every pair: level transfer at a level's first warp
+    auto set_of = [](const StepPair &q, int l) {
+        PairSet a;
+        const Bufs bf = bufs_of(q);
+        a.one.g = geom_of(q.pl, l);
+        a.one.buf[0] = bf.st[0];
+        a.one.buf[1] = bf.st[1];
+        a.one.I1 = (const float *)(q.A + q.pl.img1[l]);
+        a.one.I1x = (float *)(q.A + q.pl.I1x);
+        a.one.I1y = (float *)(q.A + q.pl.I1y);
+        return a;
+    };
     for (StepPair *qp : act) {
         StepPair &q = *qp;
         const Plan &pl = q.pl;
-        const Geom g = geom_of(pl, q.l);
-        Bufs bf = bufs_of(q);
         if (q.wp == 0) {
-            if (q.l == pl.L - 1) {
-                launch_fill(bf.st[q.cur].f + F_W, q.pflow, 3, g, 0.f, s);
-            } else {
-                const Geom gc = geom_of(pl, q.l + 1);
-                const int nxt = q.cur ^ 1;
-                launch_upsample(bf.st[q.cur].f[F_W], gc, bf.st[nxt].f[F_W], g, 1.f, q.pflow, s);
-                launch_upsample(bf.st[q.cur].f[F_U], gc, bf.st[nxt].f[F_U], g, (float)g.W / (float)gc.W, q.pflow, s);
-                launch_upsample(bf.st[q.cur].f[F_V], gc, bf.st[nxt].f[F_V], g, (float)g.H / (float)gc.H, q.pflow, s);
-                q.cur = nxt;
+            LevelArgs la;
+            la.fine = set_of(q, q.l);
+            la.first = q.l == pl.L - 1;
+            la.from = q.cur;
+            if (!la.first) {
+                la.coarse = set_of(q, q.l + 1);
+                q.cur ^= 1;
             }
-            // duals restart at 0 (ALG1 keeps its dual in the flow fields' type)
-            launch_fill(bf.st[q.cur].f + F_P1, cp ? q.pflow : q.prec, F_S - F_P1 + 1, g, 0.f, s);
-            if (!has_w) launch_fill(bf.st[q.cur].f + F_W, q.pflow, 1, g, 0.f, s);
-            if (pdr || cp) {
-                const void *src[3] = {bf.st[q.cur].f[F_W], bf.st[q.cur].f[F_U], bf.st[q.cur].f[F_V]};
-                void *dst[3] = {bf.st[q.cur].f[F_WB], bf.st[q.cur].f[F_UB], bf.st[q.cur].f[F_VB]};
-                launch_copy_planes(src, dst, 3, g, q.pflow, s);
-            }
-            launch_derivatives((float *)(q.A + pl.img1[q.l]), g, (float *)(q.A + pl.I1x), (float *)(q.A + pl.I1y), s);
+            la.to = q.cur;
+            la.has_w = has_w;
+            la.xbar = pdr || cp;
+            launch_level_begin(la, cp ? q.pflow : q.prec, q.pflow, s);
         }
         if (pl.use32_last && q.l == 0 && q.wp == p->warps - 1 && !q.in32) {
             // precision policy: the finest level's last warp runs with FP32 storage
-            const Fields to = fields_at(q.A + pl.stA32, pl.plane32);
-            launch_convert(bf.st[q.cur].f + F_W, q.pflow, to.f + F_W, PREC_F32, 3, g, s);
-            launch_convert(bf.st[q.cur].f + F_P1, cp ? q.pflow : q.prec, to.f + F_P1, PREC_F32, F_S - F_P1 + 1, g, s);
-            launch_convert(bf.st[q.cur].f + F_WB, q.pflow, to.f + F_WB, PREC_F32, 3, g, s);
+            const PairSet from = set_of(q, 0);
+            const int cur = q.cur, pd = cp ? q.pflow : q.prec, pf = q.pflow;
             q.in32 = true;
             q.cur = 0;
             q.prec = q.pflow = PREC_F32;
-            bf = bufs_of(q);
+            launch_state_to_f32(from, set_of(q, 0), cur, pdr || cp, pd, pf, s);
         }
-        Misc *m = misc_of(q);
-        cudaMemsetAsync(&m->ms_max, 0, sizeof(float) + sizeof(int), s);  // ms_max and the stop flag
-        launch_warp((float *)(q.A + pl.img0[q.l]), (float *)(q.A + pl.img1[q.l]), (float *)(q.A + pl.I1x),
-                    (float *)(q.A + pl.I1y), bf.st[q.cur].f[F_U], bf.st[q.cur].f[F_V], g, p->beta, (void *)bf.dat[0],
-                    (void *)bf.dat[1], (void *)bf.dat[2], &m->ms_max, q.prec, q.pflow, s);
         (q.in32 && pl.prec != PREC_F32 ? g32 : g16).push_back(qp);
     }
     cudaError_t e = cudaSuccess;
@@ -351,13 +356,10 @@ cudaError_t step_run(std::vector<StepPair *> &act, const of_params *p, StepTable
         if (pdr || cp) fe.f[F_S] = nullptr;
         if (!has_w) fe.f[F_W] = nullptr;
         launch_energy(fe, bf.dat[0], bf.dat[1], bf.dat[2], g, p->beta, p->lambda, q.prec, q.pflow, pe, pd, s);
-        launch_sum(pe, energy_blocks(g), &m->energy, s);
-        launch_sum(pd, energy_blocks(g), &m->dual, s);
+        launch_sum2(pe, pd, energy_blocks(g), &m->energy, &m->dual, s);
         float *out = (float *)(q.A + pl.out);
         const size_t on = (size_t)pl.H[pl.out_level] * pl.P[pl.out_level];
-        const void *src[3] = {bf.st[q.cur].f[F_U], bf.st[q.cur].f[F_V], bf.st[q.cur].f[F_W]};
-        void *dst[3] = {out, out + on, out + 2 * on};
-        launch_convert(src, q.pflow, dst, PREC_F32, 3, g, s);
+        launch_output(bf.st[q.cur], g, out, out + on, out + 2 * on, q.pflow, s);
         q.finished = true;
     }
     return cudaGetLastError();
