@@ -69,8 +69,9 @@ Plan make_plan(int H, int W, const of_params *p) {
         const Geom g{pl.H[l], pl.W[l], pl.P[l]};
         mb = std::max({mb, admm_fused_blocks(g, p->rows_per_warp != 0 ? 1 : 0), admm_plain_blocks(g),
                        pdr_plain_blocks(g, PARTIAL_ROWS_MIN), cp_blocks(g, PARTIAL_ROWS_MIN), energy_blocks(g),
-                       adapt_blocks(g), pdr_tile_blocks(g), cp_tile_blocks(g)});
+                       adapt_blocks(g), pdr_tile_blocks(g)});
         for (int q = 0; q < 4; ++q) mb = std::max(mb, admm_tile_blocks(admm_tile_plan(g, q & 1 ? TILE_ITERS : 0, q & 2)));
+        for (int q = 0; q < 2; ++q) mb = std::max(mb, admm_tile_blocks(cp_tile_plan(g, q ? TILE_ITERS : 0)));
     }
     pl.max_blocks = mb;
     pl.partials = take(3 * (size_t)mb * sizeof(double));
@@ -311,7 +312,7 @@ bool admm_tile_of(const of_params *p) {
            (p->engine == OF_ENGINE_FUSED || p->engine == OF_ENGINE_STREAM);
 }
 
-// Whether a single pair's streamed ALG1 level runs several iterations per launch (k_cp_tile.cu):
+// Whether a single pair's streamed ALG1 level runs several iterations per launch (k_cp_tile.cuh):
 // the built-in block height (a pinned or autotuned one asks for the one-iteration kernel k_cp).
 bool cp_tile_of(const of_params *p, bool batched) {
     return !batched && p->method == OF_CP && p->rows_per_warp == 0 &&
@@ -319,8 +320,8 @@ bool cp_tile_of(const of_params *p, bool batched) {
 }
 
 // Levels up to this many pixels run ALG1 level-resident when its tile kernel is the alternative
-// (measured per iteration, resident against tile kernel: 1.03 / 1.21 us at 40x30, 1.21 / 1.29 at
-// 80x60, 1.79 / 1.29 at 120x90, 2.41 / 1.32 at 160x120).
+// (measured per iteration, resident against tile kernel: 1.03 / 1.37 us at 40x30, 1.21 / 1.37 at
+// 80x60, 1.79 / 1.37 at 120x90, 2.41 / 1.37 at 160x120).
 constexpr long CP_TILE_RESIDENT_MAX_PX = 6000;
 
 // Levels up to this many pixels run the ADMM methods level-resident when the several-iterations
@@ -883,11 +884,12 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
             }
             const int start2 = (start + kw) & 1;  // where the level's engine picks the state up
             // the streamed pairs' launches: how many iterations each takes.  ADMM and ALG1 by the built-in
-            // strip rule or block height run several per launch (k_admm_tile.cuh, k_cp_tile.cu).
+            // strip rule or block height run several per launch (k_admm_tile.cuh, k_cp_tile.cuh).
             const bool res1 = !batched && use_resident(p, geom_of(*pc[0].pl, l));
             const bool tile = !B.pers[l] && (batched ? B.tp[l].R > 0 : !res1 && admm_tile_of(p));
-            const bool tile2 = tile || (!B.pers[l] && !res1 && cp_tile_of(p, batched));
+            const bool cptile = !B.pers[l] && !res1 && cp_tile_of(p, batched);
             TilePlan tp = B.tp[l];
+            if (cptile) tp = cp_tile_plan(geom_of(*pc[0].pl, l), tile_iters_of(p, rest));
             CUtensorMap maps[2][3];
             if (tile && !batched) {
                 const PairCtx &c = pc[0];
@@ -901,7 +903,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
             std::vector<int> steps;
             for (int it = 0, step = 1; it < rest; it += step) {
                 step = 1;
-                if (tile2) step = tile_step(p, tile ? tp.ni : TILE_ITERS, it, rest);
+                if (tile || cptile) step = tile_step(p, tp.ni, it, rest);
                 steps.push_back(step);
             }
             const int launches = (int)steps.size();
@@ -999,8 +1001,12 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                         else launch_pdr_fused(a, prec, pflow, s);
                     } else if (cp) {
                         if (step > 1) {
-                            launch_cp_tile(a, step, prec, pflow, s);
-                            last_nb = cp_tile_blocks(g);
+                            TileArgs t{};
+                            t.a = a;
+                            tile_set_plan(t, tp, step);
+                            t.vec = 1;
+                            launch_cp_tile(t, prec, pflow, s);
+                            last_nb = admm_tile_blocks(tp);
                         } else {
                             launch_cp(a, prec, pflow, s);
                             last_nb = blocks_of(g, l);
@@ -1020,7 +1026,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                         last_nb = blocks_of(g, l);
                     }
                     if (check) {
-                        const int nb = tile ? admm_tile_blocks(tp) : cp && step > 1 ? cp_tile_blocks(g) : blocks_of(g, l);
+                        const int nb = tile || (cp && step > 1) ? admm_tile_blocks(tp) : blocks_of(g, l);
                         const double rows = (double)g.H * g.W * (has_w ? 3.0 : 2.0);
                         launch_reduce_check(c.partials, nb, &c.misc->res_check, rows, p->tol, &c.misc->done,
                                             &c.misc->iters, 10, s);
@@ -1093,7 +1099,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                     launch_reduce_check_batched(bpart, ps, n, 0.0, 0, 1, s);
                 } else {
                     const Geom g = geom_of(*pc[0].pl, l);
-                    launch_sum(pc[0].partials, tile2 ? last_nb : blocks_of(g, l), &pc[0].misc->res_final, s);
+                    launch_sum(pc[0].partials, tile || cptile ? last_nb : blocks_of(g, l), &pc[0].misc->res_final, s);
                 }
             }
         }

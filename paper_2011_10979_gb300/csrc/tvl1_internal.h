@@ -101,7 +101,7 @@ struct IterArgs {
 constexpr int TILE_WARPS = 12, TILE_SMS = 152, TILE_MAX_ITERS = 8;
 // Rows of the staged form's frames (R is then ignored).
 constexpr int TILE_STAGED_HEIGHT = 48;
-// Iterations per launch where the number is fixed (ALG1's tile kernel too).
+// Iterations per launch where the number is fixed.
 constexpr int TILE_ITERS = 3;
 
 // A level's tiling: ni iterations of halo around tiles of ow x oh pixels whose output starts offx
@@ -307,13 +307,10 @@ void tile_set_plan(TileArgs &t, const TilePlan &p, int ni);
 bool tile_encode_maps(CUtensorMap maps[3], const Fields &f, const void *Ix, const void *Iy, Geom g, int prec,
                       int prec_flow, bool has_w);
 void launch_admm_tile(const TileArgs &a, int prec, int prec_flow, cudaStream_t s);
-// Single pair: ni (2 or 3) consecutive iterations of k_cp in one
-// launch over TT x TT tiles (cp_tile_size: 32, or 16 on small levels), reading a.in and writing
-// a.out, bitwise ni launches of the one-iteration kernel; partials (of the last iteration) in
-// cp_tile_blocks(a.g) slots.
-int cp_tile_size(Geom g);
-int cp_tile_blocks(Geom g);
-void launch_cp_tile(const IterArgs &a, int ni, int prec, int prec_flow, cudaStream_t s);
+// Single pair: a.ni consecutive iterations of k_cp in one launch, reading a.a.in and writing a.a.out,
+// bitwise ni launches of the one-iteration kernel; partials of the last iteration, one slot per tile.
+TilePlan cp_tile_plan(Geom g, int ni);
+void launch_cp_tile(const TileArgs &a, int prec, int prec_flow, cudaStream_t s);
 
 // ---------------------------------------------------------------- adaptive ADMM step (k_adapt.cu)
 // Residual balancing of c after one ADMM iteration prev -> cur (both state buffers intact): the

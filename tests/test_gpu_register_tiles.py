@@ -1,0 +1,61 @@
+"""The tile kernels that keep their frame in registers, at the sizes and data where their tiling, their
+border handling or their shortcuts change: against the one-iteration kernels (a pinned block or strip
+height), whose arithmetic they repeat, so the comparison is for equality."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2011_10979_gb300 import flow, synth  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    c = flow.Context(0)
+    yield c
+    c.close()
+
+
+def cu(a):
+    return torch.from_numpy(np.ascontiguousarray(a, np.float32)).cuda()
+
+
+def images(H, W, kind="plain"):
+    if min(H, W) > 8:
+        p = synth.random_affine_rect_pair(H, W, H + W)
+        I0, I1 = p.I0.copy(), p.I1.copy()
+    else:
+        I0, I1 = np.random.default_rng(H + W).random((2, H, W)).astype(np.float32)
+    if kind == "flat":  # zero residuals and gradients beside textured pixels
+        I0[:, W // 2:] = I1[:, W // 2:] = 0.25
+    elif kind == "faint":  # squared gradients and residuals near and below the smallest normal number
+        I0, I1 = I0 * np.float32(1e-19), I1 * np.float32(1e-19)
+    return cu(I0), cu(I1)
+
+
+def both(ctx, im, pinned, **kw):
+    a = flow.of_solve(ctx, *im, flow.default_params(rows_per_warp=pinned, **kw), want_w=True)
+    b = flow.of_solve(ctx, *im, flow.default_params(rows_per_warp=0, **kw), want_w=True)
+    for x, y in zip(a[:2], b[:2]):
+        assert torch.equal(x, y)
+    if kw.get("beta", 1.0) != 0.0:
+        assert torch.equal(a[2], b[2])
+    assert a[3]["iters_run"] == b[3]["iters_run"]
+
+
+# One frame and its neighbours: 64 columns less the halo (8 to 16), 24, 36 or 48 rows less theirs.
+@pytest.mark.parametrize("H,W", [(1, 1), (2, 300), (300, 2), (35, 49), (36, 50), (47, 65), (130, 171), (391, 590)])
+@pytest.mark.parametrize("iters", [20, 47])
+def test_alg1_tiles_at_their_edges(ctx, H, W, iters):
+    eng = flow.OF_ENGINE_STREAM if H * W < 7000 else flow.OF_ENGINE_FUSED  # (the fused engine's small levels are resident)
+    both(ctx, images(H, W), 8, method=flow.OF_CP, lam=3.0, levels=1, warps=2, iters=iters, engine=eng)
+
+
+@pytest.mark.parametrize("kind", ["flat", "faint"])
+@pytest.mark.parametrize("beta", [0.05, 0.0, 1e-16])
+def test_alg1_quotients_outside_the_usual_range(ctx, kind, beta):
+    both(ctx, images(150, 202, kind), 8, method=flow.OF_CP, lam=3.0, beta=beta, levels=1, warps=2, iters=40,
+         engine=flow.OF_ENGINE_FUSED)
