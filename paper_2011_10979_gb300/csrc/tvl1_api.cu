@@ -320,14 +320,15 @@ bool cp_tile_of(const of_params *p, bool batched) {
 }
 
 // Levels up to this many pixels run ALG1 level-resident when its tile kernel is the alternative
-// (measured per iteration, resident against tile kernel: 1.03 / 1.37 us at 40x30, 1.21 / 1.37 at
-// 80x60, 1.79 / 1.37 at 120x90, 2.41 / 1.37 at 160x120).
-constexpr long CP_TILE_RESIDENT_MAX_PX = 6000;
+// (measured per iteration, resident against tile kernel: 1.03 / 1.09 us at 40x30, 1.14 / 1.09 at 64x48,
+// 1.21 / 1.10 at 80x60, 1.78 / 1.09 at 120x90, 2.39 / 1.12 at 160x120).
+constexpr long CP_TILE_RESIDENT_MAX_PX = 2000;
 
-// Levels up to this many pixels run the ADMM methods level-resident when the several-iterations
-// tile kernel is the alternative (measured per iteration, resident against tile kernel: 1.04 /
-// 1.51 us at 40x30, 1.34 / 1.58 at 80x60, 1.93 / 1.58 at 120x90, 2.67 / 1.61 at 160x120); against
-// the row-streaming kernel the resident launch wins up to 32,000 px.
+// A single pair's level runs the ADMM methods level-resident wherever the register-resident cluster
+// form holds it (k_admm_cluster.cuh; measured per iteration, against the several-iterations tile kernel:
+// 1.03 / 1.36 us at 80x60, 1.13 / 1.36 at 120x90, 1.27 / 1.37 at 155x48, the slowest shape), else up to
+// this many pixels (levels a few rows high or a few columns wide); against the row-streaming kernel
+// the resident launch wins up to 32,000 px.
 constexpr long TILE_RESIDENT_MAX_PX = 7000;
 
 bool use_resident(const of_params *p, Geom g, bool batched = false) {
@@ -335,7 +336,8 @@ bool use_resident(const of_params *p, Geom g, bool batched = false) {
     if (p->engine == OF_ENGINE_RESIDENT) return true;
     if (p->engine != OF_ENGINE_FUSED && p->engine != OF_ENGINE_PERSISTENT) return false;
     if (pdr_tile_of(p)) return (long)g.H * g.W <= PDR_TILE_RESIDENT_MAX_PX;
-    if (admm_tile_of(p) && !batched) return (long)g.H * g.W <= TILE_RESIDENT_MAX_PX;
+    if (admm_tile_of(p) && !batched)
+        return (long)g.H * g.W <= TILE_RESIDENT_MAX_PX || admm_cluster_plan(g, admm_resident_cluster(), nullptr);
     if (cp_tile_of(p, batched)) return (long)g.H * g.W <= CP_TILE_RESIDENT_MAX_PX;
     return admm_resident_preferred(g, p->method);
 }
@@ -937,7 +939,9 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                     r.sc.rows = (double)g.H * g.W * (has_w ? 3.0 : 2.0);
                     r.sc.resident = 1;
                     const int nc = admm_resident_nc(g, p->method);
-                    launch_admm_resident(r, 1, nc, admm_resident_smem(g, p->method, nc), prec, pflow, s);
+                    r.timeout = &c.misc->timeout;
+                    if (!pdr && !cp && admm_cluster_plan(g, nc, &r)) launch_admm_cluster(r, nc, prec, pflow, s);
+                    else launch_admm_resident(r, 1, nc, admm_resident_smem(g, p->method, nc), prec, pflow, s);
                 } else {
                     r.pairs = (const PairIter *)(ctx->arena + B.table_off + B.pairs_off[l][in32 ? 1 : 0]);
                     r.scal = (const PairScalars *)(ctx->arena + B.table_off + B.scal_off[l]);

@@ -154,7 +154,13 @@ struct ResArgs {
     int parity_in = 0, parity_out = 0;
     int iters = 0, check = 0, final_res = 0;
     double tol = 0.0;
+    int gx = 0, ow = 0, oh = 0;  // launch_admm_cluster: columns of tiles, a tile's size
+    int *timeout = nullptr;      // launch_admm_cluster: set when a bounded wait ran out
 };
+// ADMM methods, single pair: the register-resident form for small levels (k_admm_cluster.cuh).  Sets the
+// tiling of a level over a cluster of nc CTAs; false where it does not fit.
+bool admm_cluster_plan(Geom g, int nc, ResArgs *a);
+cudaError_t launch_admm_cluster(const ResArgs &a, int nc, int prec, int prec_flow, cudaStream_t s);
 // Persistent engine of the ADMM methods (k_admm_persist.cuh): one launch per warp of a level runs
 // every inner iteration.  A segment is strip sx (admm_fused_strip_w() output columns) by row band
 // t of m (rows [t H / m, (t + 1) H / m)) of pair `pair`; a pair's segments are numbered

@@ -36,8 +36,9 @@ def images(H, W, kind="plain"):
     return cu(I0), cu(I1)
 
 
-def both(ctx, im, pinned, **kw):
-    a = flow.of_solve(ctx, *im, flow.default_params(rows_per_warp=pinned, **kw), want_w=True)
+def both(ctx, im, pinned, ref_engine=None, **kw):
+    ref = dict(kw, engine=kw["engine"] if ref_engine is None else ref_engine)
+    a = flow.of_solve(ctx, *im, flow.default_params(rows_per_warp=pinned, **ref), want_w=True)
     b = flow.of_solve(ctx, *im, flow.default_params(rows_per_warp=0, **kw), want_w=True)
     for x, y in zip(a[:2], b[:2]):
         assert torch.equal(x, y)
@@ -59,3 +60,25 @@ def test_alg1_tiles_at_their_edges(ctx, H, W, iters):
 def test_alg1_quotients_outside_the_usual_range(ctx, kind, beta):
     both(ctx, images(150, 202, kind), 8, method=flow.OF_CP, lam=3.0, beta=beta, levels=1, warps=2, iters=40,
          engine=flow.OF_ENGINE_FUSED)
+
+
+# Tiles of the cluster engine: one column of up to 64 pixels or several of up to 60, two to twelve rows; the last
+# size does not fit it.  Launches of an odd and an even number of iterations, and fewer than one exchange takes.
+@pytest.mark.parametrize("H,W", [(1, 1), (2, 3), (1, 64), (3, 65), (48, 64), (49, 63), (33, 120), (192, 2), (60, 80),
+                                 (12, 700), (96, 122), (97, 119)])
+@pytest.mark.parametrize("iters", [1, 2, 37])
+@pytest.mark.parametrize("kw", [dict(), dict(method=flow.OF_PADMM_II, rho=1.7), dict(beta=0.0, a_tilde_mode=1),
+                                dict(precision=2, fp32_flow=0)], ids=["I", "II", "per-pixel", "bf16"])
+def test_admm_cluster_engine_at_its_edges(ctx, H, W, iters, kw):
+    P = dict(dict(method=flow.OF_PADMM_I, lam=3.0, levels=1, warps=2, iters=iters, engine=flow.OF_ENGINE_RESIDENT), **kw)
+    both(ctx, images(H, W), 1, flow.OF_ENGINE_STREAM, **P)
+
+
+@pytest.mark.parametrize("H,W", [(30, 40), (60, 80)])
+@pytest.mark.parametrize("iters", [40, 25])
+def test_admm_cluster_engine_stops_where_the_streamed_solve_does(ctx, H, W, iters):
+    im = images(H, W)
+    kw = dict(method=flow.OF_PADMM_I, lam=3.0, levels=1, iters=iters, engine=flow.OF_ENGINE_RESIDENT)
+    tol = flow.of_solve(ctx, *im, flow.default_params(warps=1, **dict(kw, iters=20)))[3]["residual"] * 1.001
+    for t in (tol, 1e-30):
+        both(ctx, im, 1, flow.OF_ENGINE_STREAM, warps=2, tol=t, **kw)
