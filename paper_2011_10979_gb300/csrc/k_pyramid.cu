@@ -297,6 +297,8 @@ template <typename TD, typename TF> __global__ void k_level_begin(const __grid_c
         stT<TF>(to.f[F_W + c], o, x[c]);
         if (A.xbar) stT<TF>(to.f[F_WB + c], o, x[c]);
     }
+    // the iterations leave w alone without beta: zero in whichever buffer they end
+    if (!A.has_w) stT<TF>(P.buf[A.to ^ 1].f[F_W], o, 0.f);
 #pragma unroll
     for (int k = F_P1; k <= F_S; ++k) stT<TD>(to.f[k], o, 0.f);
     const int jl = max(j - 1, 0), jr = min(j + 1, g.W - 1), iu = max(i - 1, 0), id = min(i + 1, g.H - 1);
@@ -306,7 +308,7 @@ template <typename TD, typename TF> __global__ void k_level_begin(const __grid_c
 }
 
 template <typename TD, typename TF>
-__global__ void k_state_to_f32(const __grid_constant__ PairSet A, const __grid_constant__ PairSet B, int cur, int xbar) {
+__global__ void k_state_to_f32(const __grid_constant__ PairSet A, const __grid_constant__ PairSet B, int cur, int xbar, int has_w) {
     const PairIter &P = A.pairs ? A.pairs[blockIdx.z] : A.one, &Q = B.pairs ? B.pairs[blockIdx.z] : B.one;
     const Geom g = P.g;
     const int j = blockIdx.x * B2X + threadIdx.x, i = blockIdx.y * B2Y + threadIdx.y;
@@ -316,6 +318,7 @@ __global__ void k_state_to_f32(const __grid_constant__ PairSet A, const __grid_c
 #pragma unroll
     for (int k = 0; k < NFIELDS; ++k)
         if (xbar || k < F_WB) stT<float>(t.f[k], o, is_flow_field(k) ? ldT<TF>(f.f[k], o) : ldT<TD>(f.f[k], o));
+    if (!has_w) stT<float>(Q.buf[1].f[F_W], o, 0.f);
 }
 
 template <typename TF> __global__ void k_output(Fields f, Geom g, float *u, float *v, float *w) {
@@ -467,10 +470,10 @@ void launch_warp_reset(const PairSet &a, cudaStream_t s) {
     else k_warp_reset<<<(a.n + 127) / 128, 128, 0, s>>>(a);
 }
 
-void launch_state_to_f32(const PairSet &from, const PairSet &to, int cur, int xbar, int prec_dual, int prec_flow,
-                         cudaStream_t s) {
+void launch_state_to_f32(const PairSet &from, const PairSet &to, int cur, int xbar, int has_w, int prec_dual,
+                         int prec_flow, cudaStream_t s) {
     TVL1_DISPATCH_PREC(prec_dual, TD, TVL1_DISPATCH_PREC(prec_flow, TF,
-                       k_state_to_f32<TD, TF><<<grid_of(from), dim3(B2X, B2Y), 0, s>>>(from, to, cur, xbar)));
+                       k_state_to_f32<TD, TF><<<grid_of(from), dim3(B2X, B2Y), 0, s>>>(from, to, cur, xbar, has_w)));
 }
 
 void launch_output(const Fields &f, Geom g, float *u, float *v, float *w, int prec_flow, cudaStream_t s) {

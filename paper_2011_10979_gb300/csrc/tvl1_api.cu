@@ -823,7 +823,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
             const bool last_warp = (l == B.out_level) && (wp == p->warps - 1);
             const bool switch32 = B.pl[0].use32_last && l == 0 && wp == p->warps - 1;
             // precision policy: the finest level's last warp runs with FP32 storage
-            if (switch32) launch_state_to_f32(set_of(l, 0), set_of(l, 1), cur, pdr || cp, cp ? pflow : prec, pflow, s);
+            if (switch32) launch_state_to_f32(set_of(l, 0), set_of(l, 1), cur, pdr || cp, has_w, cp ? pflow : prec, pflow, s);
             if (switch32) {
                 in32 = true;
                 cur = 0;

@@ -234,9 +234,10 @@ void launch_level_begin(const LevelArgs &a, int prec_dual, int prec_flow, cudaSt
 // `prec`; ms_max raised with atomicMax (it and the stop flag behind it are zeroed by launch_warp_reset).
 void launch_warp(const PairSet &a, int cur, float beta, int prec, int prec_flow, cudaStream_t s);
 void launch_warp_reset(const PairSet &a, cudaStream_t s);
-// The state of buffer `cur` of `from` (duals in prec_dual, the rest in prec_flow) as FP32 in buffer 0 of `to`.
-void launch_state_to_f32(const PairSet &from, const PairSet &to, int cur, int xbar, int prec_dual, int prec_flow,
-                         cudaStream_t s);
+// The state of buffer `cur` of `from` (duals in prec_dual, the rest in prec_flow) as FP32 in buffer 0 of `to`;
+// without w, zero in buffer 1's.
+void launch_state_to_f32(const PairSet &from, const PairSet &to, int cur, int xbar, int has_w, int prec_dual,
+                         int prec_flow, cudaStream_t s);
 // u, v, w (prec_flow) as FP32.
 void launch_output(const Fields &f, Geom g, float *u, float *v, float *w, int prec_flow, cudaStream_t s);
 

@@ -329,7 +329,7 @@ cudaError_t step_run(std::vector<StepPair *> &act, const of_params *p, StepTable
             q.in32 = true;
             q.cur = 0;
             q.prec = q.pflow = PREC_F32;
-            launch_state_to_f32(from, set_of(q, 0), cur, pdr || cp, pd, pf, s);
+            launch_state_to_f32(from, set_of(q, 0), cur, pdr || cp, has_w, pd, pf, s);
         }
         (q.in32 && pl.prec != PREC_F32 ? g32 : g16).push_back(qp);
     }

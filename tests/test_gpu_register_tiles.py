@@ -47,6 +47,21 @@ def both(ctx, im, pinned, ref_engine=None, **kw):
     assert a[3]["iters_run"] == b[3]["iters_run"]
 
 
+@pytest.mark.parametrize("method", [flow.OF_PADMM_I, flow.OF_CP, flow.OF_PDR])
+@pytest.mark.parametrize("engine", [flow.OF_ENGINE_FUSED, flow.OF_ENGINE_STREAM, flow.OF_ENGINE_RESIDENT])
+@pytest.mark.parametrize("prec", [0, 2])
+def test_without_beta_w_is_zero_whatever_the_launch_count(ctx, method, engine, prec):
+    """The iterations leave w alone without beta: it is zero in whichever buffer the last launch ends, also
+    where the workspace held another solve's w."""
+    im = images(150, 200)
+    for iters in (11, 12, 13, 14):
+        kw = dict(method=method, engine=engine, precision=prec, lam=3.0, levels=2, warps=2, iters=iters)
+        w = flow.of_solve(ctx, *im, flow.default_params(beta=0.05, **kw), want_w=True)[2]
+        assert w.abs().max() > 0
+        w = flow.of_solve(ctx, *im, flow.default_params(beta=0.0, **kw), want_w=True)[2]
+        assert torch.equal(w, torch.zeros_like(w))
+
+
 # One frame and its neighbours: 64 columns less the halo (8 to 16), 24, 36 or 48 rows less theirs.
 @pytest.mark.parametrize("H,W", [(1, 1), (2, 300), (300, 2), (35, 49), (36, 50), (47, 65), (130, 171), (391, 590)])
 @pytest.mark.parametrize("iters", [20, 47])
