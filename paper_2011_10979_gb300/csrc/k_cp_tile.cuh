@@ -26,7 +26,7 @@
 // Bound by latency and issue with three warps per SM quarter (some 240 clocks per row and warp), beside
 // 4 to 6 us per launch for instruction fetch and the state's loads and stores.  Measured per iteration,
 // and in brackets with the frame in shared memory and scalar instructions, which this replaced:
-// 640x480 2.97 us (4.5), 320x240 1.37 (2.0), 160x120 1.37 (1.32).
+// 640x480 2.83 us (4.51), 320x240 1.30 (1.87), 160x120 1.09 (1.32), 3840x2160 75 (114).
 #pragma once
 #include <math.h>
 
@@ -62,7 +62,7 @@ template <typename T, typename TF, bool HAS_W, int R> struct Kernel {
     static __device__ __forceinline__ void body(const TileArgs &A, SH &G, int bx, int by, int lane, int wid) {
         const int H = A.a.g.H, W = A.a.g.W, P = A.a.g.pitch;
         const int c = bx * A.ow - A.offx + 2 * lane, ib = by * A.oh - A.offy + wid * R;
-        const unsigned me0 = mask_of(c < W - 1), me1 = mask_of(c + 1 < W - 1), mw0 = mask_of(c > 0);
+        const unsigned me0 = mask_of(c >= 0 && c < W - 1), me1 = mask_of(c + 1 >= 0 && c + 1 < W - 1);
         const int rlast = __shfl_sync(FULL, H - 1 - ib, 0), rfirst = __shfl_sync(FULL, -ib, 0);
         pair2 y[R][6], X[R][3], B[R][3];
         const float beta = A.a.k.beta, lam = A.a.k.lambda, sg = A.a.k.cp_sigma, sl0 = sg * lam;
@@ -145,7 +145,7 @@ template <typename T, typename TF, bool HAS_W, int R> struct Kernel {
 #pragma unroll
                     for (int k = C0; k < 3; ++k) g[2 * k + 1] = sub2(B[r + 1 < R ? r + 1 : r][k], B[r][k]);
                 }
-                if (BY && r == rlast) {
+                if (BY && (r < rfirst || r == rlast)) {
                     asm volatile("");
 #pragma unroll
                     for (int k = C0; k < 3; ++k) g[2 * k + 1] = 0ull;
@@ -171,7 +171,8 @@ template <typename T, typename TF, bool HAS_W, int R> struct Kernel {
 #pragma unroll
                 for (int k = C0; k < 3; ++k) G.bot[wid][k][lane] = y[R - 1][2 * k + 1];
             // ---- the primal step, bottom row first (row 0 needs the warp above): Z = X + sigma div y' in
-            // place of Xbar, and rho(Z)
+            // place of Xbar, and rho(Z).  y is zero where its difference crosses the image's border and one pixel
+            // outside on the west and north: it starts at zero and those differences are zero.
             pair2 rho[R];
             unsigned small = ~0u;  // least (2 |rho| - 1) as integers: zero wraps around
 #pragma unroll
@@ -179,21 +180,11 @@ template <typename T, typename TF, bool HAS_W, int R> struct Kernel {
                 if (r == 0) __syncthreads();
 #pragma unroll
                 for (int k = C0; k < 3; ++k) {
-                    pair2 n = r > 0 ? y[r > 0 ? r - 1 : 0][2 * k + 1] : wid > 0 ? G.bot[wid > 0 ? wid - 1 : 0][k][lane] : 0ull;
-                    pair2 ys = y[r][2 * k + 1];
-                    if (BY && r == rlast) {
-                        asm volatile("");
-                        ys = 0ull;
-                    }
-                    if (BY && r == rfirst) {
-                        asm volatile("");
-                        n = 0ull;
-                    }
+                    const pair2 n = r > 0 ? y[r > 0 ? r - 1 : 0][2 * k + 1] : wid > 0 ? G.bot[wid > 0 ? wid - 1 : 0][k][lane] : 0ull;
                     float a, b;
                     upk(y[r][2 * k], a, b);
                     const float wv = __shfl_up_sync(FULL, b, 1);
-                    const pair2 x = pk((BX == 2 ? keep(a, me0) : a) - (BX ? keep(wv, mw0) : wv), (BX ? keep(b, me1) : b) - a);
-                    B[r][k] = fma2(sg2, sub2(add2(x, ys), n), X[r][k]);
+                    B[r][k] = fma2(sg2, sub2(add2(pk(a - wv, b - a), y[r][2 * k + 1]), n), X[r][k]);
                 }
                 pair2 q = G.it[wid * R + r][lane];
                 if (HAS_W) q = fma2(beta2, B[r][0], q);
