@@ -95,8 +95,8 @@ void tile_set_plan(TileArgs &t, const TilePlan &p, int ni) {
     t.staged = p.staged;
 }
 
-bool tile_encode_maps(CUtensorMap maps[3], const Fields &f, const void *Ix, const void *Iy, Geom g, int prec,
-                      int prec_flow, bool has_w) {
+bool tile_encode_maps(CUtensorMap *maps, const Fields &f, const void *Ix, const void *Iy, Geom g, int prec,
+                      int prec_flow, bool has_w, bool pdr) {
     static const PFN_cuTensorMapEncodeTiled_v12000 enc = [] {
         void *fn = nullptr;
         cudaDriverEntryPointQueryResult q;
@@ -121,7 +121,8 @@ bool tile_encode_maps(CUtensorMap maps[3], const Fields &f, const void *Ix, cons
     };
     const size_t ps = (size_t)((const char *)f.f[1] - (const char *)f.f[0]), pd = (size_t)((const char *)Iy - (const char *)Ix);
     return one(&maps[0], f.f[has_w ? F_W : F_U], ps, has_w ? 3 : 2, prec_flow) &&
-           one(&maps[1], f.f[has_w ? F_P1 : F_Q11], ps, has_w ? 7 : 5, prec) && one(&maps[2], Ix, pd, 3, prec);
+           one(&maps[1], f.f[has_w ? F_P1 : F_Q11], ps, (has_w ? 7 : 5) - pdr, prec) && one(&maps[2], Ix, pd, 3, prec) &&
+           (!pdr || one(&maps[3], f.f[has_w ? F_WB : F_UB], ps, has_w ? 3 : 2, prec_flow));
 }
 
 void launch_admm_tile(const TileArgs &a, int prec, int prec_flow, cudaStream_t s) {

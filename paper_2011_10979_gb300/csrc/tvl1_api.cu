@@ -72,6 +72,7 @@ Plan make_plan(int H, int W, const of_params *p) {
                        adapt_blocks(g), pdr_tile_blocks(g)});
         for (int q = 0; q < 4; ++q) mb = std::max(mb, admm_tile_blocks(admm_tile_plan(g, q & 1 ? TILE_ITERS : 0, q & 2)));
         for (int q = 0; q < 2; ++q) mb = std::max(mb, admm_tile_blocks(cp_tile_plan(g, q ? TILE_ITERS : 0)));
+        mb = std::max(mb, admm_tile_blocks(pdr_regtile_plan(g, std::max(p->iters, 1))));
     }
     pl.max_blocks = mb;
     pl.partials = take(3 * (size_t)mb * sizeof(double));
@@ -298,6 +299,30 @@ struct Batch {
 bool pdr_tile_of(const of_params *p) {
     return p->method == OF_PDR && p->engine != OF_ENGINE_PLAIN && p->gs_sweeps == 1;
 }
+
+// Iterations of each launch of the pDR register tile kernel for `iters` iterations, at most ni per launch:
+// launches whose residual is read take one iteration (every tenth with the stopping test, the last of
+// the level), and with the test every ten iterations are an even number of launches, which leaves
+// the tested state in the buffer that the warp started from.
+std::vector<int> pdr_launches(int ni, int iters, bool tested, bool last_warp) {
+    std::vector<int> v;
+    for (int it = 0; it < iters;) {
+        const int n = tested ? std::min(10, iters - it) : iters - it;
+        const bool read = (tested && n == 10) || (last_warp && it + n == iters);
+        const int m = n - read;
+        int q = (m + ni - 1) / ni;
+        if (tested && n == 10 && (q + 1) % 2) ++q;
+        for (int k = 0; k < q; ++k) v.push_back(m / q + (k < m % q));
+        if (read) v.push_back(1);
+        it += n;
+    }
+    return v;
+}
+
+// Levels from this many pixels run a single pair's pDR on the register tile kernel (k_pdr_regtile.cuh), smaller
+// ones on the one-iteration tile kernel of k_pdr.cu (measured per iteration, register tiles against it: 4.5 / 4.4
+// us at 213x160, 4.2 / 5.6 at 240x180, 4.3 / 5.8 at 320x240).
+constexpr long PDR_REGTILE_MIN_PX = 40000;
 
 // Levels up to this many pixels run pDR level-resident when its one-launch tile kernel is the
 // alternative (measured per iteration, resident against tile kernel: 2.3 / 4.0 us at 40x30,
@@ -892,7 +917,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
             const bool cptile = !B.pers[l] && !res1 && cp_tile_of(p, batched);
             TilePlan tp = B.tp[l];
             if (cptile) tp = cp_tile_plan(geom_of(*pc[0].pl, l), tile_iters_of(p, rest));
-            CUtensorMap maps[2][3];
+            CUtensorMap maps[2][4];
             if (tile && !batched) {
                 const PairCtx &c = pc[0];
                 const Geom g = geom_of(*c.pl, l);
@@ -902,8 +927,18 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                     ok = ok && tile_encode_maps(maps[b], bufs_of(c)[b], data_of(c)[0], data_of(c)[1], g, prec, pflow, has_w);
                 if (!ok) tp = admm_tile_plan(g, tile_iters_of(p, rest), true);
             }
+            // a single pair's streamed pDR level (k_pdr_regtile.cuh), where the driver encodes its maps
+            bool pdrreg = pdr_tile && !batched && !res1 && rest > 0 && (long)pc[0].pl->H[l] * pc[0].pl->W[l] >= PDR_REGTILE_MIN_PX;
+            if (pdrreg) {
+                const PairCtx &c = pc[0];
+                const Geom g = geom_of(*c.pl, l);
+                tp = pdr_regtile_plan(g, rest);
+                for (int b = 0; b < 2; ++b)
+                    pdrreg = pdrreg && tile_encode_maps(maps[b], bufs_of(c)[b], data_of(c)[0], data_of(c)[1], g, prec, pflow, has_w, true);
+            }
             std::vector<int> steps;
-            for (int it = 0, step = 1; it < rest; it += step) {
+            if (pdrreg) steps = pdr_launches(tp.ni, rest, p->tol > 0.0, last_warp);
+            for (int it = 0, step = 1; !pdrreg && it < rest; it += step) {
                 step = 1;
                 if (tile || cptile) step = tile_step(p, tp.ni, it, rest);
                 steps.push_back(step);
@@ -1001,8 +1036,19 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                     a.tile_h = B.tile_h[l];
                     a.pdr_tile = pdr_tile;
                     if (pdr) {
-                        if (plain) launch_pdr_plain(a, s);
-                        else launch_pdr_fused(a, prec, pflow, s);
+                        if (pdrreg) {
+                            TileArgs t{};
+                            t.a = a;
+                            tile_set_plan(t, tp, step);
+                            t.timeout = &c.misc->timeout;
+                            memcpy(t.maps, maps[par], sizeof(t.maps));
+                            launch_pdr_regtile(t, prec, pflow, s);
+                            last_nb = admm_tile_blocks(tp);
+                        } else if (plain) {
+                            launch_pdr_plain(a, s);
+                        } else {
+                            launch_pdr_fused(a, prec, pflow, s);
+                        }
                     } else if (cp) {
                         if (step > 1) {
                             TileArgs t{};
@@ -1021,7 +1067,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                         tile_set_plan(t, tp, step);
                         t.vec = 1;
                         t.timeout = &c.misc->timeout;
-                        if (tp.staged) memcpy(t.maps, maps[par], sizeof(t.maps));
+                        if (tp.staged) memcpy(t.maps, maps[par], 3 * sizeof(CUtensorMap));
                         launch_admm_tile(t, prec, pflow, s);
                         last_nb = admm_tile_blocks(tp);
                     } else {
@@ -1030,7 +1076,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                         last_nb = blocks_of(g, l);
                     }
                     if (check) {
-                        const int nb = tile || (cp && step > 1) ? admm_tile_blocks(tp) : blocks_of(g, l);
+                        const int nb = tile || pdrreg || (cp && step > 1) ? admm_tile_blocks(tp) : blocks_of(g, l);
                         const double rows = (double)g.H * g.W * (has_w ? 3.0 : 2.0);
                         launch_reduce_check(c.partials, nb, &c.misc->res_check, rows, p->tol, &c.misc->done,
                                             &c.misc->iters, 10, s);
@@ -1103,7 +1149,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                     launch_reduce_check_batched(bpart, ps, n, 0.0, 0, 1, s);
                 } else {
                     const Geom g = geom_of(*pc[0].pl, l);
-                    launch_sum(pc[0].partials, tile || cptile ? last_nb : blocks_of(g, l), &pc[0].misc->res_final, s);
+                    launch_sum(pc[0].partials, tile || cptile || pdrreg ? last_nb : blocks_of(g, l), &pc[0].misc->res_final, s);
                 }
             }
         }

@@ -120,7 +120,7 @@ struct TileArgs {
     int staged;
     int vec;              // every plane's rows start on an 8-byte boundary
     int *timeout;         // set when a bounded wait ran out
-    CUtensorMap maps[3];  // staged form, single pair: flow, dual and data planes
+    CUtensorMap maps[4];  // staged form, single pair: flow, dual and data planes, Xbar (pDR)
 };
 
 // Geometry of the fused ADMM engine: each warp owns a strip of admm_fused_strip_w() output
@@ -310,14 +310,20 @@ inline int tile_cols(const TilePlan &p, Geom g) { return (g.W + p.ow - 1) / p.ow
 inline int tile_rows(const TilePlan &p, Geom g) { return (g.H + p.oh - 1) / p.oh; }
 void tile_set_plan(TileArgs &t, const TilePlan &p, int ni);
 // The staged form's tensor maps of a state buffer (its planes equally spaced) and the data planes;
-// false when the driver cannot encode them.
-bool tile_encode_maps(CUtensorMap maps[3], const Fields &f, const void *Ix, const void *Iy, Geom g, int prec,
-                      int prec_flow, bool has_w);
+// pdr: without s and with a fourth map, of Xbar.  False when the driver cannot encode them.
+bool tile_encode_maps(CUtensorMap *maps, const Fields &f, const void *Ix, const void *Iy, Geom g, int prec,
+                      int prec_flow, bool has_w, bool pdr = false);
 void launch_admm_tile(const TileArgs &a, int prec, int prec_flow, cudaStream_t s);
 // Single pair: a.ni consecutive iterations of k_cp in one launch, reading a.a.in and writing a.a.out,
 // bitwise ni launches of the one-iteration kernel; partials of the last iteration, one slot per tile.
 TilePlan cp_tile_plan(Geom g, int ni);
 void launch_cp_tile(const TileArgs &a, int prec, int prec_flow, cudaStream_t s);
+
+// Single pair, gs_sweeps = 1: a.ni consecutive iterations of pDR in one launch, reading a.a.in through
+// a.maps and writing a.a.out, bitwise ni launches of the one-launch kernel of k_pdr.cu; partials only
+// with one iteration, one slot per tile.
+TilePlan pdr_regtile_plan(Geom g, int max_ni);
+void launch_pdr_regtile(const TileArgs &a, int prec, int prec_flow, cudaStream_t s);
 
 // ---------------------------------------------------------------- adaptive ADMM step (k_adapt.cu)
 // Residual balancing of c after one ADMM iteration prev -> cur (both state buffers intact): the

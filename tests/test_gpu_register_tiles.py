@@ -97,3 +97,29 @@ def test_admm_cluster_engine_stops_where_the_streamed_solve_does(ctx, H, W, iter
     tol = flow.of_solve(ctx, *im, flow.default_params(warps=1, **dict(kw, iters=20)))[3]["residual"] * 1.001
     for t in (tol, 1e-30):
         both(ctx, im, 1, flow.OF_ENGINE_STREAM, warps=2, tol=t, **kw)
+
+
+# pDR's register tiles (levels from 40,000 pixels) against the tile kernel that batches run: frames of 64 x 48 less a
+# halo of 7 to 31 pixels, odd sizes, strips narrower and lower than a frame, one launch of every length.
+@pytest.mark.parametrize("H,W", [(200, 201), (201, 200), (127, 641), (41, 1000), (1000, 41), (7, 5801), (5801, 7), (480, 640)])
+@pytest.mark.parametrize("kw", [dict(), dict(beta=0.0), dict(precision=2, fp32_flow=1), dict(precision=1, fp32_flow=0),
+                                dict(tol=1e-30)], ids=["f32", "beta0", "bf16", "f16", "tested"])
+def test_pdr_register_tiles_equal_the_batched_tile_kernel(ctx, H, W, kw):
+    im = images(H, W)
+    for iters in (1, 13, 20):
+        P = flow.default_params(method=flow.OF_PDR, lam=3.0, levels=1, warps=2, iters=iters, engine=flow.OF_ENGINE_STREAM, **kw)
+        u, v, _, st = flow.of_solve(ctx, *im, P)
+        ub, vb, sb = flow.of_solve_batch(ctx, [im[0]] * 2, [im[1]] * 2, P)
+        assert torch.equal(u, ub[0]) and torch.equal(v, vb[0])
+        assert st["iters_run"] == sb[0]["iters_run"]
+        assert st["residual"] == pytest.approx(sb[0]["residual"], rel=1e-5, abs=1e-12)
+
+
+@pytest.mark.parametrize("kind", ["flat", "faint"])
+@pytest.mark.parametrize("beta", [0.05, 0.0, 1e-16])
+def test_pdr_quotients_outside_the_usual_range(ctx, kind, beta):
+    im = images(202, 206, kind)
+    P = flow.default_params(method=flow.OF_PDR, lam=3.0, beta=beta, levels=1, warps=2, iters=30, engine=flow.OF_ENGINE_STREAM)
+    u, v, _, _ = flow.of_solve(ctx, *im, P)
+    ub, vb, _ = flow.of_solve_batch(ctx, [im[0]] * 2, [im[1]] * 2, P)
+    assert torch.equal(u, ub[0]) and torch.equal(v, vb[0])
