@@ -21,8 +21,9 @@
 // takes some 20 bytes per clock and CTA).  A cluster barrier in place of the mbarriers waits for the
 // stores' completion: 0.82 us per iteration at 64x48 against 0.73.  Measured per iteration, in brackets
 // the engine that keeps the level in shared memory with two cluster barriers per iteration
-// (k_resident.cu), which this replaced: 40x30 0.64 us (1.04), 64x48 0.73 (1.06), 80x60 1.03 (1.34),
-// 128x55 1.18 (1.58 on the tile kernel), 120x90 1.13 (1.36 on it).
+// (k_resident.cu), which this replaced: 40x30 0.63 us (1.04), 64x48 0.72 (1.06), 80x60 1.02 (1.34),
+// 128x55 1.11 (1.58 on the tile kernel), 120x90 1.12 (1.36 on it).  Sending the duals before the rest,
+// as soon as they are final, was slower (1.18 at 80x60).
 // The per-pixel arithmetic is that of the row-streaming kernel (k_admm_math.cuh) in the same order,
 // rounded to the storage types where its stores round, so the results are bitwise the same.
 #pragma once
@@ -367,12 +368,14 @@ template <typename T, typename TF, bool HAS_W, bool II, int R> __device__ __forc
             const bool to_n = by > 0 && q0 + r < HALO, to_s = (by + 1) * oh < H && q0 + r >= oh - HALO;
             if (to_n) send(par, r, -1, 0);
             if (to_s) send(par, r, 1, 0);
-            if (to_w) {
-                send(par, r, 0, -1);
-                if (to_n) send(par, r, -1, -1);
-                if (to_s) send(par, r, 1, -1);
+            // west and east columns at once: they are different lanes but in tiles two pixels wide
+            if (to_w || to_e) {
+                const int dh = to_w ? -1 : 1;
+                send(par, r, 0, dh);
+                if (to_n) send(par, r, -1, dh);
+                if (to_s) send(par, r, 1, dh);
             }
-            if (to_e) {
+            if (to_w && to_e) {
                 send(par, r, 0, 1);
                 if (to_n) send(par, r, -1, 1);
                 if (to_s) send(par, r, 1, 1);

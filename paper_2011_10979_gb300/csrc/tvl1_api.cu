@@ -351,7 +351,7 @@ constexpr long CP_TILE_RESIDENT_MAX_PX = 2000;
 
 // A single pair's level runs the ADMM methods level-resident wherever the register-resident cluster
 // form holds it (k_admm_cluster.cuh; measured per iteration, against the several-iterations tile kernel:
-// 1.03 / 1.36 us at 80x60, 1.13 / 1.36 at 120x90, 1.27 / 1.37 at 155x48, the slowest shape), else up to
+// 1.02 / 1.36 us at 80x60, 1.12 / 1.36 at 120x90, 1.15 / 1.37 at 155x48, the slowest shape), else up to
 // this many pixels (levels a few rows high or a few columns wide); against the row-streaming kernel
 // the resident launch wins up to 32,000 px.
 constexpr long TILE_RESIDENT_MAX_PX = 7000;
