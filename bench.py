@@ -582,17 +582,17 @@ def serving_measure(flow, torch, dev, rate_hz=50.0, duration_s=15.0, drain_s=5.0
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the pADMM kernel that runs the
-# 640 x 480 level of the bench solve (ncu, cold cache): k_admm_tile2, three iterations per launch,
-# 16.00 MB read (the 13 input planes once), 0 written (the written planes stay in L2).  Set to None
+# 640 x 480 level of the bench solve (ncu, cold cache): k_admm_tile, three iterations per launch,
+# 16.07 MB read (the 13 input planes once), 0 written (the written planes stay in L2).  Set to None
 # whenever that kernel changes, until it is captured again.
-TILE2_640_DRAM_BYTES = 16.00e6
+TILE_640_DRAM_BYTES = 16.07e6
 ITERS_PER_LAUNCH = 3
 
 
 def kernel_roofline(flow, torch, dev, pr, reps=20):
     """Per-launch time of the pADMM kernel on the 640 x 480 level where it runs: inside the solve's
-    CUDA graph.  With the bench's fixed schedule that level runs three inner iterations per launch
-    (k_admm_tile2).  Two graph-launched single-level solves of the bench pair, with 220 and 20 inner
+    CUDA graph.  On the streaming engine that level runs three inner iterations per launch
+    (k_admm_tile).  Two graph-launched single-level solves of the bench pair, with 220 and 20 inner
     iterations, are timed with CUDA events on their stream; the difference / 200 is one iteration
     (with its share of graph launch gaps), three of them one launch.  Algorithmic traffic: 13
     planes read + 10 written, FP32 = 92 B per pixel-iteration, 276 B per pixel and launch."""
@@ -628,14 +628,18 @@ def kernel_roofline(flow, torch, dev, pr, reps=20):
     # the level's working set stays in L2: its bandwidth for a working set of the same size
     # (half read, half written, streamed 400 times in one launch)
     l2 = flow.of_l2_bandwidth(int(bytes_per_launch / ITERS_PER_LAUNCH), 400)
-    return {"kernel": "k_admm_tile2<float,float,1,0,32> (640x480 level, three iterations per launch)",
+    return {"kernel": "k_admm_tile<float,float,1,0,12,4,DIRECT> (640x480 level, three iterations per launch)",
             "bound": "hbm", "achieved": achieved,
             "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_source": src,
-            "traffic": TILE2_640_DRAM_BYTES, "us_per_launch": per * 1e6,
+            "traffic": TILE_640_DRAM_BYTES, "us_per_launch": per * 1e6,
             "us_per_iteration": per * 1e6 / ITERS_PER_LAUNCH, "algorithmic_bytes_per_launch": bytes_per_launch,
             "timing": "graph-launched single-level solves, (t(220 iters) - t(20 iters)) / 200 x 3 per launch",
             "l2_peak": l2, "frac_of_l2": achieved / l2,
-            "note": "the 640x480 level's 28 MB state stays in the 129 MB L2 between iterations; l2_peak is the "
+            "state_bytes_per_launch": bytes_per_launch / ITERS_PER_LAUNCH,
+            "frac_of_state_bytes": achieved / ITERS_PER_LAUNCH / peak,
+            "note": "frac counts every iteration's algorithmic bytes, of which a launch of three iterations moves one "
+                    "iteration's (frac_of_state_bytes), the rest staying in registers; "
+                    "the 640x480 level's 28 MB state stays in the 129 MB L2 between iterations; l2_peak is the "
                     "library's L2 streaming probe over a 28 MB read+write working set"}
 
 

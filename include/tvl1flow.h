@@ -272,7 +272,7 @@ of_status of_upsample(const float *coarse, int Hc, int Wc, int pc, float *fine, 
 of_status of_derivatives(const float *I, int H, int W, int pitch, float *Ix, float *Iy, void *stream);
 
 /* Warping and linearisation around d0 = (u0, v0): Ix, Iy = I1x, I1y sampled bilinearly at
- * (x + u0, y + v0) clamped to the image, It = I1(x + d0) - I0 - Ix u0 - Iy v0, computed in FP64
+ * (x + u0, y + v0) clamped to the image, It = I1(x + d0) - I0 - Ix u0 - Iy v0, computed to FP64's results
  * and rounded once to the stored type (Sec. 1: rho(d) = grad I^T d + I_t; reading: its
  * linearisation around d0 inside Sec. 4's coarse-to-fine warping, bilinear sampling).  ms_max: device
  * pointer to one float that receives max(beta^2 + Ix^2 + Iy^2) (it must hold 0 or a smaller

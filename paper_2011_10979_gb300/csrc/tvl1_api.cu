@@ -748,7 +748,7 @@ of_status upload_tables(of_ctx *ctx, const Batch &B, const of_params *p) {
 
 // Enqueues the whole schedule of every pair of the batch on `s` (arena pointers only: graph-
 // capturable).  Per pair: pyramid, level transfer, derivatives, warping, reductions.  The inner
-// iterations of all pairs go in one launch per iteration (a single pair: its own grid).
+// iterations of all pairs share their launches (a single pair: its own grid).
 void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t s) {
     const int n = B.n;
     const bool batched = n > 1;
@@ -1008,7 +1008,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                 a.tol = p->tol;
                 launch_admm_persist(a, prec, pflow, s);
             }
-            // pairs left for one launch per iteration: the tile work-list (ADMM), all pairs (pDR),
+            // pairs left for the streamed launches: the tile work-list (ADMM), all pairs (pDR),
             // the non-resident pairs (ALG1)
             const bool streamed = !persl && (batched ? ((cp || pdr) ? B.nres[l] < n : B.ntiles[l] > 0) : !res1);
             int par = start2, last_nb = 0;  // the buffer parity and the last launch's block count
