@@ -123,3 +123,35 @@ def test_pdr_quotients_outside_the_usual_range(ctx, kind, beta):
     u, v, _, _ = flow.of_solve(ctx, *im, P)
     ub, vb, _ = flow.of_solve_batch(ctx, [im[0]] * 2, [im[1]] * 2, P)
     assert torch.equal(u, ub[0]) and torch.equal(v, vb[0])
+
+
+def np64(t):
+    return t.cpu().double().numpy()
+
+
+# The one-launch pyramid step at tile edges (32 x 16 coarse pixels) and, for the smallest ratio, the three kernels it
+# falls back to where its tile does not fit: the bar of the operator's parity test.
+@pytest.mark.parametrize("H,W", [(2, 2), (63, 33), (65, 131), (128, 64)])
+@pytest.mark.parametrize("eta", [0.5, 0.8, 0.2])
+def test_pyramid_step_on_either_route(orc, H, W, eta):
+    img = np.random.default_rng(H + W).random((H, W)).astype(np.float32)
+    Hc, Wc = orc.level_size(H, eta), orc.level_size(W, eta)
+    got = np64(flow.of_pyr_down(cu(img), Hc, Wc, eta))
+    assert np.max(np.abs(got - orc.downsample(img.astype(np.float64), Hc, Wc, eta))) < 2e-5
+
+
+# Twofold FP32 with the rounding test: FP64's results rounded once.  The oracle forms the same terms in FP64 in its own
+# order, each below 16, so a value may differ where 2^-48 of that crosses a rounding boundary: one FP32 unit at most.
+@pytest.mark.parametrize("flow_kind", ["fractions", "integers", "zero", "far outside"])
+@pytest.mark.parametrize("H,W", [(1, 1), (1, 33), (9, 32), (45, 61)])
+def test_warp_gives_the_fp64_results(orc, H, W, flow_kind):
+    rng = np.random.default_rng(H * W)
+    I0, I1 = rng.random((2, H, W)).astype(np.float32)
+    u0, v0 = {"fractions": rng.uniform(-5, 5, (2, H, W)), "integers": rng.integers(-4, 5, (2, H, W)),
+              "zero": np.zeros((2, H, W)), "far outside": rng.uniform(-5, 5, (2, H, W)) + 3 * max(H, W)}[flow_kind].astype(np.float32)
+    gx, gy = flow.of_derivatives(cu(I1))
+    Ix, Iy, It, _ = flow.of_warp_linearise(cu(I0), cu(I1), gx, gy, cu(u0), cu(v0), 0.05)
+    ref = orc.warp_linearise(I0, I1, np64(gx), np64(gy), u0, v0, 0.05)
+    scale = max(1.0, float(np.abs(u0).max() + np.abs(v0).max()))
+    for a, b in zip((Ix, Iy, It), ref):
+        assert np.all(np.abs(np64(a) - b) <= np.spacing(np.abs(b).astype(np.float32)) + scale * 2.0 ** -48)
