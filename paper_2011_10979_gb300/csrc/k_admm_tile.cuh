@@ -115,6 +115,11 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// Makes a tensor map in global memory, which the host wrote before the launch, visible to this thread's
+// copies: without it they may use what an earlier launch's map at the same address left in a cache.
+__device__ __forceinline__ void map_acquire(const CUtensorMap *map) {
+    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
+}
 __device__ __forceinline__ void tma_load(void *dst, const CUtensorMap *map, int x, int y, unsigned long long *b) {
     asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
                  ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(0), "r"(smem_u32(b))
@@ -172,6 +177,9 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
         const CUtensorMap *maps =
             MODE == BATCHED ? reinterpret_cast<const CUtensorMap *>(G.pi[n % 3].maps) + 3 * A.a.parity : A.maps;
         const int x = D.bx * A.ow - A.offx, y = D.by * A.oh - A.offy;
+        // (a single pair's maps are parameters of the kernel, which need no fence)
+        if (MODE == BATCHED && (n == 0 || G.tr[n & 3].x != G.tr[(n - 1) & 3].x))
+            for (int k = 0; k < 3; ++k) map_acquire(maps + k);
         mbar_expect(&G.full, ST::FH * (NF * ST::WTF * (int)sizeof(TF) + (ND + 3) * ST::WT * (int)sizeof(T)));
         tma_load(stage + ST::flow, maps, sizeof(TF) == 4 ? x : x & ~7, y, &G.full);
         tma_load(stage + ST::dual, maps + 1, sizeof(T) == 4 ? x : x & ~7, y, &G.full);

@@ -1,0 +1,61 @@
+"""The batched tile kernel reads its tensor maps from tables in device memory that the next batch layout, or the
+serving loop's next step, overwrites at the same addresses: whatever the order of layouts and mixes, every flow
+equals its pair's own solve bit for bit."""
+import time
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2011_10979_gb300 import flow, synth  # noqa: E402
+
+SIZES = [(200, 300), (97, 131), (301, 201), (180, 260), (240, 320), (333, 203), (150, 410)]
+
+
+@pytest.fixture(scope="module")
+def pairs():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return [synth.random_affine_rect_pair(H, W, 50 + k) for k, (H, W) in enumerate(SIZES)]
+
+
+def solo(ctx, pairs, P):
+    return [flow.of_solve_host(ctx, p.I0, p.I1, P)[:2] for p in pairs]
+
+
+@pytest.mark.parametrize("prec", [flow.OF_PREC_FP32, flow.OF_PREC_BF16])
+def test_alternating_batch_layouts(pairs, prec):
+    P = flow.default_params(lam=3.0, levels=2, warps=2, iters=20, precision=prec, engine=flow.OF_ENGINE_STREAM)
+    ctx = flow.Context(0)
+    ref = solo(ctx, pairs, P)
+    dev = [(torch.from_numpy(p.I0).cuda(), torch.from_numpy(p.I1).cuda()) for p in pairs]
+    layouts = [[0, 1, 2], [3, 4, 5], [6, 5], [2, 1, 0], [5, 4, 3, 6, 0]]
+    for order in layouts * 3:
+        us, vs, _ = flow.of_solve_batch(ctx, [dev[k][0] for k in order], [dev[k][1] for k in order], P, stats=False)
+        for k, u, v in zip(order, us, vs):
+            assert np.array_equal(u.cpu().numpy(), ref[k][0]) and np.array_equal(v.cpu().numpy(), ref[k][1])
+    ctx.close()
+
+
+@pytest.mark.parametrize("prec", [flow.OF_PREC_FP32, flow.OF_PREC_BF16])
+def test_alternating_request_mixes(pairs, prec):
+    P = flow.default_params(lam=3.0, levels=3, warps=2, iters=20, precision=prec)
+    ctx = flow.Context(0)
+    ref = solo(ctx, pairs, P)
+    flow.of_server_start(ctx, P, 0, 4)
+    try:
+        for order in [[0, 1, 2, 3], [4, 5], [6, 2, 1], [3, 5, 4, 0, 6, 1]] * 3:
+            ids = [flow.of_server_submit(ctx, pairs[k].I0, pairs[k].I1) for k in order]
+            t0 = time.time()
+            for rid, k in zip(ids, order):
+                r = None
+                while r is None:
+                    r = flow.of_server_poll(ctx, rid, SIZES[k])
+                    assert time.time() - t0 < 120
+                    time.sleep(0.001)
+                assert np.array_equal(r[0], ref[k][0]) and np.array_equal(r[1], ref[k][1])
+    finally:
+        flow.of_server_stop(ctx)
+        ctx.close()
