@@ -30,6 +30,7 @@
 #include <cooperative_groups.h>
 
 #include "k_admm_math.cuh"
+#include "k_mbar.cuh"
 #include "k_pack2.cuh"
 
 namespace tvl1 {
@@ -48,9 +49,9 @@ struct Shared {
     unsigned long long full[2];      // the mbarrier an inbox completes on
     unsigned expect;                 // bytes an inbox receives
     int leader;                      // the first warp that waits for them
+    int dead;                        // set when a wait of this CTA ran out
 };
 
-__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ unsigned remote(unsigned p, int rank) {
     unsigned a;
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(p), "r"(rank));
@@ -61,20 +62,6 @@ __device__ __forceinline__ void st_remote(unsigned a, pair2 v, pair2 w, unsigned
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(a), "l"(v), "l"(w), "r"(bar)
                  : "memory");
 }
-// Waits for the phase of parity `ph`; gives up (false) after a bounded number of attempts.
-__device__ __forceinline__ bool wait_inbox(unsigned bar, unsigned ph) {
-    for (int n = 0; n < (1 << 22); ++n) {
-        unsigned ok;
-        asm volatile(
-            "{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-            : "=r"(ok)
-            : "r"(bar), "r"(ph)
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-
 template <typename T, typename TF, bool HAS_W, bool II, int R> __device__ __forceinline__ void run(const ResArgs &A) {
     constexpr int C0 = HAS_W ? 0 : 1;
     constexpr unsigned PIXEL = 16 * (HAS_W ? NQ : NQ - 2), SOUTH = 16 * (HAS_W ? 4 : 3);  // bytes sent of a pixel pair
@@ -153,8 +140,9 @@ template <typename T, typename TF, bool HAS_W, bool II, int R> __device__ __forc
     if (threadIdx.x == 0) {
         G.expect = 0;
         G.leader = MAXWARPS;
-        for (int b = 0; b < 2; ++b) asm volatile("mbarrier.init.shared.b64 [%0], 1;" ::"r"(smem_addr(&G.full[b])) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        G.dead = 0;
+        for (int b = 0; b < 2; ++b) mbar_init(&G.full[b], 1);
+        mbar_init_fence();
     }
     cl.sync();
     bool halo = false;  // whether the warp waits for its neighbours' pixels
@@ -349,8 +337,8 @@ template <typename T, typename TF, bool HAS_W, bool II, int R> __device__ __forc
     const bool to_w = bx > 0 && lane < l0 + HALO / 2, to_e = bx + 1 < gx && lane >= l1 - HALO / 2;
     auto send = [&](int par, int r, int dv, int dh) {
         const int to = rank + dv * gx + dh;
-        const unsigned a = remote(smem_addr(&G.inbox[par][wid * R + r - dv * oh][0][lane - dh * (ow / 2)]), to);
-        const unsigned b = remote(smem_addr(&G.full[par]), to);
+        const unsigned a = remote(smem_u32(&G.inbox[par][wid * R + r - dv * oh][0][lane - dh * (ow / 2)]), to);
+        const unsigned b = remote(smem_u32(&G.full[par]), to);
         if (dv >= 0 || q0 + r < HALO - 1) {  // the frame's last row gives its south differences only
             if (HAS_W) st_remote(a, y[r][0], y[r][1], b);
             st_remote(a + 512, y[r][2], y[r][3], b);
@@ -409,6 +397,7 @@ template <typename T, typename TF, bool HAS_W, bool II, int R> __device__ __forc
     bool have_tot = false, dead = false;
     double tot = 0.0;
     while (run < A.iters) {
+        const bool quit = *(volatile int *)&G.dead != 0;
         const int n = min(HALO, A.iters - run);
         const bool check = A.check && (run + n) % 10 == 0, fin = A.final_res && run + n == A.iters;
         for (int k = 1; k <= n; ++k) iteration(k == n && (check || fin));
@@ -438,15 +427,20 @@ template <typename T, typename TF, bool HAS_W, bool II, int R> __device__ __forc
         if (run >= A.iters) break;
         // the leader has waited for this inbox's last phase, so the arrival counts for the next (a warp without
         // halo may be iterations ahead)
-        if (leader && !dead)
-            asm volatile("mbarrier.arrive.expect_tx.shared.b64 _, [%0], %1;" ::"r"(smem_addr(&G.full[par])), "r"(G.expect) : "memory");
-        push(par);
-        if (halo) {
-            if (!dead && !wait_inbox(smem_addr(&G.full[par]), ph)) {
-                dead = true;  // go on without waiting: the result is reported as a timeout
+        // After a wait that ran out, the CTA goes on without sending or waiting (its neighbours' waits then run
+        // out too), and the result is reported as a timeout.
+        dead |= __any_sync(FULL, quit);
+        if (leader && !dead) mbar_expect(&G.full[par], G.expect);
+        if (!dead && rank != A.withhold) push(par);
+        if (halo && !dead) {
+            const bool here = mbar_wait<true>(&G.full[par], ph, A.wait_ns, A.timeout);
+            if (__all_sync(FULL, here)) {
+                pull(par);
+            } else {
+                dead = true;
+                G.dead = 1;
                 if (lane == 0 && A.timeout) *A.timeout = 1;
             }
-            pull(par);
         }
         __syncwarp();
         par ^= 1;

@@ -41,6 +41,7 @@
 #include <type_traits>
 
 #include "k_admm_math.cuh"
+#include "k_mbar.cuh"
 #include "k_pack2.cuh"
 
 namespace tvl1 {
@@ -89,28 +90,6 @@ template <typename T, typename TF, int FH_> struct Stage {
                          bytes = data + up(3 * FH * WT * (int)sizeof(T));
 };
 
-__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(unsigned long long *b, unsigned n) {
-    asm volatile("mbarrier.init.shared.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(n) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_expect(unsigned long long *b, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
-}
-// Waits for the phase of parity `ph`; gives up (false) after a bounded number of attempts, far
-// beyond any copy's time.
-__device__ __forceinline__ bool mbar_wait(unsigned long long *b, unsigned ph) {
-    for (int n = 0; n < (1 << 22); ++n) {
-        unsigned ok;
-        asm volatile(
-            "{ .reg .pred p; mbarrier.try_wait.parity.shared.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-            : "=r"(ok)
-            : "r"(smem_u32(b)), "r"(ph)
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
@@ -119,11 +98,6 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_al
 // copies: without it they may use what an earlier launch's map at the same address left in a cache.
 __device__ __forceinline__ void map_acquire(const CUtensorMap *map) {
     asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
-}
-__device__ __forceinline__ void tma_load(void *dst, const CUtensorMap *map, int x, int y, unsigned long long *b) {
-    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-                 ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(0), "r"(smem_u32(b))
-                 : "memory");
 }
 
 // Step constants as pairs.
@@ -181,6 +155,7 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
         if (MODE == BATCHED && (n == 0 || G.tr[n & 3].x != G.tr[(n - 1) & 3].x))
             for (int k = 0; k < 3; ++k) map_acquire(maps + k);
         mbar_expect(&G.full, ST::FH * (NF * ST::WTF * (int)sizeof(TF) + (ND + 3) * ST::WT * (int)sizeof(T)));
+        if (t == A.withhold) return;
         tma_load(stage + ST::flow, maps, sizeof(TF) == 4 ? x : x & ~7, y, &G.full);
         tma_load(stage + ST::dual, maps + 1, sizeof(T) == 4 ? x : x & ~7, y, &G.full);
         tma_load(stage + ST::data, maps + 2, sizeof(T) == 4 ? x : x & ~7, y, &G.full);
@@ -201,8 +176,9 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
     // aligned.  Column borders mask (logic instructions: floating-point selects cost the FMA pipe), row
     // borders branch (masks in every row made a tile with both borders 20% slower).
     // BY: it touches the top or bottom one.
+    // False when the frame's copies did not arrive in time.
     template <int BX, bool BY>
-    static __device__ __forceinline__ void body(const TileArgs &A, SH &G, char *stage, const Tile &D, int n, int lane,
+    static __device__ __forceinline__ bool body(const TileArgs &A, SH &G, char *stage, const Tile &D, int n, int lane,
                                                 int wid) {
         const int H = D.H, W = D.W, P = D.P;
         const int c = D.bx * A.ow - A.offx + 2 * lane;   // this lane's even column
@@ -220,7 +196,7 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
         // ---- the frame, zero outside the image
         pair2 it[R];
         if constexpr (STAGE) {
-            if (!mbar_wait(&G.full, n & 1) && A.timeout) *A.timeout = 1;
+            const bool here = mbar_wait(&G.full, n & 1, A.wait_ns, A.timeout);
             const int x = c - 2 * lane;
             const int at_ = sizeof(T) == 4 ? 2 * lane : 2 * lane + (x & 7), af_ = sizeof(TF) == 4 ? 2 * lane : 2 * lane + (x & 7);
 #pragma unroll
@@ -241,7 +217,7 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
             }
             // the stage is free for the next tile, whose descriptor the first warp has by now
             if (MODE == BATCHED && wid == 0) cp_async_wait();
-            __syncthreads();
+            if (__syncthreads_or(!here)) return false;
             const int t1 = D.id + gridDim.x;
             if (t1 < A.ntiles) {
                 if (threadIdx.x == 0) prefetch(A, G, stage, t1, n + 1);
@@ -250,7 +226,7 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
                     fetch_ref(A, G, t1 + 2 * gridDim.x, n + 3, lane);
                 }
             }
-            if (done) return;  // the pair's warp met its stopping test
+            if (done) return true;  // the pair's warp met its stopping test
         } else {
             // pixels outside are read at the nearest pixel inside
             const int c0 = BX ? min(max(c, 0), W - 1) : c, c1 = BX ? min(max(c + 1, 0), W - 1) : c + 1;
@@ -563,6 +539,7 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
             const double tot = block_sum((double)res, G.red);
             if (threadIdx.x == 0) A.a.partials[D.id] = tot;
         }
+        return true;
     }
 
     static __device__ __forceinline__ void run(const TileArgs &A) {
@@ -572,7 +549,10 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
         const int lane = threadIdx.x & 31, wid = __shfl_sync(FULL, threadIdx.x >> 5, 0);
         if (MODE != BATCHED && A.a.done && *A.a.done) return;  // the pair's warp met its stopping test
         if (STAGE) {
-            if (threadIdx.x == 0) mbar_init(&G.full, 1);
+            if (threadIdx.x == 0) {
+                mbar_init(&G.full, 1);
+                mbar_init_fence();
+            }
             if (MODE == BATCHED && wid == 0) {
                 for (int k = 0; k < 3; ++k) fetch_ref(A, G, blockIdx.x + k * gridDim.x, k, lane);
                 cp_async_wait();
@@ -588,15 +568,24 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
 #pragma unroll 1
         for (int t = blockIdx.x; t < A.ntiles; t += gridDim.x, ++n) {
             const Tile D = tile_at(A, G, t, n);
+            bool ok;
             const int fj = D.bx * A.ow - A.offx;
             if (fj >= 1 && fj + FW <= D.W - 1 && A.vec) {
                 const int fi = D.by * A.oh - A.offy;
-                if (fi >= 1 && fi + R * NW <= D.H - 1) body<0, false>(A, G, stage, D, n, lane, wid);
-                else body<0, true>(A, G, stage, D, n, lane, wid);
+                if (fi >= 1 && fi + R * NW <= D.H - 1) ok = body<0, false>(A, G, stage, D, n, lane, wid);
+                else ok = body<0, true>(A, G, stage, D, n, lane, wid);
             } else if (D.W % 2 == 0 && A.vec) {
-                body<1, true>(A, G, stage, D, n, lane, wid);
+                ok = body<1, true>(A, G, stage, D, n, lane, wid);
             } else {
-                body<2, true>(A, G, stage, D, n, lane, wid);
+                ok = body<2, true>(A, G, stage, D, n, lane, wid);
+            }
+            if (STAGE && !ok) {
+                // the block leaves this tile and its later ones; the copies in flight have the same time again
+                if (threadIdx.x == 0) {
+                    if (A.timeout) *A.timeout = 1;
+                    mbar_wait(&G.full, n & 1, A.wait_ns, nullptr);
+                }
+                return;
             }
         }
     }

@@ -36,6 +36,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "k_mbar.cuh"
 #include "k_pack2.cuh"
 #include "k_pdr_math.cuh"
 
@@ -76,26 +77,6 @@ template <typename T, typename TF> struct Stage {
     static constexpr int own = x, own_b = x + 3 * FH * 256, own_rc = x + 6 * FH * 256;
 };
 
-__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void tma_load(void *dst, const CUtensorMap *map, int x, int y, unsigned long long *b) {
-    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-                 ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(0), "r"(smem_u32(b))
-                 : "memory");
-}
-// Waits for the copies; gives up (false) after a bounded number of attempts, far beyond their time.
-__device__ __forceinline__ bool mbar_wait(unsigned long long *b) {
-    for (int n = 0; n < (1 << 22); ++n) {
-        unsigned ok;
-        asm volatile(
-            "{ .reg .pred p; mbarrier.try_wait.parity.shared.b64 p, [%1], 0; selp.u32 %0, 1, 0, p; }"
-            : "=r"(ok)
-            : "r"(smem_u32(b))
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-
 template <typename T, typename TF, bool HAS_W> struct Kernel {
     static_assert(R % 2 == 0, "a row's colours must not depend on the warp");
     static constexpr int C0 = HAS_W ? 0 : 1;
@@ -124,7 +105,10 @@ template <typename T, typename TF, bool HAS_W> struct Kernel {
         auto own = [&](int base, int k, int r) -> pair2 & {
             return *reinterpret_cast<pair2 *>(stage + base + ((k * FH + wid * R + r) * 32 + lane) * 8);
         };
-        if (!mbar_wait(&G.full) && A.timeout) *A.timeout = 1;
+        if (!mbar_wait(&G.full, 0, A.wait_ns, A.timeout)) {  // reported; the copies in flight have the same time again
+            if (A.timeout) *A.timeout = 1;
+            mbar_wait(&G.full, 0, A.wait_ns, nullptr);
+        }
         auto rcp_of = [](float e) { return e > 0.f ? __frcp_rn(e) : 0.f; };  // (zero outside the image without beta)
         pair2 rcp[R];
 #pragma unroll
@@ -439,16 +423,16 @@ template <typename T, typename TF, bool HAS_W> struct Kernel {
         const int bx = blockIdx.x % A.gx, by = blockIdx.x / A.gx;
         const int fj = bx * A.ow - A.offx, fi = by * A.oh - A.offy;
         if (threadIdx.x == 0) {
-            asm volatile("mbarrier.init.shared.b64 [%0], 1;" ::"r"(smem_u32(&G.full)) : "memory");
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            asm volatile("mbarrier.arrive.expect_tx.shared.b64 _, [%0], %1;" ::"r"(smem_u32(&G.full)),
-                         "r"(2 * NF * ST::ptf + (ND + 3) * ST::pt)
-                         : "memory");
+            mbar_init(&G.full, 1);
+            mbar_init_fence();
+            mbar_expect(&G.full, 2 * NF * ST::ptf + (ND + 3) * ST::pt);
             const int xf = sizeof(TF) == 4 ? fj : fj & ~7, xt = sizeof(T) == 4 ? fj : fj & ~7;
-            tma_load(stage + ST::x, A.maps, xf, fi, &G.full);
-            tma_load(stage + ST::y, A.maps + 1, xt, fi, &G.full);
-            tma_load(stage + ST::data, A.maps + 2, xt, fi, &G.full);
-            tma_load(stage + ST::xbar, A.maps + 3, xf, fi, &G.full);
+            if (blockIdx.x != A.withhold) {
+                tma_load(stage + ST::x, A.maps, xf, fi, &G.full);
+                tma_load(stage + ST::y, A.maps + 1, xt, fi, &G.full);
+                tma_load(stage + ST::data, A.maps + 2, xt, fi, &G.full);
+                tma_load(stage + ST::xbar, A.maps + 3, xf, fi, &G.full);
+            }
         }
         __syncthreads();
         if (fj >= 1 && fj + 64 <= A.a.g.W - 1) {

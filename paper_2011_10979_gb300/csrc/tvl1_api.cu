@@ -1577,6 +1577,77 @@ of_status of_persistent_selftest(int H, int W, int iters, int withhold, double w
     return OF_OK;
 }
 
+of_status of_wait_selftest(int kernel, int withhold, double wait_ms, int *timed_out, int *parts) {
+    if (!timed_out || kernel < 0 || kernel > 2 || !(wait_ms > 0.0) || !isfinite(wait_ms))
+        return fail(OF_EINVAL, "of_wait_selftest: bad arguments");
+    of_params p;
+    of_default_params(&p);
+    if (kernel == 1) p.method = OF_PDR;
+    // levels of many tiles, some blocks with several; of one cluster
+    const int H = kernel == 2 ? 60 : 720, W = kernel == 2 ? 80 : 1280;
+    const Geom g{H, W, pitch_of(W)};
+    ResArgs r{};
+    const int nc = admm_resident_cluster();
+    TilePlan tp = kernel == 1 ? pdr_regtile_plan(g, 1) : admm_tile_plan(g, 4);
+    if (kernel == 2 ? !admm_cluster_plan(g, nc, &r) : !tp.staged) return fail(OF_ECUDA, "of_wait_selftest: no such plan");
+    const int np = kernel == 2 ? r.gx * ((H + r.oh - 1) / r.oh) : admm_tile_blocks(tp);
+    if (withhold >= np) return fail(OF_EINVAL, "of_wait_selftest: withhold beyond the number of parts");
+    if (parts) *parts = np;
+    // one device block, zero: 2 x 13 state planes, 3 data planes, the pair's scalars
+    const size_t plane = align_up((size_t)g.H * g.pitch * 4, 256), total = (2 * NFIELDS + 3) * plane + align_up(sizeof(Misc), 256);
+    char *D = nullptr;
+    cudaError_t e = cudaMalloc(&D, total);
+    if (e != cudaSuccess) return fail(OF_ECUDA, std::string("of_wait_selftest: cudaMalloc: ") + cudaGetErrorString(e));
+    Misc *misc = (Misc *)(D + (2 * NFIELDS + 3) * plane);
+    char *data = D + 2 * NFIELDS * plane;
+    TileArgs t{};
+    t.a.g = g;
+    t.a.k = coefs_of(&p);
+    t.a.in = fields_at(D, plane);
+    t.a.out = fields_at(D + NFIELDS * plane, plane);
+    t.a.Ix = data;
+    t.a.Iy = data + plane;
+    t.a.It = data + 2 * plane;
+    t.a.ms_max = &misc->ms_max;
+    e = cudaMemset(D, 0, total);
+    const long long ns = (long long)(wait_ms * 1e6);
+    if (e != cudaSuccess) {
+    } else if (kernel == 2) {
+        r.g = g;
+        r.k = t.a.k;
+        r.in = t.a.in;
+        r.out = t.a.out;
+        r.Ix = t.a.Ix;
+        r.Iy = t.a.Iy;
+        r.It = t.a.It;
+        r.ms_max = t.a.ms_max;
+        r.iters = 20;
+        r.sc.iters = &misc->iters;
+        r.timeout = &misc->timeout;
+        r.wait_ns = ns;
+        r.withhold = withhold;
+        e = launch_admm_cluster(r, nc, PREC_F32, PREC_F32, nullptr);
+    } else if (!tile_encode_maps(t.maps, t.a.in, t.a.Ix, t.a.Iy, g, PREC_F32, PREC_F32, true, kernel == 1)) {
+        e = cudaErrorUnknown;
+    } else {
+        tile_set_plan(t, tp, tp.ni);
+        t.vec = 1;
+        t.timeout = &misc->timeout;
+        t.wait_ns = ns;
+        t.withhold = withhold;
+        if (kernel == 1) launch_pdr_regtile(t, PREC_F32, PREC_F32, nullptr);
+        else launch_admm_tile(t, PREC_F32, PREC_F32, nullptr);
+        e = cudaGetLastError();
+    }
+    int to = 0;
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaMemcpy(&to, &misc->timeout, sizeof(int), cudaMemcpyDeviceToHost);
+    cudaFree(D);
+    if (e != cudaSuccess) return fail(OF_ECUDA, std::string("of_wait_selftest: ") + cudaGetErrorString(e));
+    *timed_out = to ? 1 : 0;
+    return OF_OK;
+}
+
 of_status of_rows_per_warp(of_ctx *ctx, int n, const int *H, const int *W, const of_params *params, int *rows) {
     if (!ctx || !H || !W || !params || !rows || n < 1) return fail(OF_EINVAL, "of_rows_per_warp: NULL argument or n < 1");
     for (int q = 0; q < n; ++q) {

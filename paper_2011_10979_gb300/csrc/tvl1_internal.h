@@ -39,6 +39,9 @@ struct Coefs {
                           // ms_max[-1] (Misc::c_cur); 0: c above
 };
 
+// Bound of every device-side wait, in nanoseconds: far beyond any copy's or neighbour's time.
+constexpr long long WAIT_NS = 2000000000LL;
+
 // One pair at one level, for the batched (work-list) form of the fused engines: both ping-pong
 // state buffers, the linearisation data and the pair's device scalars.
 struct __align__(16) PairIter {
@@ -120,6 +123,8 @@ struct TileArgs {
     int staged;
     int vec;              // every plane's rows start on an 8-byte boundary
     int *timeout;         // set when a bounded wait ran out
+    long long wait_ns = WAIT_NS;  // bound of every device-side wait
+    int withhold = -1;    // self-test: the tile whose copies are never started
     CUtensorMap maps[4];  // staged form, single pair: flow, dual and data planes, Xbar (pDR)
 };
 
@@ -156,6 +161,8 @@ struct ResArgs {
     double tol = 0.0;
     int gx = 0, ow = 0, oh = 0;  // launch_admm_cluster: columns of tiles, a tile's size
     int *timeout = nullptr;      // launch_admm_cluster: set when a bounded wait ran out
+    long long wait_ns = WAIT_NS;  // bound of its waits
+    int withhold = -1;           // self-test: the CTA that never sends
 };
 // ADMM methods, single pair: the register-resident form for small levels (k_admm_cluster.cuh).  Sets the
 // tiling of a level over a cluster of nc CTAs; false where it does not fit.
@@ -181,7 +188,7 @@ struct PersistArgs {
     double *partials = nullptr;         // per segment: FP64 residual partial
     int parity = 0, iters = 0, check = 0, final_res = 0;
     double tol = 0.0;
-    long long wait_ns = 2000000000LL;   // bound of every device-side wait
+    long long wait_ns = WAIT_NS;        // bound of every device-side wait
     int withhold = -1;                  // self-test: this segment never publishes its counter
 };
 // Co-resident blocks (of admm_fused_warps() warps) of the persistent instance for these storage

@@ -82,6 +82,7 @@ def lib():
             "of_rows_per_warp": (i, [vp, i, P(i), P(i), P(of_params), P(i)]),
             "of_resident_clusters": (i, [P(i), P(i)]),
             "of_persistent_selftest": (i, [i, i, i, i, d, P(i), P(i)]),
+            "of_wait_selftest": (i, [i, i, d, P(i), P(i)]),
             "of_l2_bandwidth": (i, [sz, i, P(d)]),
             "of_solve": (i, [vp, vp, vp, i, i, i, P(of_params), vp, vp, vp, i, vp, P(of_stats)]),
             "of_solve_host": (i, [vp, vp, vp, i, i, P(of_params), vp, vp, vp, vp, P(of_stats)]),
@@ -206,6 +207,13 @@ def of_persistent_selftest(H, W, iters, withhold, wait_ms) -> tuple:
     to, nseg = ctypes.c_int(0), ctypes.c_int(0)
     check(lib().of_persistent_selftest(H, W, iters, withhold, float(wait_ms), ctypes.byref(to), ctypes.byref(nseg)))
     return to.value, nseg.value
+
+
+def of_wait_selftest(kernel, withhold, wait_ms) -> tuple:
+    """(timed_out, parts) of the bounded-wait self-test of the tile kernels and the cluster engine."""
+    to, parts = ctypes.c_int(0), ctypes.c_int(0)
+    check(lib().of_wait_selftest(kernel, withhold, float(wait_ms), ctypes.byref(to), ctypes.byref(parts)))
+    return to.value, parts.value
 
 
 def of_l2_bandwidth(nbytes: int, passes: int) -> float:
