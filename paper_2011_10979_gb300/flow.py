@@ -21,7 +21,7 @@ OF_PREC_FP32, OF_PREC_FP16, OF_PREC_BF16 = 0, 1, 2
 OF_ENGINE_FUSED, OF_ENGINE_PLAIN, OF_ENGINE_STREAM, OF_ENGINE_RESIDENT, OF_ENGINE_PERSISTENT = 0, 1, 2, 3, 4
 
 EXPORTS = ("of_default_params", "of_create", "of_destroy", "of_last_error", "of_arena_bytes",
-           "of_solve_kernel_count", "of_rows_per_warp", "of_resident_clusters", "of_persistent_selftest", "of_l2_bandwidth", "of_solve",
+           "of_solve_kernel_count", "of_rows_per_warp", "of_resident_clusters", "of_persistent_selftest", "of_wait_selftest", "of_l2_bandwidth", "of_solve",
            "of_solve_host", "of_solve_batch", "of_pyr_down", "of_upsample", "of_derivatives",
            "of_warp_linearise", "of_admm_iterate", "of_admm_iterate_noalloc", "of_pdr_iterate", "of_cp_iterate",
            "of_fields_bytes", "of_energy",
