@@ -219,9 +219,10 @@ of_status of_persistent_selftest(int H, int W, int iters, int withhold, double w
 
 /* The same for the bounded waits of the kernels that wait for copies or neighbours within one launch:
  * kernel 0 = the several-iterations ADMM tile kernel on tiles copied ahead, 1 = pDR's, 2 = the ADMM
- * methods' cluster engine (small levels); one launch on zero-filled fields.  withhold: the tile whose
- * copies are never started, or the CTA that never sends (-1: none); *parts (optional) receives the
- * number of tiles or of CTAs with pixels.  *timed_out receives 1 when a wait ran out, else 0. */
+ * methods' cluster engine (small levels), 3 = the tile kernel over three pairs; one launch on zero-filled
+ * fields.  withhold: the tile whose copies are never started, or the CTA that never sends (-1: none);
+ * *parts (optional) receives the number of tiles or of CTAs with pixels.  *timed_out receives bit q when
+ * a wait that ran out left pair q unfinished (bit 0 but for kernel 3). */
 of_status of_wait_selftest(int kernel, int withhold, double wait_ms, int *timed_out, int *parts);
 
 /* Bandwidth of the L2 cache for a working set of `bytes` (half read, half written, FP32 words):

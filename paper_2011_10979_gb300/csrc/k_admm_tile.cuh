@@ -196,7 +196,7 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
         // ---- the frame, zero outside the image
         pair2 it[R];
         if constexpr (STAGE) {
-            const bool here = mbar_wait(&G.full, n & 1, A.wait_ns, A.timeout);
+            const bool here = mbar_wait(&G.full, n & 1, A.wait_ns, MODE == BATCHED ? G.pi[n % 3].timeout : A.timeout);
             const int x = c - 2 * lane;
             const int at_ = sizeof(T) == 4 ? 2 * lane : 2 * lane + (x & 7), af_ = sizeof(TF) == 4 ? 2 * lane : 2 * lane + (x & 7);
 #pragma unroll
@@ -580,9 +580,12 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
                 ok = body<2, true>(A, G, stage, D, n, lane, wid);
             }
             if (STAGE && !ok) {
-                // the block leaves this tile and its later ones; the copies in flight have the same time again
+                // the block leaves this tile and its later ones, whose pairs are reported; the copies in flight
+                // have the same time again
                 if (threadIdx.x == 0) {
-                    if (A.timeout) *A.timeout = 1;
+                    if (MODE == BATCHED)
+                        for (int k = t; k < A.ntiles; k += gridDim.x) *A.a.pairs[A.a.tiles[k].pair].timeout = 1;
+                    else if (A.timeout) *A.timeout = 1;
                     mbar_wait(&G.full, n & 1, A.wait_ns, nullptr);
                 }
                 return;

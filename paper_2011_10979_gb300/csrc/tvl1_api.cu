@@ -667,6 +667,7 @@ of_status upload_tables(of_ctx *ctx, const Batch &B, const of_params *p) {
             P.I1 = (const float *)(A + pl.img1[l]);
             P.I1x = (float *)(A + pl.I1x);
             P.I1y = (float *)(A + pl.I1y);
+            P.timeout = &misc->timeout;
             if (B.maps_off[l][v] > 0 && !B.res[l][k]) {
                 const size_t o = B.maps_off[l][v] + 6 * sizeof(CUtensorMap) * k;
                 P.maps = ctx->arena + B.table_off + o;
@@ -1106,7 +1107,6 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                         t.a = a;
                         tile_set_plan(t, tp, step);
                         t.vec = 1;
-                        t.timeout = &pc[0].misc->timeout;
                         launch_admm_tile(t, prec, pflow, s);
                     } else {
                         a.tiles = (const TileRef *)(ctx->arena + B.table_off + B.tiles_off[l]);
@@ -1375,10 +1375,9 @@ of_status read_stats(of_ctx *ctx, const Batch &B, int q, const of_params *p, cud
     stats->dual_value = (p->method == OF_PDR || p->method == OF_CP) ? NAN : m.dual;
     const bool adapt = p->c_adapt_iters > 0;
     stats->c = p->method == OF_PDR ? p->sigma * (adapt ? m.c_cur : 1.f) : adapt ? m.c_cur : p->c;
-    if (m.timeout) return fail(OF_ETIMEOUT, "a bounded wait of the persistent engine ran out");
-    if (!isfinite(stats->residual) || !isfinite(stats->energy))
-        return fail(OF_ENUMERIC, "non-finite residual or energy (NaN/Inf in the inputs or parameters?)");
-    return OF_OK;
+    const char *why = "";
+    const int st = tvl1_result_status(m.timeout, stats->residual, stats->energy, &why);
+    return st == OF_OK ? OF_OK : fail((of_status)st, why);
 }
 
 }  // namespace
@@ -1578,42 +1577,89 @@ of_status of_persistent_selftest(int H, int W, int iters, int withhold, double w
 }
 
 of_status of_wait_selftest(int kernel, int withhold, double wait_ms, int *timed_out, int *parts) {
-    if (!timed_out || kernel < 0 || kernel > 2 || !(wait_ms > 0.0) || !isfinite(wait_ms))
+    if (!timed_out || kernel < 0 || kernel > 3 || !(wait_ms > 0.0) || !isfinite(wait_ms))
         return fail(OF_EINVAL, "of_wait_selftest: bad arguments");
     of_params p;
     of_default_params(&p);
     if (kernel == 1) p.method = OF_PDR;
-    // levels of many tiles, some blocks with several; of one cluster
-    const int H = kernel == 2 ? 60 : 720, W = kernel == 2 ? 80 : 1280;
-    const Geom g{H, W, pitch_of(W)};
+    // levels of many tiles, some blocks with several; of one cluster; three pairs, the first the largest
+    const int n = kernel == 3 ? 3 : 1, H[3] = {kernel == 2 ? 60 : 720, 240, 240}, W[3] = {kernel == 2 ? 80 : 1280, 320, 320};
+    Geom g[3];
+    size_t base[3], plane[3], total = 0;
+    for (int q = 0; q < n; ++q) {
+        // a pair's 2 x 13 state planes, 3 data planes and scalars
+        g[q] = Geom{H[q], W[q], pitch_of(W[q])};
+        plane[q] = align_up((size_t)g[q].H * g[q].pitch * 4, 256);
+        base[q] = total;
+        total += (2 * NFIELDS + 3) * plane[q] + align_up(sizeof(Misc), 256);
+    }
     ResArgs r{};
     const int nc = admm_resident_cluster();
-    TilePlan tp = kernel == 1 ? pdr_regtile_plan(g, 1) : admm_tile_plan(g, 4);
-    if (kernel == 2 ? !admm_cluster_plan(g, nc, &r) : !tp.staged) return fail(OF_ECUDA, "of_wait_selftest: no such plan");
-    const int np = kernel == 2 ? r.gx * ((H + r.oh - 1) / r.oh) : admm_tile_blocks(tp);
+    TilePlan tp;
+    if (kernel == 1) tp = pdr_regtile_plan(g[0], 1);
+    else if (kernel == 3) tp = admm_tile_plan_batch(g, n, 4);
+    else tp = admm_tile_plan(g[0], 4);
+    if (kernel == 2 ? !admm_cluster_plan(g[0], nc, &r) : !tp.staged) return fail(OF_ECUDA, "of_wait_selftest: no such plan");
+    const int np = kernel == 2 ? r.gx * ((H[0] + r.oh - 1) / r.oh) : admm_tile_blocks(tp);
     if (withhold >= np) return fail(OF_EINVAL, "of_wait_selftest: withhold beyond the number of parts");
     if (parts) *parts = np;
-    // one device block, zero: 2 x 13 state planes, 3 data planes, the pair's scalars
-    const size_t plane = align_up((size_t)g.H * g.pitch * 4, 256), total = (2 * NFIELDS + 3) * plane + align_up(sizeof(Misc), 256);
+    // the work-list's tables behind the pairs: descriptors, tensor maps, tiles
+    const size_t o_pi = total, o_tm = o_pi + align_up(sizeof(PairIter) * n, 256);
+    const size_t o_tr = o_tm + align_up(6 * sizeof(CUtensorMap) * n, 256);
+    if (kernel == 3) total = o_tr + sizeof(TileRef) * np;
     char *D = nullptr;
     cudaError_t e = cudaMalloc(&D, total);
     if (e != cudaSuccess) return fail(OF_ECUDA, std::string("of_wait_selftest: cudaMalloc: ") + cudaGetErrorString(e));
-    Misc *misc = (Misc *)(D + (2 * NFIELDS + 3) * plane);
-    char *data = D + 2 * NFIELDS * plane;
-    TileArgs t{};
-    t.a.g = g;
-    t.a.k = coefs_of(&p);
-    t.a.in = fields_at(D, plane);
-    t.a.out = fields_at(D + NFIELDS * plane, plane);
-    t.a.Ix = data;
-    t.a.Iy = data + plane;
-    t.a.It = data + 2 * plane;
-    t.a.ms_max = &misc->ms_max;
     e = cudaMemset(D, 0, total);
+    auto misc_of = [&](int q) { return (Misc *)(D + base[q] + (2 * NFIELDS + 3) * plane[q]); };
+    auto state = [&](int q, int b) { return fields_at(D + base[q] + b * NFIELDS * plane[q], plane[q]); };
+    auto data = [&](int q, int d) { return D + base[q] + (2 * NFIELDS + d) * plane[q]; };
     const long long ns = (long long)(wait_ms * 1e6);
-    if (e != cudaSuccess) {
-    } else if (kernel == 2) {
-        r.g = g;
+    bool maps_ok = true;
+    TileArgs t{};
+    t.a.k = coefs_of(&p);
+    t.vec = 1;
+    t.wait_ns = ns;
+    t.withhold = withhold;
+    if (kernel == 3) {
+        std::vector<char> img(total - o_pi, 0);
+        TileRef *tr = (TileRef *)(img.data() + (o_tr - o_pi));
+        for (int q = 0; q < n; ++q) {
+            PairIter &P = ((PairIter *)img.data())[q];
+            P.g = g[q];
+            for (int b = 0; b < 2; ++b) P.buf[b] = state(q, b);
+            P.Ix = data(q, 0);
+            P.Iy = data(q, 1);
+            P.It = data(q, 2);
+            P.ms_max = &misc_of(q)->ms_max;
+            P.timeout = &misc_of(q)->timeout;
+            P.maps = D + o_tm + 6 * sizeof(CUtensorMap) * q;
+            for (int b = 0; b < 2; ++b) {
+                CUtensorMap m[3];
+                maps_ok = maps_ok && tile_encode_maps(m, P.buf[b], P.Ix, P.Iy, g[q], PREC_F32, PREC_F32, true);
+                memcpy(img.data() + (o_tm - o_pi) + (6 * q + 3 * b) * sizeof(CUtensorMap), m, sizeof(m));
+            }
+            for (int y = 0; y < tile_rows(tp, g[q]); ++y)
+                for (int x = 0; x < tile_cols(tp, g[q]); ++x) *tr++ = TileRef{q, x, y, 0};
+        }
+        t.a.pairs = (const PairIter *)(D + o_pi);
+        t.a.tiles = (const TileRef *)(D + o_tr);
+        if (e == cudaSuccess) e = cudaMemcpy(D + o_pi, img.data(), img.size(), cudaMemcpyHostToDevice);
+    } else {
+        t.a.g = g[0];
+        t.a.in = state(0, 0);
+        t.a.out = state(0, 1);
+        t.a.Ix = data(0, 0);
+        t.a.Iy = data(0, 1);
+        t.a.It = data(0, 2);
+        t.a.ms_max = &misc_of(0)->ms_max;
+        t.timeout = &misc_of(0)->timeout;
+        if (kernel != 2)
+            maps_ok = tile_encode_maps(t.maps, t.a.in, t.a.Ix, t.a.Iy, g[0], PREC_F32, PREC_F32, true, kernel == 1);
+    }
+    if (!maps_ok) e = cudaErrorUnknown;
+    if (e == cudaSuccess && kernel == 2) {
+        r.g = g[0];
         r.k = t.a.k;
         r.in = t.a.in;
         r.out = t.a.out;
@@ -1622,29 +1668,27 @@ of_status of_wait_selftest(int kernel, int withhold, double wait_ms, int *timed_
         r.It = t.a.It;
         r.ms_max = t.a.ms_max;
         r.iters = 20;
-        r.sc.iters = &misc->iters;
-        r.timeout = &misc->timeout;
+        r.sc.iters = &misc_of(0)->iters;
+        r.timeout = t.timeout;
         r.wait_ns = ns;
         r.withhold = withhold;
         e = launch_admm_cluster(r, nc, PREC_F32, PREC_F32, nullptr);
-    } else if (!tile_encode_maps(t.maps, t.a.in, t.a.Ix, t.a.Iy, g, PREC_F32, PREC_F32, true, kernel == 1)) {
-        e = cudaErrorUnknown;
-    } else {
+    } else if (e == cudaSuccess) {
         tile_set_plan(t, tp, tp.ni);
-        t.vec = 1;
-        t.timeout = &misc->timeout;
-        t.wait_ns = ns;
-        t.withhold = withhold;
         if (kernel == 1) launch_pdr_regtile(t, PREC_F32, PREC_F32, nullptr);
         else launch_admm_tile(t, PREC_F32, PREC_F32, nullptr);
         e = cudaGetLastError();
     }
-    int to = 0;
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    if (e == cudaSuccess) e = cudaMemcpy(&to, &misc->timeout, sizeof(int), cudaMemcpyDeviceToHost);
+    int out = 0;
+    for (int q = 0; q < n; ++q) {
+        int to = 0;
+        if (e == cudaSuccess) e = cudaMemcpy(&to, &misc_of(q)->timeout, sizeof(int), cudaMemcpyDeviceToHost);
+        out |= (to ? 1 : 0) << q;
+    }
     cudaFree(D);
     if (e != cudaSuccess) return fail(OF_ECUDA, std::string("of_wait_selftest: ") + cudaGetErrorString(e));
-    *timed_out = to ? 1 : 0;
+    *timed_out = out;
     return OF_OK;
 }
 
@@ -1778,6 +1822,19 @@ int tvl1_solve_async(of_ctx *ctx, const float *I0, const float *I1, int H, int W
 size_t tvl1_ctx_bytes(of_ctx *ctx) { return ctx ? ctx->arena_bytes : 0; }
 
 void tvl1_set_error(const char *msg) { g_err = msg; }
+
+extern "C" int tvl1_result_status(int timeout, double residual, double energy, const char **why) {
+    if (timeout) {
+        *why = "a bounded device-side wait ran out";
+        return OF_ETIMEOUT;
+    }
+    if (!std::isfinite(residual) || !std::isfinite(energy)) {
+        *why = "non-finite residual or energy (NaN/Inf in the inputs or parameters?)";
+        return OF_ENUMERIC;
+    }
+    *why = "";
+    return OF_OK;
+}
 
 extern "C" {
 

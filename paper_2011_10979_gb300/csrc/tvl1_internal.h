@@ -55,6 +55,7 @@ struct __align__(16) PairIter {
     const void *maps;  // tensor maps of the staged tile kernel: per buffer, flow, dual and data planes
     const float *I0, *I1;  // the level's images
     float *I1x, *I1y;      // the derivatives of I1
+    int *timeout;          // set when a bounded wait left the pair unfinished
 };
 
 // Device scalars of one pair in a batch, for the batched reductions: the partial sums of the
@@ -122,7 +123,7 @@ struct TileArgs {
     int gx, ntiles;       // single pair: tiles per row; tiles in all
     int staged;
     int vec;              // every plane's rows start on an 8-byte boundary
-    int *timeout;         // set when a bounded wait ran out
+    int *timeout;         // set when a bounded wait ran out (work-lists: the pairs' own flags)
     long long wait_ns = WAIT_NS;  // bound of every device-side wait
     int withhold = -1;    // self-test: the tile whose copies are never started
     CUtensorMap maps[4];  // staged form, single pair: flow, dual and data planes, Xbar (pDR)
@@ -371,3 +372,5 @@ int tvl1_solve_async(of_ctx *ctx, const float *I0, const float *I1, int H, int W
 size_t tvl1_ctx_bytes(of_ctx *ctx);
 // Sets the thread-local error message returned by of_last_error.
 void tvl1_set_error(const char *msg);
+// The of_status of a pair's finished solve from its timeout flag, residual and energy; *why: the reason.
+extern "C" int tvl1_result_status(int timeout, double residual, double energy, const char **why);

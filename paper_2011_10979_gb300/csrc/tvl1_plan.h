@@ -45,7 +45,7 @@ struct Misc {
     int done;
     long long iters;
     double res_check, res_final, energy, dual;
-    int timeout;  // a bounded wait of the persistent engine ran out
+    int timeout;  // a bounded device-side wait ran out
 };
 static_assert(offsetof(Misc, ms_max) == offsetof(Misc, c_cur) + sizeof(float), "c_cur must precede ms_max");
 static_assert(offsetof(Misc, done) == offsetof(Misc, ms_max) + sizeof(float), "done must follow ms_max");

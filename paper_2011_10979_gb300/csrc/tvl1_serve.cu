@@ -166,9 +166,9 @@ void retire(Server *S) {
             const size_t nin = (size_t)r->H * r->W, n = (size_t)r->h * r->w;
             r->u.assign(r->pin + 2 * nin, r->pin + 2 * nin + n);
             r->v.assign(r->pin + 2 * nin + n, r->pin + 2 * nin + 2 * n);
-            const bool finite = std::isfinite(r->misc.res_final) && std::isfinite(r->misc.energy);
-            finish_request(S, r, finite ? OF_OK : OF_ENUMERIC,
-                           finite ? "" : "non-finite residual or energy (NaN/Inf in the inputs?)");
+            const char *why = "";
+            const int st = tvl1_result_status(r->misc.timeout, r->misc.res_final, r->misc.energy, &why);
+            finish_request(S, r, st, why);
         } else {
             finish_request(S, r, OF_ECUDA, std::string("request failed on the device: ") + cudaGetErrorString(e));
         }

@@ -197,6 +197,7 @@ cudaError_t run_group(std::vector<StepPair *> &G, const of_params *p, StepTables
         P.I1 = (const float *)(q.A + q.pl.img1[q.l]);
         P.I1x = (float *)(q.A + q.pl.I1x);
         P.I1y = (float *)(q.A + q.pl.I1y);
+        P.timeout = &m->timeout;
         pl[k] = k;
         const int t0 = t;
         if (tile) {
@@ -260,7 +261,6 @@ cudaError_t run_group(std::vector<StepPair *> &G, const of_params *p, StepTables
             ta.a = a;
             tile_set_plan(ta, tp, step);
             ta.vec = 1;
-            ta.timeout = &misc_of(*G[0])->timeout;
             launch_admm_tile(ta, prec, pflow, s);
         } else {
             a.tiles = dtr;

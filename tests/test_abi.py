@@ -136,3 +136,13 @@ def test_adaptive_step_validation_without_gpu(L):
         assert b"c_adapt_iters" in L.of_last_error(None)
     with pytest.raises(TypeError):
         flow.default_params(c_adapt=20)
+
+
+def test_a_solve_whose_wait_ran_out_is_no_success(L):
+    """What of_solve's statistics and the serving loop report for a finished pair."""
+    why = ctypes.c_char_p()
+    L.tvl1_result_status.argtypes = [ctypes.c_int, ctypes.c_double, ctypes.c_double, ctypes.POINTER(ctypes.c_char_p)]
+    got = [L.tvl1_result_status(t, r, e, ctypes.byref(why))
+           for t, r, e in ((0, 0.1, 2.0), (1, 0.1, 2.0), (1, float("nan"), 2.0), (0, float("inf"), 2.0), (0, 0.1, float("nan")))]
+    assert got == [flow.OF_OK, flow.OF_ETIMEOUT, flow.OF_ETIMEOUT, flow.OF_ENUMERIC, flow.OF_ENUMERIC]
+    assert b"non-finite" in why.value

@@ -31,3 +31,15 @@ def test_a_wait_that_runs_out_is_reported_within_its_bound(kernel):
     st = flow.of_solve(ctx, torch.from_numpy(pr.I0).cuda(), torch.from_numpy(pr.I1).cuda(), flow.default_params())[3]
     assert st["energy"] == st["energy"]
     ctx.close()
+
+
+def test_the_pairs_that_a_wait_leaves_unfinished_are_the_ones_reported():
+    """A launch over three pairs whose last tile's copies never start: the last pair is reported, the others
+    are finished; a block that gives up at its first tile reports the pairs of all its tiles."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    to, parts = flow.of_wait_selftest(3, -1, 2000.0)
+    assert to == 0 and parts > 3 * 152
+    assert flow.of_wait_selftest(3, parts - 1, 100.0)[0] == 4
+    assert flow.of_wait_selftest(3, 0, 100.0)[0] & 1
+    assert flow.of_wait_selftest(3, -1, 2000.0)[0] == 0
