@@ -2028,10 +2028,13 @@ of_status iterate_common(of_fields f, const float *Ix, const float *Iy, const fl
     }
     if (pingpong && (launches & 1)) {
         // after an odd number of launches the result sits in the scratch buffer; an early stop
-        // (always after an even count) leaves it in the caller's planes.  Copy back unless stopped.
+        // (always after an even count) leaves it in the caller's planes.  Copy back unless stopped, and only
+        // what the iterations write: the scratch buffer's other planes hold nothing.
         Fields from = bufs[1], to = bufs[0];
-        for (int q = 0; q < NFIELDS; ++q)
-            if (!uf[q]) from.f[q] = to.f[q] = nullptr;
+        for (int q = 0; q < NFIELDS; ++q) {
+            const bool illum = q == F_W || q == F_P1 || q == F_P2 || q == F_WB, barred = q == F_WB || q == F_UB || q == F_VB;
+            if (!uf[q] || (illum && !has_w) || (cp ? q == F_S : barred)) from.f[q] = to.f[q] = nullptr;
+        }
         launch_parity_fix(from, to, g, PREC_F32, PREC_F32, params->tol > 0.0 ? &misc->done : nullptr, 0, s);
     }
     if (res2) {
