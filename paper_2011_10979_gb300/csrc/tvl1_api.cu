@@ -1583,7 +1583,7 @@ of_status of_wait_selftest(int kernel, int withhold, double wait_ms, int *timed_
     of_default_params(&p);
     if (kernel == 1) p.method = OF_PDR;
     // levels of many tiles, some blocks with several; of one cluster; three pairs, the first the largest
-    const int n = kernel == 3 ? 3 : 1, H[3] = {kernel == 2 ? 60 : 720, 240, 240}, W[3] = {kernel == 2 ? 80 : 1280, 320, 320};
+    const int n = kernel == 3 ? 3 : 1, H[3] = {kernel == 2 ? 60 : 1080, 240, 240}, W[3] = {kernel == 2 ? 80 : 1920, 320, 320};
     Geom g[3];
     size_t base[3], plane[3], total = 0;
     for (int q = 0; q < n; ++q) {
