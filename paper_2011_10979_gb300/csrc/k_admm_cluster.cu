@@ -3,7 +3,6 @@
 #include "k_admm_cluster.cuh"
 
 #include <algorithm>
-#include <mutex>
 
 namespace tvl1 {
 
@@ -11,13 +10,12 @@ namespace {
 
 template <typename T, typename TF, bool HAS_W, bool II, int R> cudaError_t launch_r(const ResArgs &a, int nc, cudaStream_t s) {
     auto kern = cluster::k_admm_cluster<T, TF, HAS_W, II, R>;
-    static std::once_flag once;
-    static cudaError_t prep;
-    std::call_once(once, [&] {
-        prep = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(cluster::Shared));
-        if (prep == cudaSuccess) prep = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    static DeviceOnce once;
+    const int prep = once.run(current_device(), [&] {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(cluster::Shared));
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     });
-    if (prep != cudaSuccess) return prep;
+    if (prep != cudaSuccess) return (cudaError_t)prep;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nc);
     cfg.blockDim = dim3((a.oh + 2 * cluster::HALO + R - 1) / R * 32);

@@ -37,7 +37,6 @@
 #include <cuda.h>
 #include <math.h>
 
-#include <mutex>
 #include <type_traits>
 
 #include "k_admm_math.cuh"
@@ -603,9 +602,9 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
 void launch_r(const TileArgs &a, cudaStream_t s) {
     constexpr int SMEM = (int)sizeof(Shared<NW, R>) + (MODE != DIRECT ? Stage<T, TF, NW * R>::bytes : 0);
     static_assert(SMEM <= 227 * 1024, "shared memory");
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(k_admm_tile<T, TF, HAS_W, VARIANT, NW, R, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    static DeviceOnce once;
+    once.run(current_device(), [] {
+        return cudaFuncSetAttribute(k_admm_tile<T, TF, HAS_W, VARIANT, NW, R, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     });
     const int blocks = MODE != DIRECT && a.ntiles > TILE_SMS ? TILE_SMS : a.ntiles;
     k_admm_tile<T, TF, HAS_W, VARIANT, NW, R, MODE><<<blocks, NW * 32, SMEM, s>>>(a);

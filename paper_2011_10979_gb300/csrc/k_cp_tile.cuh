@@ -30,7 +30,6 @@
 #pragma once
 #include <math.h>
 
-#include <mutex>
 #include <type_traits>
 
 #include "k_cp_math.cuh"
@@ -302,9 +301,9 @@ __global__ void __launch_bounds__(NW * 32, 1) k_cp_tile(const __grid_constant__ 
 
 template <typename T, typename TF, bool HAS_W, int R> void launch_r(const TileArgs &a, cudaStream_t s) {
     constexpr int SMEM = (int)sizeof(Shared<R>);
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(k_cp_tile<T, TF, HAS_W, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    static DeviceOnce once;
+    once.run(current_device(), [] {
+        return cudaFuncSetAttribute(k_cp_tile<T, TF, HAS_W, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     });
     k_cp_tile<T, TF, HAS_W, R><<<a.ntiles, NW * 32, SMEM, s>>>(a);
 }

@@ -481,10 +481,10 @@ __global__ void __launch_bounds__(TileShape<TT>::NT) k_pdr_tile(IterArgs A) {
 
 template <typename T, typename TF, int TT> void launch_pdr_tile_tt(const IterArgs &a, cudaStream_t s) {
     using TS = TileShape<TT>;
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static DeviceOnce once;
+    once.run(current_device(), [] {
         cudaFuncSetAttribute(k_pdr_tile<T, TF, true, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize, TS::SMEM);
-        cudaFuncSetAttribute(k_pdr_tile<T, TF, false, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize, TS::SMEM);
+        return cudaFuncSetAttribute(k_pdr_tile<T, TF, false, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize, TS::SMEM);
     });
     dim3 grid((a.g.W + TT - 1) / TT, (a.g.H + TT - 1) / TT, a.pairs ? a.ntiles : 1);
     if (a.k.beta != 0.f) k_pdr_tile<T, TF, true, TT><<<grid, TS::NT, TS::SMEM, s>>>(a);

@@ -33,7 +33,6 @@
 #include <cuda.h>
 #include <math.h>
 
-#include <mutex>
 #include <type_traits>
 
 #include "k_mbar.cuh"
@@ -454,9 +453,9 @@ __global__ void __launch_bounds__(NW * 32, 1) k_pdr_regtile(const __grid_constan
 template <typename T, typename TF, bool HAS_W> void launch_w(const TileArgs &a, cudaStream_t s) {
     constexpr int SMEM = (int)sizeof(Shared) + Stage<T, TF>::bytes;
     static_assert(SMEM <= 227 * 1024, "shared memory");
-    static std::once_flag once;
-    std::call_once(once, [] {
-        cudaFuncSetAttribute(k_pdr_regtile<T, TF, HAS_W>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    static DeviceOnce once;
+    once.run(current_device(), [] {
+        return cudaFuncSetAttribute(k_pdr_regtile<T, TF, HAS_W>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     });
     k_pdr_regtile<T, TF, HAS_W><<<a.ntiles, NW * 32, SMEM, s>>>(a);
 }

@@ -6,7 +6,14 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "tvl1_device_once.h"
+
 namespace tvl1 {
+
+inline int current_device() {
+    int dev = -1;
+    return cudaGetDevice(&dev) == cudaSuccess ? dev : -1;
+}
 
 // Storage precision of the iterated fields and linearisation data; arithmetic is always FP32.
 enum Prec { PREC_F32 = 0, PREC_F16 = 1, PREC_BF16 = 2 };
