@@ -95,8 +95,9 @@ void tile_set_plan(TileArgs &t, const TilePlan &p, int ni) {
     t.staged = p.staged;
 }
 
-bool tile_encode_maps(CUtensorMap *maps, const Fields &f, const void *Ix, const void *Iy, Geom g, int prec,
-                      int prec_flow, bool has_w, bool pdr) {
+namespace {
+
+PFN_cuTensorMapEncodeTiled_v12000 map_encoder() {
     static const PFN_cuTensorMapEncodeTiled_v12000 enc = [] {
         void *fn = nullptr;
         cudaDriverEntryPointQueryResult q;
@@ -106,6 +107,16 @@ bool tile_encode_maps(CUtensorMap *maps, const Fields &f, const void *Ix, const 
         }
         return (PFN_cuTensorMapEncodeTiled_v12000)fn;
     }();
+    return enc;
+}
+
+}  // namespace
+
+bool tile_maps_available() { return map_encoder() != nullptr; }
+
+bool tile_encode_maps(CUtensorMap *maps, const Fields &f, const void *Ix, const void *Iy, Geom g, int prec,
+                      int prec_flow, bool has_w, bool pdr) {
+    const PFN_cuTensorMapEncodeTiled_v12000 enc = map_encoder();
     if (!enc) return false;
     auto one = [&](CUtensorMap *m, const void *base, size_t plane, int n, int pr) {
         const int eb = (int)prec_bytes(pr);

@@ -107,6 +107,11 @@ int tile_iters_of(const of_params *p, int iters) {
     return p->engine == OF_ENGINE_STREAM || p->tol > 0.0 || iters <= 10 ? TILE_ITERS : 0;
 }
 
+bool batch_tile_of(const of_params *p, bool maps) {
+    return maps && (p->method == OF_PADMM_I || p->method == OF_PADMM_II) && p->a_tilde_mode == 0 && p->rows_per_warp == 0 &&
+           (p->engine == OF_ENGINE_FUSED || p->engine == OF_ENGINE_STREAM);
+}
+
 int tile_step(const of_params *p, int ni, int it, int iters) {
     int step = std::min(ni, iters - it);
     if (p->tol > 0.0) {
@@ -552,7 +557,7 @@ Batch make_batch(int n, const int *H, const int *W, const of_params *p) {
             t += align_up(sizeof(int) * n, 256);
             B.streamlist_off[l] = t;
             t += align_up(sizeof(int) * n, 256);
-            if (admm_tile_of(p) && p->a_tilde_mode == 0 && B.nres[l] < n && l >= B.out_level) {
+            if (batch_tile_of(p, tile_maps_available()) && B.nres[l] < n && l >= B.out_level) {
                 std::vector<Geom> gs;
                 for (int k = 0; k < n; ++k)
                     if (!B.res[l][k]) gs.push_back(geom_of(B.pl[k], l));
@@ -1822,6 +1827,8 @@ int tvl1_solve_async(of_ctx *ctx, const float *I0, const float *I1, int H, int W
 size_t tvl1_ctx_bytes(of_ctx *ctx) { return ctx ? ctx->arena_bytes : 0; }
 
 void tvl1_set_error(const char *msg) { g_err = msg; }
+
+extern "C" int tvl1_batch_tile(const of_params *params, int maps) { return batch_tile_of(params, maps != 0); }
 
 extern "C" int tvl1_result_status(int timeout, double residual, double energy, const char **why) {
     if (timeout) {

@@ -324,6 +324,8 @@ int admm_tile_blocks(const TilePlan &p);  // partial-sum slots of a launch
 inline int tile_cols(const TilePlan &p, Geom g) { return (g.W + p.ow - 1) / p.ow; }
 inline int tile_rows(const TilePlan &p, Geom g) { return (g.H + p.oh - 1) / p.oh; }
 void tile_set_plan(TileArgs &t, const TilePlan &p, int ni);
+// Whether the driver encodes tensor maps at all.
+bool tile_maps_available();
 // The staged form's tensor maps of a state buffer (its planes equally spaced) and the data planes;
 // pdr: without s and with a fourth map, of Xbar.  False when the driver cannot encode them.
 bool tile_encode_maps(CUtensorMap *maps, const Fields &f, const void *Ix, const void *Iy, Geom g, int prec,

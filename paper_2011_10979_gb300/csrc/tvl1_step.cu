@@ -140,7 +140,7 @@ cudaError_t run_group(std::vector<StepPair *> &G, const of_params *p, StepTables
     }
     // the ADMM tile kernel, several iterations per launch, by the built-in strip rule (as the whole
     // solve; the launches of 3, 3, 3 and 1 per ten iterations with the stopping test)
-    const bool tile = !(pdr || cp) && p->rows_per_warp == 0 && p->a_tilde_mode == 0 && (p->engine == OF_ENGINE_FUSED || p->engine == OF_ENGINE_STREAM);
+    const bool tile = batch_tile_of(p, tile_maps_available());
     TilePlan tp;
     if (tile) {
         std::vector<Geom> gs;

@@ -138,6 +138,19 @@ def test_adaptive_step_validation_without_gpu(L):
         flow.default_params(c_adapt=20)
 
 
+def test_batches_without_tensor_maps_keep_a_kernel(L):
+    """Where the driver encodes no tensor maps, batches and the serving loop run the row-streaming kernel instead
+    of failing; so do the settings that ask for it."""
+    def tile(maps, **kw):
+        return L.tvl1_batch_tile(ctypes.byref(flow.default_params(**kw)), maps)
+    L.tvl1_batch_tile.argtypes = [ctypes.POINTER(flow.of_params), ctypes.c_int]
+    for kw in (dict(), dict(method=flow.OF_PADMM_II), dict(engine=flow.OF_ENGINE_STREAM), dict(precision=2)):
+        assert tile(1, **kw) == 1 and tile(0, **kw) == 0, kw
+    for kw in (dict(method=flow.OF_PDR), dict(method=flow.OF_CP), dict(a_tilde_mode=1), dict(rows_per_warp=8),
+               dict(engine=flow.OF_ENGINE_PERSISTENT), dict(engine=flow.OF_ENGINE_RESIDENT)):
+        assert tile(1, **kw) == 0 and tile(0, **kw) == 0, kw
+
+
 def test_a_solve_whose_wait_ran_out_is_no_success(L):
     """What of_solve's statistics and the serving loop report for a finished pair."""
     why = ctypes.c_char_p()
