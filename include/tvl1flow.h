@@ -112,18 +112,21 @@ typedef struct {
                             ||M_s|| = max M_s, Prop. 3.1); 1 = the per-pixel diagonal
                             a~_ij = max(M_s(ij), 1e-12), which keeps c(diag(a~) - M_s) positive
                             semidefinite because M_s is diagonal (an extension, not in the paper) */
-    int rows_per_warp;   /* ADMM methods: strip height of the fused streaming kernel (rows each
-                            warp finishes per inner iteration; the strip is 29 columns wide):
-                            0 = chosen per level from the level's size by the built-in rule;
-                            1, 2, 8 or 32 = that height on every streamed level.
+    int rows_per_warp;   /* ADMM methods: 0 = the built-in choice per level (the tile kernel, several
+                            iterations per launch, or the level-resident launch);
+                            1, 2, 8 or 32 = one iteration per launch of the row-streaming
+                            kernel with that strip height (rows each warp finishes; the strip
+                            is 29 columns wide) on every streamed level.
                             pDR with gs_sweeps > 1 and ALG1: block height of their per-iteration
                             kernels (blocks of 32 columns): 0 = 8; 4, 8 or 16 = that height
-                            (pDR with one sweep runs one kernel of fixed 32 x 32 tiles per
-                            iteration and ignores it).
+                            (pDR with one sweep runs tile kernels of fixed shapes and ignores
+                            it).
                             -1 = autotuned: the first solve of a layout on a context times every
                             height on each level that runs those kernels (a few iterations of the
                             real launch on the arena, after a device synchronisation) and keeps
-                            the fastest for that context.  The flow does not depend on it (the
+                            the fastest for that context.  A batch of an ADMM method also times
+                            the tile kernel; a single pair's levels take the fastest height (0
+                            is the faster choice there).  The flow does not depend on it (the
                             per-pixel arithmetic is the same); only the grouping of the
                             residual's partial sums changes, so the residual (and a stopping
                             decision taken on it) can differ in the last FP32 digits.  Used by

@@ -108,7 +108,7 @@ int tile_iters_of(const of_params *p, int iters) {
 }
 
 bool batch_tile_of(const of_params *p, bool maps) {
-    return maps && (p->method == OF_PADMM_I || p->method == OF_PADMM_II) && p->a_tilde_mode == 0 && p->rows_per_warp == 0 &&
+    return maps && (p->method == OF_PADMM_I || p->method == OF_PADMM_II) && p->a_tilde_mode == 0 && p->rows_per_warp <= 0 &&
            (p->engine == OF_ENGINE_FUSED || p->engine == OF_ENGINE_STREAM);
 }
 
@@ -335,8 +335,8 @@ constexpr long PDR_REGTILE_MIN_PX = 40000;
 constexpr long PDR_TILE_RESIDENT_MAX_PX = 12000;
 
 // Whether streamed ADMM levels run several iterations per launch (k_admm_tile.cuh): the built-in
-// strip rule (a pinned or autotuned height asks for the row-streaming kernel), at any size, single
-// pairs and batches.
+// strip rule (a pinned or, for a single pair, autotuned height asks for the row-streaming kernel), at any
+// size; batches: batch_tile_of.
 bool admm_tile_of(const of_params *p) {
     return (p->method == OF_PADMM_I || p->method == OF_PADMM_II) && p->rows_per_warp == 0 &&
            (p->engine == OF_ENGINE_FUSED || p->engine == OF_ENGINE_STREAM);
@@ -1198,10 +1198,11 @@ int level_rows(const Batch &B, int l) {
     return admm_fused_tile_h(geom_of(B.pl[0], l), B.pl[0].prec != PREC_F32);
 }
 
-// What the kernel's speed depends on: the kernel instance (method, per-pixel a~, beta > 0,
-// storage types), single or batched form, and the geometries of the streamed pairs.
+// What the choice depends on: the kernel instance (method, per-pixel a~, beta > 0, storage types), single or
+// batched form, whether the tile kernel is a candidate, and the geometries of the streamed pairs.
 std::string tune_key(const Batch &B, const of_params *p, int l) {
-    const int hdr[6] = {p->method, p->a_tilde_mode, p->beta != 0.f ? 1 : 0, B.pl[0].prec, B.pl[0].pflow, B.n > 1 ? 1 : 0};
+    const int hdr[7] = {p->method, p->a_tilde_mode, p->beta != 0.f ? 1 : 0, B.pl[0].prec, B.pl[0].pflow, B.n > 1 ? 1 : 0,
+                        B.tp[l].R > 0 ? 1 : 0};
     std::string k((const char *)hdr, sizeof(hdr));
     for (int q = 0; q < B.n; ++q) {
         if (B.n > 1 && B.res[l][q]) continue;
@@ -1212,8 +1213,8 @@ std::string tune_key(const Batch &B, const of_params *p, int l) {
     return k;
 }
 
-// One inner iteration of level l on its per-iteration kernel, as the solve launches it (storage
-// precision of the level's main warps; no stop flag, no residual partials).
+// One launch of level l's per-iteration kernel (one iteration; the tile kernel: its plan's number), as the
+// solve launches it (storage precision of the level's main warps; no stop flag, no residual partials).
 void launch_level_iteration(of_ctx *ctx, const Batch &B, const of_params *p, int l, int parity, cudaStream_t s) {
     const bool pdr = p->method == OF_PDR, cp = p->method == OF_CP;
     IterArgs a{};
@@ -1240,6 +1241,15 @@ void launch_level_iteration(of_ctx *ctx, const Batch &B, const of_params *p, int
             a.ntiles = B.n - B.nres[l];
             a.plist = (const int *)(ctx->arena + B.table_off + B.streamlist_off[l]);
             a.parity = pdr && !pdr_tile_of(p) ? 0 : parity;
+        } else if (B.tp[l].R > 0) {
+            TileArgs t{};
+            a.tiles = (const TileRef *)(ctx->arena + B.table_off + B.ttiles_off[l]);
+            a.parity = parity;
+            t.a = a;
+            tile_set_plan(t, B.tp[l], B.tp[l].ni);
+            t.vec = 1;
+            launch_admm_tile(t, B.pl[0].prec, B.pl[0].pflow, s);
+            return;
         } else {
             a.tiles = (const TileRef *)(ctx->arena + B.table_off + B.tiles_off[l]);
             a.ntiles = B.ntiles[l];
@@ -1252,9 +1262,20 @@ void launch_level_iteration(of_ctx *ctx, const Batch &B, const of_params *p, int
     else launch_admm_fused(a, B.pl[0].prec, B.pl[0].pflow, s);
 }
 
-// Times every candidate shape on level l -- the strip heights of the streaming ADMM kernel, or the
-// block heights of the pDR / ALG1 kernels -- (2 untimed and 6 timed iterations each, CUDA events
-// on the context's own stream) and returns the fastest; ties keep the lower one.
+constexpr int TUNED_TILE = 0;
+
+// Sets level l to a tuned shape: TUNED_TILE (the batched tile kernel of plan tp, the level's height staying
+// `height`), or a strip or block height.
+void set_rows(Batch &B, const of_params *p, int l, int ty, const TilePlan &tp, int height) {
+    B.tp[l] = ty == TUNED_TILE ? tp : TilePlan();
+    B.tile_h[l] = ty == TUNED_TILE ? height : ty;
+    if (B.n > 1 && block_height_of(p) == 0) B.ntiles[l] = batch_tiles(B, l, B.tile_h[l]);
+}
+
+// Times every candidate shape on level l -- the strip heights of the streaming ADMM kernel and, for a batch, the
+// tile kernel (TUNED_TILE), or the block heights of the pDR / ALG1 kernels -- (2 untimed and 6 timed
+// iterations each, the tile kernel's in launches of its plan's length; CUDA events on the context's own stream)
+// and returns the fastest; ties keep the lower one.
 of_status tune_level(of_ctx *ctx, Batch &B, const of_params *p, int l, int *best) {
     static const int cand_admm[4] = {1, 2, 8, 32}, cand_blocks[3] = {4, 8, 16};
     const bool blocks = p->method == OF_PDR || p->method == OF_CP;
@@ -1270,16 +1291,18 @@ of_status tune_level(of_ctx *ctx, Batch &B, const of_params *p, int l, int *best
         if (st != OF_OK) return st;
     }
     float best_ms = 0.f;
-    *best = 0;
-    for (int c = 0; c < ncand; ++c) {
-        const int ty = cand[c];
-        B.tile_h[l] = ty;
+    *best = -1;
+    const TilePlan tp = B.tp[l];
+    const int height = B.tile_h[l];  // the built-in rule's, which a level on the tile kernel reports
+    for (int c = tp.R > 0 ? -1 : 0; c < ncand; ++c) {
+        const int ty = c < 0 ? TUNED_TILE : cand[c];
+        set_rows(B, p, l, ty, tp, height);
         if (B.n > 1 && !blocks) {
-            B.ntiles[l] = batch_tiles(B, l, ty);
             of_status st = upload_tables(ctx, B, &q);
             ctx->tables_key.clear();
             if (st != OF_OK) return st;
         }
+        const int len = B.tp[l].R > 0 ? tp.ni : 1;  // iterations per launch
         for (int it = 0; it < WARM + REPS; ++it) {
             if (it == WARM) OF_CUDA(cudaEventRecord(ctx->ev0, ctx->cap));
             launch_level_iteration(ctx, B, &q, l, it & 1, ctx->cap);
@@ -1289,11 +1312,13 @@ of_status tune_level(of_ctx *ctx, Batch &B, const of_params *p, int l, int *best
         OF_CUDA(cudaGetLastError());
         float ms = 0.f;
         OF_CUDA(cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1));
-        if (*best == 0 || ms < best_ms) {
+        ms /= len;
+        if (*best < 0 || ms < best_ms) {
             best_ms = ms;
             *best = ty;
         }
     }
+    set_rows(B, p, l, *best, tp, height);
     return OF_OK;
 }
 
@@ -1327,8 +1352,7 @@ of_status resolve_rows(of_ctx *ctx, Batch &B, const of_params *p) {
             if (st != OF_OK) return st;
             ctx->tuned[key] = ty;
         }
-        B.tile_h[l] = ty;
-        if (B.n > 1 && block_height_of(p) == 0) B.ntiles[l] = batch_tiles(B, l, ty);
+        set_rows(B, p, l, ty, B.tp[l], B.tile_h[l]);
     }
     return OF_OK;
 }

@@ -56,9 +56,10 @@ Plan make_plan(int H, int W, const of_params *p);
 // Kernel coefficients of the parameters.
 Coefs coefs_of(const of_params *p);
 
-// Whether the shared launches of a batch, or of the serving loop, run the ADMM tile kernel: with the built-in strip
-// rule (a pinned or autotuned height asks for the row-streaming kernel) and one a~ per warp, where the driver
-// encodes tensor maps (maps); the row-streaming kernel needs none.
+// Whether the shared launches of a batch, or of the serving loop, may run the ADMM tile kernel: without a pinned
+// strip height (which asks for the row-streaming kernel; a batch's autotuner times both kernels, the serving loop
+// does not tune) and with one a~ per warp, where the driver encodes tensor maps (maps); the row-streaming
+// kernel needs none.
 bool batch_tile_of(const of_params *p, bool maps);
 
 // Iterations per launch of the ADMM tile kernel for a warp of `iters` iterations: the level's choice

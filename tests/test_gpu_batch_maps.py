@@ -59,3 +59,22 @@ def test_alternating_request_mixes(pairs, prec):
     finally:
         flow.of_server_stop(ctx)
         ctx.close()
+
+
+def test_autotuned_batch_is_not_slower_than_the_built_in_choice(pairs):
+    """The autotuner of a batch times the tile kernel beside the strip heights: what it keeps is no slower than the
+    built-in choice (a quarter allowed for noise; the fastest height takes about 1.6 times as long), and the
+    flows are the same."""
+    big = [synth.random_affine_rect_pair(480, 640, 70 + k) for k in range(6)]
+    I0, I1 = [torch.from_numpy(p.I0).cuda() for p in big], [torch.from_numpy(p.I1).cuda() for p in big]
+    ctx = flow.Context(0)
+    ms, out = {}, {}
+    for rows in (0, -1, 0, -1):
+        P = flow.default_params(lam=5.0, levels=2, warps=2, iters=60, precision=flow.OF_PREC_BF16, rows_per_warp=rows)
+        for _ in range(3):
+            us, vs, st = flow.of_solve_batch(ctx, I0, I1, P)
+            ms[rows] = min(ms.get(rows, 1e9), st[0]["ms"])
+        out[rows] = us + vs
+    assert all(torch.equal(a, b) for a, b in zip(out[0], out[-1]))
+    assert ms[-1] <= 1.25 * ms[0], ms
+    ctx.close()
