@@ -69,6 +69,7 @@ template <int NW, int R> struct Shared {
     PairIter pi[3];
     int4 tr[4];
     double red[32];
+    int dead;                              // staged form: the first thread's wait for copies ran out
     unsigned long long full;               // staged form: the mbarrier the copies complete on
 };
 
@@ -144,6 +145,19 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
         return D;
     }
 
+    // After a wait that ran out: reports the pair (what the block makes of the tile is void).  The first thread starts
+    // no more copies, so it reports the pairs of all the block's later tiles, and gives the copies in flight the
+    // same time again.
+    static __device__ __noinline__ void missed(const TileArgs &A, SH &G, int t, int n) {
+        if (MODE == BATCHED) *G.pi[n % 3].timeout = 1;
+        else if (A.timeout) *A.timeout = 1;
+        if (threadIdx.x != 0) return;
+        G.dead = 1;
+        if (MODE == BATCHED)
+            for (t += gridDim.x; t < A.ntiles; t += gridDim.x) *A.a.pairs[A.a.tiles[t].pair].timeout = 1;
+        mbar_wait(&G.full, n & 1, A.wait_ns, nullptr);
+    }
+
     // Starts the copies of a tile's frame into the stage (one thread); zeros outside the image.
     static __device__ __forceinline__ void prefetch(const TileArgs &A, SH &G, char *stage, int t, int n) {
         const Tile D = tile_at(A, G, t, n);
@@ -175,9 +189,8 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
     // aligned.  Column borders mask (logic instructions: floating-point selects cost the FMA pipe), row
     // borders branch (masks in every row made a tile with both borders 20% slower).
     // BY: it touches the top or bottom one.
-    // False when the frame's copies did not arrive in time.
     template <int BX, bool BY>
-    static __device__ __forceinline__ bool body(const TileArgs &A, SH &G, char *stage, const Tile &D, int n, int lane,
+    static __device__ __forceinline__ void body(const TileArgs &A, SH &G, char *stage, const Tile &D, int n, int lane,
                                                 int wid) {
         const int H = D.H, W = D.W, P = D.P;
         const int c = D.bx * A.ow - A.offx + 2 * lane;   // this lane's even column
@@ -195,7 +208,7 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
         // ---- the frame, zero outside the image
         pair2 it[R];
         if constexpr (STAGE) {
-            const bool here = mbar_wait(&G.full, n & 1, A.wait_ns, MODE == BATCHED ? G.pi[n % 3].timeout : A.timeout);
+            if (!mbar_wait(&G.full, n & 1, A.wait_ns, MODE == BATCHED ? G.pi[n % 3].timeout : A.timeout)) missed(A, G, D.id, n);
             const int x = c - 2 * lane;
             const int at_ = sizeof(T) == 4 ? 2 * lane : 2 * lane + (x & 7), af_ = sizeof(TF) == 4 ? 2 * lane : 2 * lane + (x & 7);
 #pragma unroll
@@ -216,16 +229,17 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
             }
             // the stage is free for the next tile, whose descriptor the first warp has by now
             if (MODE == BATCHED && wid == 0) cp_async_wait();
-            if (__syncthreads_or(!here)) return false;
+            const bool dead = threadIdx.x == 0 && *(volatile int *)&G.dead;
+            __syncthreads();
             const int t1 = D.id + gridDim.x;
             if (t1 < A.ntiles) {
-                if (threadIdx.x == 0) prefetch(A, G, stage, t1, n + 1);
+                if (threadIdx.x == 0 && !dead) prefetch(A, G, stage, t1, n + 1);
                 if (MODE == BATCHED && wid == 0) {
                     fetch_pair(A, G, n + 2, lane);
                     fetch_ref(A, G, t1 + 2 * gridDim.x, n + 3, lane);
                 }
             }
-            if (done) return true;  // the pair's warp met its stopping test
+            if (done) return;  // the pair's warp met its stopping test
         } else {
             // pixels outside are read at the nearest pixel inside
             const int c0 = BX ? min(max(c, 0), W - 1) : c, c1 = BX ? min(max(c + 1, 0), W - 1) : c + 1;
@@ -538,7 +552,6 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
             const double tot = block_sum((double)res, G.red);
             if (threadIdx.x == 0) A.a.partials[D.id] = tot;
         }
-        return true;
     }
 
     static __device__ __forceinline__ void run(const TileArgs &A) {
@@ -549,6 +562,7 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
         if (MODE != BATCHED && A.a.done && *A.a.done) return;  // the pair's warp met its stopping test
         if (STAGE) {
             if (threadIdx.x == 0) {
+                G.dead = 0;
                 mbar_init(&G.full, 1);
                 mbar_init_fence();
             }
@@ -567,27 +581,15 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
 #pragma unroll 1
         for (int t = blockIdx.x; t < A.ntiles; t += gridDim.x, ++n) {
             const Tile D = tile_at(A, G, t, n);
-            bool ok;
             const int fj = D.bx * A.ow - A.offx;
             if (fj >= 1 && fj + FW <= D.W - 1 && A.vec) {
                 const int fi = D.by * A.oh - A.offy;
-                if (fi >= 1 && fi + R * NW <= D.H - 1) ok = body<0, false>(A, G, stage, D, n, lane, wid);
-                else ok = body<0, true>(A, G, stage, D, n, lane, wid);
+                if (fi >= 1 && fi + R * NW <= D.H - 1) body<0, false>(A, G, stage, D, n, lane, wid);
+                else body<0, true>(A, G, stage, D, n, lane, wid);
             } else if (D.W % 2 == 0 && A.vec) {
-                ok = body<1, true>(A, G, stage, D, n, lane, wid);
+                body<1, true>(A, G, stage, D, n, lane, wid);
             } else {
-                ok = body<2, true>(A, G, stage, D, n, lane, wid);
-            }
-            if (STAGE && !ok) {
-                // the block leaves this tile and its later ones, whose pairs are reported; the copies in flight
-                // have the same time again
-                if (threadIdx.x == 0) {
-                    if (MODE == BATCHED)
-                        for (int k = t; k < A.ntiles; k += gridDim.x) *A.a.pairs[A.a.tiles[k].pair].timeout = 1;
-                    else if (A.timeout) *A.timeout = 1;
-                    mbar_wait(&G.full, n & 1, A.wait_ns, nullptr);
-                }
-                return;
+                body<2, true>(A, G, stage, D, n, lane, wid);
             }
         }
     }

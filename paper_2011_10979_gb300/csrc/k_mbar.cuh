@@ -42,12 +42,9 @@ template <bool CLUSTER> __device__ __forceinline__ bool mbar_try(unsigned long l
                      : "memory");
     return ok;
 }
-// Waits for the phase of parity ph, at most ns nanoseconds, or one millisecond when *flag (may be NULL) is set;
-// false when the time ran out.
-template <bool CLUSTER = false>
-__device__ __forceinline__ bool mbar_wait(unsigned long long *b, unsigned ph, long long ns, const int *flag) {
-    for (int k = 0; k < 32; ++k)
-        if (mbar_try<CLUSTER>(b, ph)) return true;
+// The rest of a wait that its first attempts did not end: at most ns nanoseconds, or one millisecond when *flag (may
+// be NULL) is set; false when the time ran out.  Out of line, beside the registers and the code of the kernels.
+template <bool CLUSTER> __device__ __noinline__ bool mbar_wait_timed(unsigned long long *b, unsigned ph, long long ns, const int *flag) {
     unsigned long long t0, t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
     for (;;) {
@@ -56,6 +53,14 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long *b, unsigned ph, lo
         const long long dt = (long long)(t - t0);
         if (dt > ns || (dt > 1000000 && flag && *(const volatile int *)flag)) return false;
     }
+}
+// Waits for the phase of parity ph (reading the timer takes longer than a wait usually does).
+template <bool CLUSTER = false>
+__device__ __forceinline__ bool mbar_wait(unsigned long long *b, unsigned ph, long long ns, const int *flag) {
+#pragma unroll 1
+    for (int k = 0; k < 4096; ++k)
+        if (mbar_try<CLUSTER>(b, ph)) return true;
+    return mbar_wait_timed<CLUSTER>(b, ph, ns, flag);
 }
 
 }  // namespace tvl1
