@@ -35,11 +35,12 @@ TilePlan plan_of(Geom g, int R, int ni, bool staged) {
 // over the SMs: a part per tile and one per iteration; FP32, beta > 0).  Measured against it: 320x240,
 // R = 2, five iterations 8.4 us; 640x480, R = 4, three 10.6 and R = 3, six 20.7; 1024x436 staged, six
 // 27.1 and R = 3, three 14.5; 3840x2160 staged, four 239.
-float plan_us(const TilePlan &p) {
+float plan_us(const TilePlan &p, int R, int ni) {
     static const float per_iter[5] = {0.f, 0.f, 0.95f, 1.2f, 1.7f}, per_tile[5] = {0.f, 0.f, 3.2f, 3.7f, 4.9f};
     const int n = p.gx * p.gy, rounds = (n + TILE_SMS - 1) / TILE_SMS;
-    return p.staged ? 3.4f + rounds * (3.8f + 1.25f * p.ni) : 0.4f + rounds * (per_tile[p.R] + p.ni * per_iter[p.R]);
+    return p.staged ? 3.4f + rounds * (3.8f + 1.25f * ni) : 0.4f + rounds * (per_tile[R] + ni * per_iter[R]);
 }
+float plan_us(const TilePlan &p) { return plan_us(p, p.R, p.ni); }
 
 }  // namespace
 
@@ -80,6 +81,8 @@ TilePlan admm_tile_plan_batch(const Geom *g, int n, int ni) {
     }
     return best;
 }
+
+float admm_tile_us(const TilePlan &p, int ni, bool per_pixel) { return plan_us(p, per_pixel ? 4 : p.R, ni); }
 
 int admm_tile_blocks(const TilePlan &p) { return p.gx * p.gy; }
 

@@ -1948,6 +1948,29 @@ size_t of_fields_bytes(int H, int pitch) {
 
 namespace {
 
+// Iterations of a step-level call's next launch of the tile kernel, after `it` iterations in `launches` launches:
+// an even number of launches leaves the state in the caller's planes.
+int iterate_step(const of_params *p, const TilePlan &tp, int it, int iters, int launches) {
+    const int step = tile_step(p, tp.ni, it, iters);
+    return it + step == iters && step > 1 && launches % 2 == 0 ? step - 1 : step;
+}
+
+// Whether a step-level ADMM call runs the tile kernel, rather than one launch per iteration of the row-streaming
+// kernel: by the estimated time of all its launches.  Launched one by one, a launch takes 4.1 us at least and an
+// iteration of the row-streaming kernel 4.5 us + 18.7 ps per pixel (measured: 6.2 us at 320x240, 10.3 at 640x480,
+// 43 at 1920x1080).  Levels a few rows high are faster row by row (312 us against 518 for fifty iterations with a
+// per-pixel a~ at 30000x2), and so are one and two iterations at every size (a call of two: 89 us against 130 at
+// 1920x1080, 25 against 26.5 at 64x48).
+bool iterate_tile_of(const of_params *p, Geom g, const TilePlan &tp, int iters) {
+    float us = 0.f;
+    for (int it = 0, launches = 0; it < iters; ++launches) {
+        const int step = iterate_step(p, tp, it, iters, launches);
+        us += std::max(4.1f, admm_tile_us(tp, step, p->a_tilde_mode == 1));
+        it += step;
+    }
+    return iters > 2 && us < iters * (4.5f + 1.87e-5f * (float)g.W * (float)g.H);
+}
+
 // Step-level iterations of one method family: KIND_ADMM (rpADMMI / rpADMMII), KIND_PDR, KIND_CP.
 enum { KIND_ADMM = 0, KIND_PDR = 1, KIND_CP = 2 };
 
@@ -1990,43 +2013,39 @@ of_status iterate_common(of_fields f, const float *Ix, const float *Iy, const fl
     float *tmp = (float *)(S + NFIELDS * plane);
     // the scratch layout depends on (H, pitch) only, as of_fields_bytes does; the engine in use
     // must find room for its partial sums in it
+    const bool plain = params->engine == OF_ENGINE_PLAIN;
+    // ADMM, fused engines: the tile kernel straight from the caller's planes, several iterations per launch,
+    // or the row-streaming kernel
+    const TilePlan tp = admm_tile_plan(g, params->tol > 0.0 ? TILE_ITERS : 0, true);
+    const bool tile = !xb && !plain && iterate_tile_of(params, g, tp, iters);
     const int mb = fields_partial_slots(H, pitch);
-    const int nb_used = pdr ? pdr_plain_blocks(g)
-                            : cp ? cp_blocks(g)
-                                 : (params->engine == OF_ENGINE_PLAIN
-                                        ? admm_plain_blocks(g)
-                                        : admm_tile_blocks(admm_tile_plan(g, params->tol > 0.0 ? TILE_ITERS : 0, true)));
+    const int nb_used = pdr     ? pdr_plain_blocks(g)
+                        : cp    ? cp_blocks(g)
+                        : plain ? admm_plain_blocks(g)
+                        : tile  ? admm_tile_blocks(tp)
+                                : admm_fused_blocks(g);
     if (nb_used > mb) return fail(OF_EINVAL, "internal: partial sums exceed the scratch layout");
     double *partials = (double *)(S + (NFIELDS + 6) * plane);
     Misc *misc = (Misc *)(S + (NFIELDS + 6) * plane + align_up((size_t)mb * sizeof(double), 256));
     OF_CUDA(cudaMemsetAsync(misc, 0, sizeof(Misc), s));
     for (int k = 0; k < NFIELDS; ++k)
         if (!uf[k]) OF_CUDA(cudaMemset2DAsync(user.f[k], (size_t)pitch * 4, 0, (size_t)W * 4, H, s));
-    const bool plain = params->engine == OF_ENGINE_PLAIN;
     const bool pingpong = !pdr && !plain;
     Fields bufs[2] = {user, other};
     of_params pp = *params;
     pp.a_tilde = xb ? 1.f : a_tilde;
     const Coefs k = coefs_of(&pp);
     const double rows = (double)H * W * (has_w ? 3.0 : 2.0);
-    // ADMM, fused engines: the tile kernel straight from the caller's planes (8-byte loads where every
-    // plane and row allows them), several iterations per launch
-    const bool tile = !xb && !plain;
-    TilePlan tp;
+    // 8-byte loads where every plane and row allows them
     bool vec = W % 2 == 0 && pitch % 2 == 0;
     if (tile) {
-        tp = admm_tile_plan(g, params->tol > 0.0 ? TILE_ITERS : 0, true);
         for (int q = 0; q < NFIELDS; ++q) vec = vec && (uintptr_t)user.f[q] % 8 == 0;
         vec = vec && (uintptr_t)Ix % 8 == 0 && (uintptr_t)Iy % 8 == 0 && (uintptr_t)It % 8 == 0 && (uintptr_t)scratch % 8 == 0;
     }
     int launches = 0;
     for (int it = 0, step = 1; it < iters; it += step, ++launches) {
         step = 1;
-        if (tile) {
-            step = tile_step(params, tp.ni, it, iters);
-            // an even number of launches leaves the state in the caller's planes
-            if (it + step == iters && step > 1 && launches % 2 == 0) --step;
-        }
+        if (tile) step = iterate_step(params, tp, it, iters, launches);
         const bool check = params->tol > 0.0 && (it + step) % 10 == 0;
         IterArgs a{};
         a.g = g;
@@ -2047,6 +2066,8 @@ of_status iterate_common(of_fields f, const float *Ix, const float *Iy, const fl
             launch_cp(a, PREC_F32, PREC_F32, s);
         } else if (plain) {
             launch_admm_plain(a, s);
+        } else if (!tile) {
+            launch_admm_fused(a, PREC_F32, PREC_F32, s);
         } else {
             TileArgs t{};
             t.a = a;

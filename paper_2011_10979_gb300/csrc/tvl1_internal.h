@@ -320,6 +320,8 @@ TilePlan admm_tile_plan(Geom g, int ni, bool direct = false);
 // The tiling of n pairs' levels in one batched launch (gx: tiles in all).
 TilePlan admm_tile_plan_batch(const Geom *g, int n, int ni);
 int admm_tile_blocks(const TilePlan &p);  // partial-sum slots of a launch
+// Estimated microseconds of a launch of ni iterations (per-pixel a~: the kernel's frames are four rows per warp).
+float admm_tile_us(const TilePlan &p, int ni, bool per_pixel);
 // Tiles of one pair's level in a batched launch.
 inline int tile_cols(const TilePlan &p, Geom g) { return (g.W + p.ow - 1) / p.ow; }
 inline int tile_rows(const TilePlan &p, Geom g) { return (g.H + p.oh - 1) / p.oh; }

@@ -40,3 +40,29 @@ def test_unused_planes_are_left_alone(method, entry, beta, iters):
             assert torch.equal(planes[n], old[n]), n
         elif n in ("u", "v", "q11", "q22"):
             assert not torch.equal(planes[n], old[n]), n
+
+
+# Sizes and counts on either side of the rule that chooses between the tile kernel and the row-streaming one.
+@pytest.mark.parametrize("H,W", [(1, 1), (48, 64), (2, 9000), (3, 30000), (241, 323), (700, 900)])
+@pytest.mark.parametrize("kw", [dict(), dict(method=flow.OF_PADMM_II, rho=1.8), dict(beta=0.0), dict(a_tilde_mode=1)],
+                         ids=["I", "II", "beta0", "per-pixel"])
+def test_admm_iterations_in_one_call_equal_single_ones(H, W, kw):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    g = torch.Generator(device="cuda").manual_seed(H + W)
+    Ix, Iy, It = (0.2 * torch.randn(H, W, device="cuda", generator=g) for _ in range(3))
+    start = {n: torch.zeros(H, W, device="cuda") for n in PLANES[:10]}
+    P = flow.default_params(lam=2.0, **kw)
+    single = {n: t.clone() for n, t in start.items()}
+    done = 0
+    for iters in (2, 3, 5, 14):
+        while done < iters:
+            r1 = flow.of_admm_iterate(single, Ix, Iy, It, 0.5, P, 1)
+            done += 1
+        many = {n: t.clone() for n, t in start.items()}
+        r = flow.of_admm_iterate(many, Ix, Iy, It, 0.5, P, iters)
+        assert all(torch.equal(many[n], single[n]) for n in start), iters
+        assert r == pytest.approx(r1, rel=1e-5)
+        tested = {n: t.clone() for n, t in start.items()}
+        flow.of_admm_iterate(tested, Ix, Iy, It, 0.5, flow.default_params(lam=2.0, tol=1e-30, **kw), iters)
+        assert all(torch.equal(tested[n], single[n]) for n in start), iters
