@@ -1961,14 +1961,14 @@ int iterate_step(const of_params *p, const TilePlan &tp, int it, int iters, int 
 // 43 at 1920x1080).  Levels a few rows high are faster row by row (312 us against 518 for fifty iterations with a
 // per-pixel a~ at 30000x2), and so are one and two iterations at every size (a call of two: 89 us against 130 at
 // 1920x1080, 25 against 26.5 at 64x48).
-bool iterate_tile_of(const of_params *p, Geom g, const TilePlan &tp, int iters) {
+bool iterate_tile_of(const of_params *p, Geom g, const TilePlan &tp, int iters) {  // (more than two)
     float us = 0.f;
     for (int it = 0, launches = 0; it < iters; ++launches) {
         const int step = iterate_step(p, tp, it, iters, launches);
         us += std::max(4.1f, admm_tile_us(tp, step, p->a_tilde_mode == 1));
         it += step;
     }
-    return iters > 2 && us < iters * (4.5f + 1.87e-5f * (float)g.W * (float)g.H);
+    return us < iters * (4.5f + 1.87e-5f * (float)g.W * (float)g.H);
 }
 
 // Step-level iterations of one method family: KIND_ADMM (rpADMMI / rpADMMII), KIND_PDR, KIND_CP.
@@ -2016,8 +2016,9 @@ of_status iterate_common(of_fields f, const float *Ix, const float *Iy, const fl
     const bool plain = params->engine == OF_ENGINE_PLAIN;
     // ADMM, fused engines: the tile kernel straight from the caller's planes, several iterations per launch,
     // or the row-streaming kernel
-    const TilePlan tp = admm_tile_plan(g, params->tol > 0.0 ? TILE_ITERS : 0, true);
-    const bool tile = !xb && !plain && iterate_tile_of(params, g, tp, iters);
+    TilePlan tp;
+    if (!xb && !plain && iters > 2) tp = admm_tile_plan(g, params->tol > 0.0 ? TILE_ITERS : 0, true);
+    const bool tile = tp.R > 0 && iterate_tile_of(params, g, tp, iters);
     const int mb = fields_partial_slots(H, pitch);
     const int nb_used = pdr     ? pdr_plain_blocks(g)
                         : cp    ? cp_blocks(g)
