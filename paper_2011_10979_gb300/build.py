@@ -19,7 +19,7 @@ SOURCES = ["tvl1_api.cu", "tvl1_serve.cu", "tvl1_step.cu", "tvl1_noalloc.cu", "k
            "k_admm_cluster.cu",
            "k_pdr_regtile.cu", "k_pdr_regtile_f16.cu", "k_pdr_regtile_bf16.cu", "k_cp_tile.cu", "k_cp_tile_f16.cu", "k_cp_tile_bf16.cu"]
 HEADERS = ["tvl1_internal.h", "tvl1_device.cuh", "k_admm_roll.cuh", "k_admm_math.cuh", "k_pdr_math.cuh",
-           "k_cp_math.cuh", "k_cp_tile.cuh", "k_admm_cluster.cuh", "k_pdr_regtile.cuh", "k_admm_persist.cuh", "k_admm_tile.cuh", "k_pack2.cuh", "k_mbar.cuh", "tvl1_plan.h", "tvl1_device_once.h", "tvl1_step.h"]
+           "k_cp_math.cuh", "k_cp_tile.cuh", "k_admm_cluster.cuh", "k_pdr_regtile.cuh", "k_admm_persist.cuh", "k_admm_tile.cuh", "k_pack2.cuh", "k_mbar.cuh", "k_quot2.cuh", "tvl1_plan.h", "tvl1_device_once.h", "tvl1_step.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 

@@ -1047,6 +1047,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                             t.a = a;
                             tile_set_plan(t, tp, step);
                             t.timeout = &c.misc->timeout;
+                            t.tiny = &c.misc->tiny;
                             memcpy(t.maps, maps[par], sizeof(t.maps));
                             launch_pdr_regtile(t, prec, pflow, s);
                             last_nb = admm_tile_blocks(tp);

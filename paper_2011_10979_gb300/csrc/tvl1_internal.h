@@ -133,6 +133,7 @@ struct TileArgs {
     int *timeout;         // set when a bounded wait ran out (work-lists: the pairs' own flags)
     long long wait_ns = WAIT_NS;  // bound of every device-side wait
     int withhold = -1;    // self-test: the tile whose copies are never started
+    int *tiny;            // set when a tile needed the quotients' form for any numerator
     CUtensorMap maps[4];  // staged form, single pair: flow, dual and data planes, Xbar (pDR)
 };
 

@@ -46,6 +46,7 @@ struct Misc {
     long long iters;
     double res_check, res_final, energy, dual;
     int timeout;  // a bounded device-side wait ran out
+    int tiny;     // a tile has needed the quotients' form for any numerator (k_quot2.cuh)
 };
 static_assert(offsetof(Misc, ms_max) == offsetof(Misc, c_cur) + sizeof(float), "c_cur must precede ms_max");
 static_assert(offsetof(Misc, done) == offsetof(Misc, ms_max) + sizeof(float), "done must follow ms_max");
