@@ -14,12 +14,14 @@
 // stores round it (y^{k+1} when read as y, X and Xbar when written), so ni iterations here are bitwise
 // ni launches of k_cp.
 //
-// The primal step divides by |e|^2, a constant of the pixel: -rho / |e|^2 is formed from the correctly
-// rounded reciprocal with two remainder steps, the first of which makes the quotient faithful and the
-// second correctly rounded (Markstein, "Computation of elementary functions on the IBM RISC
-// System/6000 processor", IBM J. Res. Dev. 34, 1990), as long as neither the remainders nor the
-// quotient underflow: |e|^2 in (2^-100, 2^40) and |rho| = 0 or at least 2^-80, else the warp's
-// iteration divides.  So that this costs one branch per iteration and not one per row (a branch in a
+// The primal step divides by |e|^2, a constant of the pixel: by its reciprocal and remainder steps
+// (k_quot2.cuh).  A warp that holds a pixel whose |e|^2 is outside (2^-100, 2^40), or a numerator below 2^-80,
+// divides, and sets a flag by which the pair's later launches take a body of its own, whose quotients take any
+// numerator and pixels without data (beta = 0 on a flat region): images with flat regions have such numerators
+// wherever the illumination and the flow decay into them, and a launch is as slow as its slowest tile.  Measured
+// over a solve (three warps of 40 iterations, four levels), in brackets where every such warp divided, and the
+// kernel before this one: 640x480 with one half
+// flat 1.20 ms (2.08, 1.73), textured 0.97 (0.97, 1.51); 1920x1080 without beta, one half flat, 2.94 (2.64, 3.50).  So that this costs one branch per iteration and not one per row (a branch in a
 // row keeps the rows from overlapping: 2.8 against 1.5 us per iteration at R = 4), the primal step
 // first forms Z and rho of all rows, Z in the registers of the spent Xbar.
 //
@@ -34,6 +36,7 @@
 
 #include "k_cp_math.cuh"
 #include "k_pack2.cuh"
+#include "k_quot2.cuh"
 
 namespace tvl1 {
 
@@ -50,15 +53,17 @@ template <int R> struct Shared {
     pair2 bot[NW][3][32];   // y2 components of the bottom rows, read by the warp below
     pair2 ix[NW * R][32], iy[NW * R][32], it[NW * R][32], rc[NW * R][32];  // data and 1 / |e|^2 (each thread its own)
     double red[32];
+    int any, met;           // the pair takes the quotients' form for any numerator; the usual form had to divide
 };
 
 template <typename T, typename TF, bool HAS_W, int R> struct Kernel {
     static constexpr int C0 = HAS_W ? 0 : 1;
     using SH = Shared<R>;
 
-    // BX, BY: as the ADMM tile kernel's.
-    template <int BX, bool BY>
-    static __device__ __forceinline__ void body(const TileArgs &A, SH &G, int bx, int by, int lane, int wid) {
+    // BX, BY: as the ADMM tile kernel's.  ANY: the quotients' form for any numerator, with divisions where the divisors
+    // need them.  False (the usual form only): the pair takes the other form; nothing is stored.
+    template <int BX, bool BY, bool ANY>
+    static __device__ __forceinline__ bool body(const TileArgs &A, SH &G, int bx, int by, int lane, int wid) {
         const int H = A.a.g.H, W = A.a.g.W, P = A.a.g.pitch;
         const int c = bx * A.ow - A.offx + 2 * lane, ib = by * A.oh - A.offy + wid * R;
         const unsigned me0 = mask_of(c >= 0 && c < W - 1), me1 = mask_of(c + 1 >= 0 && c + 1 < W - 1);
@@ -66,7 +71,9 @@ template <typename T, typename TF, bool HAS_W, int R> struct Kernel {
         pair2 y[R][6], X[R][3], B[R][3];
         const float beta = A.a.k.beta, lam = A.a.k.lambda, sg = A.a.k.cp_sigma, sl0 = sg * lam;
         const pair2 tau2 = bc2(A.a.k.cp_tau), sg2 = bc2(sg), beta2 = bc2(beta), bb2 = bc2(beta * beta), sl02 = bc2(sl0);
-        bool odd = !(sl0 < 0x1p20f);  // quotients outside the fast division's range
+        // (set by another block of this launch, either will do; stored behind the frame's loads)
+        const int any = !ANY && threadIdx.x == 0 && A.tiny ? *(const volatile int *)A.tiny : 0;
+        bool odd = !(sl0 < 0x1p20f);  // quotients outside the range of the reciprocal's
         {
             const int c0 = BX ? min(max(c, 0), W - 1) : c, c1 = BX ? min(max(c + 1, 0), W - 1) : c + 1;
             auto load = [&](auto VEC_) {
@@ -104,11 +111,10 @@ template <typename T, typename TF, bool HAS_W, int R> struct Kernel {
                     const pair2 ix = LT(A.a.Ix), iy = LT(A.a.Iy);
                     G.ix[wid * R + r][lane] = ix;
                     G.iy[wid * R + r][lane] = iy;
-                    G.it[wid * R + r][lane] = LT(A.a.It);
-                    float e0, e1;
-                    upk(fma2(iy, iy, fma2(ix, ix, bb2)), e0, e1);
-                    odd = odd || !(fminf(e0, e1) > 0x1p-100f && fmaxf(e0, e1) < 0x1p40f);
-                    G.rc[wid * R + r][lane] = pk(__frcp_rn(e0), __frcp_rn(e1));
+                    const pair2 it = LT(A.a.It), e2 = fma2(iy, iy, fma2(ix, ix, bb2));
+                    G.it[wid * R + r][lane] = it;
+                    odd = odd || prox_unusual(e2);
+                    G.rc[wid * R + r][lane] = pk(__frcp_rn(lo2(e2)), __frcp_rn(hi2(e2)));
                 }
             };
             if (BX < 2 || A.vec) load(std::true_type{});
@@ -120,8 +126,23 @@ template <typename T, typename TF, bool HAS_W, int R> struct Kernel {
                 for (int k = C0; k < 3; ++k) G.top[wid][k][lane] = B[0][k];
         };
         put_top();
+        if (threadIdx.x == 0) {
+            G.met = 0;
+            G.any = any;
+        }
         odd = __syncthreads_or(odd);
+        if (!ANY && G.any) return false;
         float res = 0.f;
+        if (ANY && odd) {  // by what: a pixel without data takes a zero reciprocal
+            bool bad = !(sl0 < 0x1p20f);
+#pragma unroll 1
+            for (int r = 0; r < R; ++r) {
+                const pair2 ix = G.ix[wid * R + r][lane], iy = G.iy[wid * R + r][lane], e2 = fma2(iy, iy, fma2(ix, ix, bb2));
+                bad = bad || !prox_empty(e2, ix, iy, G.it[wid * R + r][lane], beta);
+                G.rc[wid * R + r][lane] = prox_rcp2(e2);
+            }
+            odd = __any_sync(FULL, bad);
+        }
 #pragma unroll 1
         for (int kk = 0; kk < A.ni; ++kk) {
             const bool last = kk == A.ni - 1;
@@ -199,27 +220,9 @@ template <typename T, typename TF, bool HAS_W, int R> struct Kernel {
                 for (int r = 0; r < R; ++r) {
                     const pair2 ix = G.ix[wid * R + r][lane], iy = G.iy[wid * R + r][lane];
                     const pair2 e2 = fma2(iy, iy, fma2(ix, ix, bb2));
-                    float r0, r1, s0, s1, q0, q1;
-                    upk(rho[r], r0, r1);
-                    upk(mul2(sl02, e2), s0, s1);
-                    if (SLOW) {
-                        float e0, e1;
-                        upk(e2, e0, e1);
-                        q0 = e0 <= 0.f ? 0.f : r0 < -s0 ? sl0 : r0 > s0 ? -sl0 : -r0 / e0;
-                        q1 = e1 <= 0.f ? 0.f : r1 < -s1 ? sl0 : r1 > s1 ? -sl0 : -r1 / e1;
-                    } else {  // |t| first, then the sign of -rho
-                        const pair2 rc = G.rc[wid * R + r][lane], ne = neg2(e2);
-                        pair2 q = mul2(rho[r], rc);
-                        q = fma2(fma2(ne, q, rho[r]), rc, q);
-                        q = fma2(fma2(ne, q, rho[r]), rc, q);
-                        upk(q, q0, q1);
-                        auto sgn = [](float m, float x) {
-                            return __uint_as_float((__float_as_uint(m) & 0x7fffffffu) | (~__float_as_uint(x) & 0x80000000u));
-                        };
-                        q0 = sgn(fabsf(r0) > s0 ? sl0 : q0, r0);
-                        q1 = sgn(fabsf(r1) > s1 ? sl0 : q1, r1);
-                    }
-                    const pair2 t = pk(q0, q1);
+                    const pair2 thr = mul2(sl02, e2);
+                    const pair2 t = SLOW ? prox_div2(rho[r], e2, thr, sl0)
+                                         : prox_quot2<ANY>(rho[r], e2, G.rc[wid * R + r][lane], thr, sl0);
                     pair2 z[3] = {0ull, fma2(t, ix, B[r][1]), fma2(t, iy, B[r][2])};
                     if (HAS_W) z[0] = fma2(t, beta2, B[r][0]);
                     if (last && A.a.partials) {
@@ -239,8 +242,12 @@ template <typename T, typename TF, bool HAS_W, int R> struct Kernel {
                     }
                 }
             };
-            if (__any_sync(FULL, odd || small < 2 * 0x17800000u)) finish(std::true_type{});  // |rho| < 2^-80
-            else finish(std::false_type{});
+            if (__any_sync(FULL, odd || (!ANY && small < QUOT_SMALL_BITS))) {
+                if (!ANY) G.met = 1;
+                finish(std::true_type{});
+            } else {
+                finish(std::false_type{});
+            }
             if (!last) put_top();
         }
         // ---- store the tile
@@ -274,6 +281,7 @@ template <typename T, typename TF, bool HAS_W, int R> struct Kernel {
             const double tot = block_sum((double)res, G.red);
             if (threadIdx.x == 0) A.a.partials[blockIdx.x] = tot;
         }
+        return true;
     }
 
     static __device__ __forceinline__ void run(const TileArgs &A) {
@@ -283,14 +291,18 @@ template <typename T, typename TF, bool HAS_W, int R> struct Kernel {
         const int lane = threadIdx.x & 31, wid = __shfl_sync(FULL, threadIdx.x >> 5, 0);
         const int bx = blockIdx.x % A.gx, by = blockIdx.x / A.gx;
         const int fj = bx * A.ow - A.offx, fi = by * A.oh - A.offy;
+        bool ok;
         if (fj >= 1 && fj + 64 <= A.a.g.W - 1 && A.vec) {
-            if (fi >= 1 && fi + R * NW <= A.a.g.H - 1) body<0, false>(A, G, bx, by, lane, wid);
-            else body<0, true>(A, G, bx, by, lane, wid);
+            if (fi >= 1 && fi + R * NW <= A.a.g.H - 1) ok = body<0, false, false>(A, G, bx, by, lane, wid);
+            else ok = body<0, true, false>(A, G, bx, by, lane, wid);
         } else if (A.a.g.W % 2 == 0 && A.vec) {
-            body<1, true>(A, G, bx, by, lane, wid);
+            ok = body<1, true, false>(A, G, bx, by, lane, wid);
         } else {
-            body<2, true>(A, G, bx, by, lane, wid);
+            ok = body<2, true, false>(A, G, bx, by, lane, wid);
         }
+        // (a second body of the other form, for tiles inside the image, made the usual one 1% slower)
+        if (!ok) body<2, true, true>(A, G, bx, by, lane, wid);
+        else if (lane == 0 && *(volatile int *)&G.met && A.tiny) *A.tiny = 1;  // the pair's next launches take the other form
     }
 };
 

@@ -1062,6 +1062,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                             t.a = a;
                             tile_set_plan(t, tp, step);
                             t.vec = 1;
+                            t.tiny = &c.misc->tiny;
                             launch_cp_tile(t, prec, pflow, s);
                             last_nb = admm_tile_blocks(tp);
                         } else {

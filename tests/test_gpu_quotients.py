@@ -1,4 +1,4 @@
-"""The quotients of the register kernels on images with regions without data: beside textured pixels the
+"""The quotients of the ALG1 and pDR register kernels on images with regions without data: beside textured pixels the
 flow and the illumination decay through every magnitude to zero, pixels without any gradient have no divisor, and
 clipped images mix both in every warp.  Against the kernels that divide, for equality."""
 import numpy as np
@@ -32,6 +32,17 @@ def images(H, W, kind):
     elif kind == "faint":  # quotients that are subnormal from the first iteration
         I *= np.float32(1e-36)
     return [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in I]
+
+
+@pytest.mark.parametrize("kind", ["box", "half", "clipped", "faint"])
+@pytest.mark.parametrize("beta", [0.05, 0.0])
+@pytest.mark.parametrize("H,W", [(260, 350), (203, 301)])
+def test_alg1(ctx, kind, beta, H, W):
+    im = images(H, W, kind)
+    kw = dict(method=flow.OF_CP, lam=3.0, beta=beta, levels=1, warps=2, iters=70, engine=flow.OF_ENGINE_STREAM)
+    a = flow.of_solve(ctx, *im, flow.default_params(rows_per_warp=8, **kw), want_w=True)
+    b = flow.of_solve(ctx, *im, flow.default_params(**kw), want_w=True)
+    assert all(torch.equal(x, y) for x, y in zip(a[:3], b[:3]))
 
 
 @pytest.mark.parametrize("kind", ["box", "half", "clipped", "faint"])
