@@ -60,6 +60,11 @@ TilePlan admm_tile_plan(Geom g, int ni, bool direct) {
     return best;
 }
 
+TilePlan admm_tile_plan_tested(Geom g, bool direct) {
+    const TilePlan a = admm_tile_plan(g, TILE_ITERS, direct), b = admm_tile_plan(g, TILE_TEST_ITERS, direct);
+    return 2 * plan_us(b) < 3 * plan_us(a) + plan_us(a, a.R, 1) ? b : a;
+}
+
 // Batches run the staged form; the iterations per launch that cost the least over all pairs' tiles.
 TilePlan admm_tile_plan_batch(const Geom *g, int n, int ni) {
     TilePlan best;

@@ -20,10 +20,10 @@
 // numerator and pixels without data (beta = 0 on a flat region): images with flat regions have such numerators
 // wherever the illumination and the flow decay into them, and a launch is as slow as its slowest tile.  Measured
 // over a solve (three warps of 40 iterations, four levels), in brackets where every such warp divided, and the
-// kernel before this one: 640x480 with one half
-// flat 1.20 ms (2.08, 1.73), textured 0.97 (0.97, 1.51); 1920x1080 without beta, one half flat, 2.94 (2.64, 3.50).  So that this costs one branch per iteration and not one per row (a branch in a
-// row keeps the rows from overlapping: 2.8 against 1.5 us per iteration at R = 4), the primal step
-// first forms Z and rho of all rows, Z in the registers of the spent Xbar.
+// kernel before this one: 640x480 with one half flat 1.20 ms (2.08, 1.73), textured 0.97 (0.97, 1.51); 1920x1080
+// without beta, one half flat, 2.94 (2.64, 3.50).  So that this costs one branch per iteration and not one per
+// row (a branch in a row keeps the rows from overlapping: 2.8 against 1.5 us per iteration at R = 4), the primal
+// step first forms Z and rho of all rows, Z in the registers of the spent Xbar.
 //
 // Bound by latency and issue with three warps per SM quarter (some 240 clocks per row and warp), beside
 // 4 to 6 us per launch for instruction fetch and the state's loads and stores.  Measured per iteration,

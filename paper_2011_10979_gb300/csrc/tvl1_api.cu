@@ -70,8 +70,9 @@ Plan make_plan(int H, int W, const of_params *p) {
         mb = std::max({mb, admm_fused_blocks(g, p->rows_per_warp != 0 ? 1 : 0), admm_plain_blocks(g),
                        pdr_plain_blocks(g, PARTIAL_ROWS_MIN), cp_blocks(g, PARTIAL_ROWS_MIN), energy_blocks(g),
                        adapt_blocks(g), pdr_tile_blocks(g)});
-        for (int q = 0; q < 4; ++q) mb = std::max(mb, admm_tile_blocks(admm_tile_plan(g, q & 1 ? TILE_ITERS : 0, q & 2)));
-        for (int q = 0; q < 2; ++q) mb = std::max(mb, admm_tile_blocks(cp_tile_plan(g, q ? TILE_ITERS : 0)));
+        for (int ni : {0, TILE_ITERS, TILE_TEST_ITERS})
+            mb = std::max({mb, admm_tile_blocks(admm_tile_plan(g, ni)), admm_tile_blocks(admm_tile_plan(g, ni, true)),
+                           admm_tile_blocks(cp_tile_plan(g, ni))});
         mb = std::max(mb, admm_tile_blocks(pdr_regtile_plan(g, std::max(p->iters, 1))));
     }
     pl.max_blocks = mb;
@@ -116,7 +117,7 @@ int tile_step(const of_params *p, int ni, int it, int iters) {
     int step = std::min(ni, iters - it);
     if (p->tol > 0.0) {
         step = std::min(step, 10 - it % 10);
-        if (step > 1 && it + step == iters) --step;
+        if (ni == TILE_ITERS && step > 1 && it + step == iters) --step;
     }
     return step;
 }
@@ -349,10 +350,17 @@ bool cp_tile_of(const of_params *p, bool batched) {
            (p->engine == OF_ENGINE_FUSED || p->engine == OF_ENGINE_STREAM);
 }
 
-// Levels up to this many pixels run ALG1 level-resident when its tile kernel is the alternative
-// (measured per iteration, resident against tile kernel: 1.03 / 1.09 us at 40x30, 1.14 / 1.09 at 64x48,
-// 1.21 / 1.10 at 80x60, 1.78 / 1.09 at 120x90, 2.39 / 1.12 at 160x120).
-constexpr long CP_TILE_RESIDENT_MAX_PX = 2000;
+// Whether a level runs ALG1 level-resident when its tile kernel is the alternative (measured per iteration,
+// resident against tile kernel: 1.03 / 1.09 us at 40x30, 1.14 / 1.09 at 64x48, 1.21 / 1.10 at 80x60, 1.78 / 1.09 at
+// 120x90, 2.39 / 1.12 at 160x120): up to 2,000 px, and up to 6,000 with the stopping test, whose launches are
+// shorter (ten iterations at 80x60: 18 us / 25), and where the level is a strip of too many tiles (1x4096: 1.4 / 2.3).
+bool cp_resident_preferred(const of_params *p, Geom g) {
+    const long px = (long)g.H * g.W;
+    if (px <= 2000 || px > 6000) return px <= 2000;
+    if (p->tol > 0.0) return true;
+    const TilePlan t = cp_tile_plan(g, 0);
+    return cp_tile_us(t, t.ni) > 1.3f * t.ni;
+}
 
 // A single pair's level runs the ADMM methods level-resident wherever the register-resident cluster
 // form holds it (k_admm_cluster.cuh; measured per iteration, against the several-iterations tile kernel:
@@ -368,7 +376,7 @@ bool use_resident(const of_params *p, Geom g, bool batched = false) {
     if (pdr_tile_of(p)) return (long)g.H * g.W <= PDR_TILE_RESIDENT_MAX_PX;
     if (admm_tile_of(p) && !batched)
         return (long)g.H * g.W <= TILE_RESIDENT_MAX_PX || admm_cluster_plan(g, admm_resident_cluster(), nullptr);
-    if (cp_tile_of(p, batched)) return (long)g.H * g.W <= CP_TILE_RESIDENT_MAX_PX;
+    if (cp_tile_of(p, batched)) return cp_resident_preferred(p, g);
     return admm_resident_preferred(g, p->method);
 }
 
@@ -922,16 +930,22 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
             const bool tile = !B.pers[l] && (batched ? B.tp[l].R > 0 : !res1 && admm_tile_of(p));
             const bool cptile = !B.pers[l] && !res1 && cp_tile_of(p, batched);
             TilePlan tp = B.tp[l];
-            if (cptile) tp = cp_tile_plan(geom_of(*pc[0].pl, l), tile_iters_of(p, rest));
+            if (cptile) {
+                const Geom g = geom_of(*pc[0].pl, l);
+                tp = p->tol > 0.0 ? cp_tile_plan_tested(g) : cp_tile_plan(g, tile_iters_of(p, rest));
+            }
             CUtensorMap maps[2][4];
             if (tile && !batched) {
                 const PairCtx &c = pc[0];
                 const Geom g = geom_of(*c.pl, l);
-                tp = admm_tile_plan(g, tile_iters_of(p, rest));
+                auto plan = [&](bool direct) {
+                    return p->tol > 0.0 ? admm_tile_plan_tested(g, direct) : admm_tile_plan(g, tile_iters_of(p, rest), direct);
+                };
+                tp = plan(false);
                 bool ok = true;
                 for (int b = 0; b < 2 && tp.staged; ++b)
                     ok = ok && tile_encode_maps(maps[b], bufs_of(c)[b], data_of(c)[0], data_of(c)[1], g, prec, pflow, has_w);
-                if (!ok) tp = admm_tile_plan(g, tile_iters_of(p, rest), true);
+                if (!ok) tp = plan(true);
             }
             // a single pair's streamed pDR level (k_pdr_regtile.cuh), where the driver encodes its maps
             bool pdrreg = pdr_tile && !batched && !res1 && rest > 0 && (long)pc[0].pl->H[l] * pc[0].pl->W[l] >= PDR_REGTILE_MIN_PX;
@@ -1017,6 +1031,8 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
             // pairs left for the streamed launches: the tile work-list (ADMM), all pairs (pDR),
             // the non-resident pairs (ALG1)
             const bool streamed = !persl && (batched ? ((cp || pdr) ? B.nres[l] < n : B.ntiles[l] > 0) : !res1);
+            // ALG1: a single iteration runs on k_cp, unless the tested launches are the tile kernel's
+            auto cp_on_tile = [&](int step) { return step > 1 || (cptile && p->tol > 0.0 && tp.ni > TILE_ITERS); };
             int par = start2, last_nb = 0;  // the buffer parity and the last launch's block count
             for (int it = 0, q = 0, step = 1; streamed && it < rest; it += step) {
                 step = steps[q++];
@@ -1057,7 +1073,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                             launch_pdr_fused(a, prec, pflow, s);
                         }
                     } else if (cp) {
-                        if (step > 1) {
+                        if (cp_on_tile(step)) {
                             TileArgs t{};
                             t.a = a;
                             tile_set_plan(t, tp, step);
@@ -1084,7 +1100,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                         last_nb = blocks_of(g, l);
                     }
                     if (check) {
-                        const int nb = tile || pdrreg || (cp && step > 1) ? admm_tile_blocks(tp) : blocks_of(g, l);
+                        const int nb = tile || pdrreg || (cp && cp_on_tile(step)) ? admm_tile_blocks(tp) : blocks_of(g, l);
                         const double rows = (double)g.H * g.W * (has_w ? 3.0 : 2.0);
                         launch_reduce_check(c.partials, nb, &c.misc->res_check, rows, p->tol, &c.misc->done,
                                             &c.misc->iters, 10, s);

@@ -114,6 +114,8 @@ constexpr int TILE_WARPS = 12, TILE_SMS = 152, TILE_MAX_ITERS = 8;
 constexpr int TILE_STAGED_HEIGHT = 48;
 // Iterations per launch where the number is fixed.
 constexpr int TILE_ITERS = 3;
+// Iterations per launch with the stopping test where two launches per test are the faster ones.
+constexpr int TILE_TEST_ITERS = 5;
 
 // A level's tiling: ni iterations of halo around tiles of ow x oh pixels whose output starts offx
 // columns and offy rows into their frames; gx x gy tiles.
@@ -318,6 +320,10 @@ void launch_parity_fix(const Fields &from, const Fields &to, Geom g, int prec, i
 // The tiling of a single pair's level for launches of ni iterations (0: the rule's choice); direct:
 // without the staged form, which needs the library's own planes.
 TilePlan admm_tile_plan(Geom g, int ni, bool direct = false);
+// The tiling for a single pair's launches with the stopping test: ten iterations, the last tested, take an even number of
+// launches, 3, 3, 3 and 1 or 5 and 5, whichever is estimated to be faster (38.2 against 39.6 us at 640x480, 23.9
+// against 16.7 at 160x120).
+TilePlan admm_tile_plan_tested(Geom g, bool direct = false);
 // The tiling of n pairs' levels in one batched launch (gx: tiles in all).
 TilePlan admm_tile_plan_batch(const Geom *g, int n, int ni);
 int admm_tile_blocks(const TilePlan &p);  // partial-sum slots of a launch
@@ -337,6 +343,8 @@ void launch_admm_tile(const TileArgs &a, int prec, int prec_flow, cudaStream_t s
 // Single pair: a.ni consecutive iterations of k_cp in one launch, reading a.a.in and writing a.a.out,
 // bitwise ni launches of the one-iteration kernel; partials of the last iteration, one slot per tile.
 TilePlan cp_tile_plan(Geom g, int ni);
+TilePlan cp_tile_plan_tested(Geom g);  // as admm_tile_plan_tested; the single launch is k_cp's
+float cp_tile_us(const TilePlan &p, int k);  // estimated microseconds of a launch of k iterations
 void launch_cp_tile(const TileArgs &a, int prec, int prec_flow, cudaStream_t s);
 
 // Single pair, gs_sweeps = 1: a.ni consecutive iterations of pDR in one launch, reading a.a.in through

@@ -69,10 +69,10 @@ bool batch_tile_of(const of_params *p, bool maps);
 int tile_iters_of(const of_params *p, int iters);
 
 // Iterations of the launch that starts after `it` of a warp's `iters` iterations, at most ni.  With the
-// stopping test every ten iterations run as launches of 3, 3, 3 and 1: an even number of launches
-// leaves the tested state in the buffer the warp started from, as on the one-launch-per-iteration
-// path, and the warp's last launch is a single iteration, so that the final residual sums the same
-// partials whether or not the test stopped the warp.
+// stopping test every ten iterations run as launches of 3, 3, 3 and 1, or of 5 and 5 (ni = TILE_TEST_ITERS): an
+// even number of launches leaves the tested state in the buffer the warp started from, as on the
+// one-launch-per-iteration path.  With three, the warp's last launch is a single iteration (ALG1 runs those on k_cp,
+// and the final residual has to sum the same kernel's partials whether or not the test stopped the warp).
 int tile_step(const of_params *p, int ni, int it, int iters);
 
 // The 13 planes of a state buffer at `base`, `plane` bytes apart.

@@ -70,3 +70,21 @@ def test_batches_of_more_tiles_than_blocks(ctx, kind):
             assert torch.equal(u, us[k]) and torch.equal(v, vs[k]), BATCH[k]
             counts.add(s["iters_run"])
         assert len(counts) == (1 if tol == 0.0 else len(counts)) and (tol == 0.0 or len(counts) > 1)
+
+
+# The stopping test's launches, 5 and 5 or 3, 3, 3 and 1 per ten iterations, with remainders of one to nine iterations.
+@pytest.mark.parametrize("H,W", [(120, 160), (80, 107), (150, 201), (3, 4000), (4000, 2), (240, 320), (375, 1242)])
+@pytest.mark.parametrize("method,pinned", [(flow.OF_PADMM_I, 8), (flow.OF_PADMM_II, 8), (flow.OF_CP, 8)])
+@pytest.mark.parametrize("prec", [0, 2])
+def test_single_pairs_with_the_stopping_test(ctx, H, W, method, pinned, prec):
+    im = images(H, W) if min(H, W) > 8 else [cu(a) for a in np.random.default_rng(H).random((2, H, W))]
+    kw = dict(method=method, lam=3.0, levels=1, precision=prec, fp32_last_warp=0)
+    ref = dict(kw, engine=flow.OF_ENGINE_STREAM, rows_per_warp=pinned)
+    met = flow.of_solve(ctx, *im, flow.default_params(warps=1, iters=20, **ref))[3]["residual"] * 1.001
+    for iters in (20, 21, 25, 39):
+        for tol in (met, 1e-30):
+            a = flow.of_solve(ctx, *im, flow.default_params(warps=2, iters=iters, tol=tol, **ref), want_w=True)
+            b = flow.of_solve(ctx, *im, flow.default_params(warps=2, iters=iters, tol=tol, **kw), want_w=True)
+            assert all(torch.equal(x, y) for x, y in zip(a[:3], b[:3])), (iters, tol)
+            assert a[3]["iters_run"] == b[3]["iters_run"]
+            assert a[3]["residual"] == pytest.approx(b[3]["residual"], rel=1e-5)
