@@ -4,6 +4,13 @@
 
 namespace tvl1 {
 
+// Microseconds of a launch of k iterations, fitted to launches of one round: 640x480, one iteration, 10.8 us;
+// 320x240, five, 21.6.
+float pdr_regtile_us(const TilePlan &p, int k) {
+    const int rounds = (p.gx * p.gy + TILE_SMS - 1) / TILE_SMS;
+    return 0.4f + rounds * (7.7f + 2.7f * k);
+}
+
 // The tiling of a level into frames of 64 x TILE_STAGED_HEIGHT with the least estimated time per iteration:
 // an iteration takes three pixels of halo on every side and one more on the east and south.  Frames
 // start at multiples of four columns (16-byte aligned copies) and of two rows (a row's colours).
@@ -20,9 +27,7 @@ TilePlan pdr_regtile_plan(Geom g, int max_ni) {
         p.oh = (TILE_STAGED_HEIGHT - p.offy - (3 * k + 1)) / 2 * 2;
         p.gx = (g.W + p.ow - 1) / p.ow;
         p.gy = (g.H + p.oh - 1) / p.oh;
-        // fitted to launches of one round: 640x480, one iteration, 10.8 us; 320x240, five, 21.6
-        const int rounds = (p.gx * p.gy + TILE_SMS - 1) / TILE_SMS;
-        const float t = (0.4f + rounds * (7.7f + 2.7f * k)) / k;
+        const float t = pdr_regtile_us(p, k) / k;
         if (us == 0.f || t < us) {
             us = t;
             best = p;

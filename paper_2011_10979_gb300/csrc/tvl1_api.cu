@@ -325,10 +325,27 @@ std::vector<int> pdr_launches(int ni, int iters, bool tested, bool last_warp) {
     return v;
 }
 
-// Levels from this many pixels run a single pair's pDR on the register tile kernel (k_pdr_regtile.cuh), smaller
-// ones on the one-iteration tile kernel of k_pdr.cu (measured per iteration, register tiles against it: 4.5 / 4.4
-// us at 213x160, 4.2 / 5.6 at 240x180, 4.3 / 5.8 at 320x240).
-constexpr long PDR_REGTILE_MIN_PX = 40000;
+// Whether a single pair's streamed pDR level runs on the register tile kernel (k_pdr_regtile.cuh) rather than on the
+// one-iteration tile kernel of k_pdr.cu.  Levels from 40,000 pixels (measured per iteration, register tiles
+// against it: 4.5 / 4.4 us at 213x160, 4.2 / 5.6 at 240x180, 4.3 / 5.8 at 320x240), with the stopping test, whose
+// tested iterations are launches of their own, from 60,000 but for strips (7.0 / 6.5 at 201x200), where the
+// estimated time is the smaller: the one-iteration kernel takes some 6.2 us per wave of 32 x 32 tiles over the SMs, less on strips that
+// leave most of a tile's rows outside the image (20000x2: 15.4 / 13.2 us; 32768x8: 23.7 / 20.9; 5000x8: 4.8 / 7.0),
+// and the register tiles a quarter more than estimated on strips narrower than a few lanes (11x4000: 6.7 / 6.2).
+bool pdr_regtile_of(const of_params *p, Geom g, const TilePlan &tp) {
+    const bool tested = p->tol > 0.0;
+    const bool strip = std::min(g.H, g.W) < 32;
+    if ((long)g.H * g.W < (tested && !strip ? 60000 : 40000)) return false;
+    float us = 0.f;
+    int iters = 0;
+    for (int k : pdr_launches(tp.ni, tested ? 10 : tp.ni, tested, false)) {
+        us += pdr_regtile_us(tp, k);
+        iters += k;
+    }
+    if (g.W < 16) us *= 1.25f;
+    const int waves = (((g.W + 31) / 32) * ((g.H + 31) / 32) + TILE_SMS - 1) / TILE_SMS;
+    return us < iters * (g.H < 16 ? 3.2f + 2.2f * waves : 6.2f * waves);
+}
 
 // Levels up to this many pixels run pDR level-resident when its one-launch tile kernel is the
 // alternative (measured per iteration, resident against tile kernel: 2.3 / 4.0 us at 40x30,
@@ -948,11 +965,12 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                 if (!ok) tp = plan(true);
             }
             // a single pair's streamed pDR level (k_pdr_regtile.cuh), where the driver encodes its maps
-            bool pdrreg = pdr_tile && !batched && !res1 && rest > 0 && (long)pc[0].pl->H[l] * pc[0].pl->W[l] >= PDR_REGTILE_MIN_PX;
+            bool pdrreg = pdr_tile && !batched && !res1 && rest > 0;
             if (pdrreg) {
                 const PairCtx &c = pc[0];
                 const Geom g = geom_of(*c.pl, l);
                 tp = pdr_regtile_plan(g, rest);
+                pdrreg = pdr_regtile_of(p, g, tp);
                 for (int b = 0; b < 2; ++b)
                     pdrreg = pdrreg && tile_encode_maps(maps[b], bufs_of(c)[b], data_of(c)[0], data_of(c)[1], g, prec, pflow, has_w, true);
             }

@@ -351,6 +351,7 @@ void launch_cp_tile(const TileArgs &a, int prec, int prec_flow, cudaStream_t s);
 // a.maps and writing a.a.out, bitwise ni launches of the one-launch kernel of k_pdr.cu; partials only
 // with one iteration, one slot per tile.
 TilePlan pdr_regtile_plan(Geom g, int max_ni);
+float pdr_regtile_us(const TilePlan &p, int k);  // estimated microseconds of a launch of k iterations
 void launch_pdr_regtile(const TileArgs &a, int prec, int prec_flow, cudaStream_t s);
 
 // ---------------------------------------------------------------- adaptive ADMM step (k_adapt.cu)

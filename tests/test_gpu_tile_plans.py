@@ -88,3 +88,16 @@ def test_single_pairs_with_the_stopping_test(ctx, H, W, method, pinned, prec):
             assert all(torch.equal(x, y) for x, y in zip(a[:3], b[:3])), (iters, tol)
             assert a[3]["iters_run"] == b[3]["iters_run"]
             assert a[3]["residual"] == pytest.approx(b[3]["residual"], rel=1e-5)
+
+
+# pDR's register tiles and one-iteration tiles on either side of the rule that chooses: strips, odd widths near its
+# smallest level, with and without the stopping test.
+@pytest.mark.parametrize("H,W", [(2, 20000), (3, 32768), (8, 5000), (5000, 8), (4000, 11), (200, 201), (240, 320)])
+@pytest.mark.parametrize("tol", [0.0, 1e-30])
+def test_pdr_on_either_tile_kernel(ctx, H, W, tol):
+    im = images(H, W) if min(H, W) > 8 else [cu(a) for a in np.random.default_rng(H).random((2, H, W))]
+    P = flow.default_params(method=flow.OF_PDR, lam=3.0, levels=1, warps=2, iters=23, tol=tol, engine=flow.OF_ENGINE_STREAM)
+    u, v, _, st = flow.of_solve(ctx, *im, P)
+    ub, vb, sb = flow.of_solve_batch(ctx, [im[0]] * 2, [im[1]] * 2, P)  # one iteration per launch
+    assert torch.equal(u, ub[0]) and torch.equal(v, vb[0])
+    assert st["iters_run"] == sb[0]["iters_run"]
