@@ -446,22 +446,38 @@ void launch_derivatives(const float *I, Geom g, float *Ix, float *Iy, cudaStream
 
 namespace {
 
-dim3 grid_of(const PairSet &a) {
+// f(first pair, grid) for every launch over the pairs of a set: a grid holds 65,535 in its third dimension.
+template <typename F> void over_pairs(const PairSet &a, F f) {
     dim3 d = grid2(a.pairs ? a.grid.H : a.one.g.H, a.pairs ? a.grid.W : a.one.g.W);
-    d.z = a.pairs ? a.n : 1;
-    return d;
+    const int n = a.pairs ? a.n : 1;
+    for (int k = 0; k < n; k += 65535) {
+        d.z = std::min(n - k, 65535);
+        f(k, d);
+    }
+}
+PairSet from_pair(PairSet a, int k) {
+    if (a.pairs) a.pairs += k;
+    return a;
 }
 
 }  // namespace
 
 void launch_level_begin(const LevelArgs &a, int prec_dual, int prec_flow, cudaStream_t s) {
-    TVL1_DISPATCH_PREC(prec_dual, TD, TVL1_DISPATCH_PREC(prec_flow, TF,
-                       k_level_begin<TD, TF><<<grid_of(a.fine), dim3(B2X, B2Y), 0, s>>>(a)));
+    over_pairs(a.fine, [&](int k, dim3 grid) {
+        LevelArgs b = a;
+        b.fine = from_pair(a.fine, k);
+        b.coarse = from_pair(a.coarse, k);
+        TVL1_DISPATCH_PREC(prec_dual, TD, TVL1_DISPATCH_PREC(prec_flow, TF,
+                           k_level_begin<TD, TF><<<grid, dim3(B2X, B2Y), 0, s>>>(b)));
+    });
 }
 
 void launch_warp(const PairSet &a, int cur, float beta, int prec, int prec_flow, cudaStream_t s) {
-    TVL1_DISPATCH_PREC(prec, T, TVL1_DISPATCH_PREC(prec_flow, TF,
-                       k_warp<T, TF><<<grid_of(a), dim3(B2X, B2Y), 0, s>>>(a, cur, beta)));
+    over_pairs(a, [&](int k, dim3 grid) {
+        const PairSet b = from_pair(a, k);
+        TVL1_DISPATCH_PREC(prec, T, TVL1_DISPATCH_PREC(prec_flow, TF,
+                           k_warp<T, TF><<<grid, dim3(B2X, B2Y), 0, s>>>(b, cur, beta)));
+    });
 }
 
 void launch_warp_reset(const PairSet &a, cudaStream_t s) {
@@ -472,8 +488,11 @@ void launch_warp_reset(const PairSet &a, cudaStream_t s) {
 
 void launch_state_to_f32(const PairSet &from, const PairSet &to, int cur, int xbar, int has_w, int prec_dual,
                          int prec_flow, cudaStream_t s) {
-    TVL1_DISPATCH_PREC(prec_dual, TD, TVL1_DISPATCH_PREC(prec_flow, TF,
-                       k_state_to_f32<TD, TF><<<grid_of(from), dim3(B2X, B2Y), 0, s>>>(from, to, cur, xbar, has_w)));
+    over_pairs(from, [&](int k, dim3 grid) {
+        const PairSet f = from_pair(from, k), t = from_pair(to, k);
+        TVL1_DISPATCH_PREC(prec_dual, TD, TVL1_DISPATCH_PREC(prec_flow, TF,
+                           k_state_to_f32<TD, TF><<<grid, dim3(B2X, B2Y), 0, s>>>(f, t, cur, xbar, has_w)));
+    });
 }
 
 void launch_output(const Fields &f, Geom g, float *u, float *v, float *w, int prec_flow, cudaStream_t s) {

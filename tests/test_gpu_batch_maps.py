@@ -78,3 +78,19 @@ def test_autotuned_batch_is_not_slower_than_the_built_in_choice(pairs):
     assert all(torch.equal(a, b) for a, b in zip(out[0], out[-1]))
     assert ms[-1] <= 1.25 * ms[0], ms
     ctx.close()
+
+
+def test_more_pairs_than_a_grid_dimension_holds():
+    """65,537 pairs of 2 x 1 pixels: the launches over the pairs of a batch take 65,535 at most."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    n = 65537
+    I = torch.rand(2, n, 1, 2, device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
+    I0, I1 = list(I[0]), list(I[1])
+    ctx = flow.Context(0)
+    P = flow.default_params(lam=2.0, levels=1, warps=1, iters=2)
+    us, vs, _ = flow.of_solve_batch(ctx, I0, I1, P, stats=False)
+    for k in (0, 1, 65534, 65535, 65536):
+        u, v, _, _ = flow.of_solve(ctx, I0[k], I1[k], P)
+        assert torch.equal(u, us[k]) and torch.equal(v, vs[k]), k
+    ctx.close()
