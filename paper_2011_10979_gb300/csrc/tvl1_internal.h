@@ -225,8 +225,9 @@ struct GaussTaps {
     int R;
 };
 GaussTaps gauss_taps(float eta);
-// One pyramid step of n (1 or 2) images of one geometry.  scratch: two planes of the fine geometry per
-// image, used only where a tile's fine pixels do not fit in shared memory (eta far below 1/2).
+// One pyramid step of n (1 or 2) images of one geometry.  scratch: two planes of the fine geometry, used for one
+// image after the other where the step runs as three kernels (a tile's fine pixels do not fit in shared
+// memory, eta far below 1/2; large images with eta near 1).
 void launch_pyr_down(const float *const *fine, Geom gf, float *const *coarse, Geom gc, int n, const GaussTaps &taps,
                      float *scratch, cudaStream_t s);
 void launch_upsample_f32(const float *coarse, Geom gc, float *fine, Geom gf, float scale, cudaStream_t s);

@@ -101,3 +101,15 @@ def test_pdr_on_either_tile_kernel(ctx, H, W, tol):
     ub, vb, sb = flow.of_solve_batch(ctx, [im[0]] * 2, [im[1]] * 2, P)  # one iteration per launch
     assert torch.equal(u, ub[0]) and torch.equal(v, vb[0])
     assert st["iters_run"] == sb[0]["iters_run"]
+
+
+# Pyramid steps that keep nearly all of the pixels: three kernels take the larger image and one the smaller, its upper
+# rows, with the same sampling positions in both.
+@pytest.mark.parametrize("eta", [0.95, 0.9])
+def test_pyramid_steps_that_keep_most_pixels(eta):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    big = torch.rand(1400, 1900, device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
+    a = flow.of_pyr_down(big, round(1400 * eta), round(1900 * eta), eta)
+    b = flow.of_pyr_down(big[:1300], round(1300 * eta), round(1900 * eta), eta)
+    assert torch.equal(a[:1100], b[:1100])
