@@ -63,11 +63,6 @@ __device__ __forceinline__ unsigned mask_of(bool on) {
 // x where the mask is ~0, +0 where it is 0: one logic instruction, which runs beside the FMA pipe
 // (a floating-point select does not).
 __device__ __forceinline__ float keep(float x, unsigned m) { return __uint_as_float(__float_as_uint(x) & m); }
-__device__ __forceinline__ pair2 keep2(pair2 v, unsigned m) {
-    float a, b;
-    upk(v, a, b);
-    return pk(keep(a, m), keep(b, m));
-}
 
 // Both halves rounded to storage type T and back.
 template <typename T> __device__ __forceinline__ pair2 round2(pair2 v) {

@@ -4,12 +4,13 @@
 // schedule of Sec. 4 in a captured CUDA graph.  The serving loop instead keeps a changing set of
 // requests in flight: each step advances every active pair by one stage -- one warp (one
 // linearisation) of its current pyramid level -- and the inner iterations of all of them run in
-// shared launches over a work-list rebuilt for the step: the streaming ADMM kernel's tiles (or,
-// for pDR and ALG1, one grid slice per pair) of every pair at its own level and size.  A request
+// shared launches over a work-list rebuilt for the step: the ADMM tile kernel's tiles (several
+// iterations per launch; the row-streaming kernel's with a pinned strip height or per-pixel a~; for
+// pDR and ALG1 one grid slice per pair) of every pair at its own level and size.  A request
 // that arrives joins at the next step; one that finishes its last stage leaves.  Per pair the
-// kernels and their order are those of the whole solve, so a request's flow does not depend on
-// the others in the step (the streaming kernel computes every pixel alike for any strip height
-// and work-list, and it equals the level-resident engine bitwise).
+// arithmetic and its order are those of the whole solve, so a request's flow does not depend on
+// the others in the step: every ADMM kernel computes a pixel alike, whatever its tiling, work-list,
+// iterations per launch or engine (k_admm_math.cuh), bit for bit.
 //
 // Each pair's descriptor lists its current state buffer first, so pairs whose ping-pong
 // parities differ share one launch.  Pairs in the finest level's last warp with FP32 storage
