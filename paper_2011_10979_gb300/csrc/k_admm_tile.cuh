@@ -158,15 +158,28 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
         mbar_wait(&G.full, n & 1, A.wait_ns, nullptr);
     }
 
+    // Batched form: a pair's three tensor maps.
+    static __device__ __forceinline__ const CUtensorMap *maps_of(const TileArgs &A, int pair) {
+        return A.table + 6 * pair + 3 * A.a.parity;
+    }
+    // Batched form, first warp: acquires the tensor maps of the block's tiles n to n + m - 1, a map per lane, but those
+    // of the tile before (a single pair's maps are parameters of the kernel, which need no fence).
+    static constexpr int ACQUIRED = 10;
+    static __device__ __forceinline__ void acquire_maps(const TileArgs &A, int n, int m, int lane) {
+        const int q = n + lane / 3, t = blockIdx.x + q * gridDim.x;
+        if (lane < 3 * m && t < A.ntiles) {
+            const int pair = A.a.tiles[t].pair;
+            if (lane < 3 || A.a.tiles[t - gridDim.x].pair != pair) map_acquire(maps_of(A, pair) + lane % 3);
+        }
+        __syncwarp();
+    }
+
     // Starts the copies of a tile's frame into the stage (one thread); zeros outside the image.
     static __device__ __forceinline__ void prefetch(const TileArgs &A, SH &G, char *stage, int t, int n) {
         const Tile D = tile_at(A, G, t, n);
         const CUtensorMap *maps =
-            MODE == BATCHED ? reinterpret_cast<const CUtensorMap *>(G.pi[n % 3].maps) + 3 * A.a.parity : A.maps;
+            MODE == BATCHED ? maps_of(A, G.tr[n & 3].x) : A.maps;
         const int x = D.bx * A.ow - A.offx, y = D.by * A.oh - A.offy;
-        // (a single pair's maps are parameters of the kernel, which need no fence)
-        if (MODE == BATCHED && (n == 0 || G.tr[n & 3].x != G.tr[(n - 1) & 3].x))
-            for (int k = 0; k < 3; ++k) map_acquire(maps + k);
         mbar_expect(&G.full, ST::FH * (NF * ST::WTF * (int)sizeof(TF) + (ND + 3) * ST::WT * (int)sizeof(T)));
         if (t == A.withhold) return;
         tma_load(stage + ST::flow, maps, sizeof(TF) == 4 ? x : x & ~7, y, &G.full);
@@ -233,6 +246,7 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
             __syncthreads();
             const int t1 = D.id + gridDim.x;
             if (t1 < A.ntiles) {
+                if (MODE == BATCHED && wid == 0 && (n + 1) % ACQUIRED == 0) acquire_maps(A, n + 1, ACQUIRED, lane);
                 if (threadIdx.x == 0 && !dead) prefetch(A, G, stage, t1, n + 1);
                 if (MODE == BATCHED && wid == 0) {
                     fetch_pair(A, G, n + 2, lane);
@@ -572,10 +586,12 @@ template <typename T, typename TF, bool HAS_W, int VARIANT, int NW, int R, Mode 
                 __syncwarp();
                 fetch_pair(A, G, 0, lane);
                 fetch_pair(A, G, 1, lane);
+                acquire_maps(A, 0, 1, lane);
                 cp_async_wait();
             }
             __syncthreads();
             if (threadIdx.x == 0) prefetch(A, G, stage, blockIdx.x, 0);
+            if (MODE == BATCHED && wid == 0) acquire_maps(A, 1, ACQUIRED - 1, lane);  // while the first copies arrive
         }
         int n = 0;
 #pragma unroll 1

@@ -700,7 +700,6 @@ of_status upload_tables(of_ctx *ctx, const Batch &B, const of_params *p) {
             P.timeout = &misc->timeout;
             if (B.maps_off[l][v] > 0 && !B.res[l][k]) {
                 const size_t o = B.maps_off[l][v] + 6 * sizeof(CUtensorMap) * k;
-                P.maps = ctx->arena + B.table_off + o;
                 for (int b = 0; b < 2; ++b) {
                     CUtensorMap m[3];  // aligned as the encoder asks for
                     maps_ok = maps_ok && tile_encode_maps(m, P.buf[b], P.Ix, P.Iy, P.g, v ? PREC_F32 : pl.prec,
@@ -1148,6 +1147,7 @@ void enqueue_solve(of_ctx *ctx, const Batch &B, const of_params *p, cudaStream_t
                         t.a = a;
                         tile_set_plan(t, tp, step);
                         t.vec = 1;
+                        t.table = (const CUtensorMap *)(ctx->arena + B.table_off + B.maps_off[l][in32 ? 1 : 0]);
                         launch_admm_tile(t, prec, pflow, s);
                     } else {
                         a.tiles = (const TileRef *)(ctx->arena + B.table_off + B.tiles_off[l]);
@@ -1284,6 +1284,7 @@ void launch_level_iteration(of_ctx *ctx, const Batch &B, const of_params *p, int
             t.a = a;
             tile_set_plan(t, B.tp[l], B.tp[l].ni);
             t.vec = 1;
+            t.table = (const CUtensorMap *)(ctx->arena + B.table_off + B.maps_off[l][0]);
             launch_admm_tile(t, B.pl[0].prec, B.pl[0].pflow, s);
             return;
         } else {
@@ -1698,7 +1699,6 @@ of_status of_wait_selftest(int kernel, int withhold, double wait_ms, int *timed_
             P.It = data(q, 2);
             P.ms_max = &misc_of(q)->ms_max;
             P.timeout = &misc_of(q)->timeout;
-            P.maps = D + o_tm + 6 * sizeof(CUtensorMap) * q;
             for (int b = 0; b < 2; ++b) {
                 CUtensorMap m[3];
                 maps_ok = maps_ok && tile_encode_maps(m, P.buf[b], P.Ix, P.Iy, g[q], PREC_F32, PREC_F32, true);
@@ -1709,6 +1709,7 @@ of_status of_wait_selftest(int kernel, int withhold, double wait_ms, int *timed_
         }
         t.a.pairs = (const PairIter *)(D + o_pi);
         t.a.tiles = (const TileRef *)(D + o_tr);
+        t.table = (const CUtensorMap *)(D + o_tm);
         if (e == cudaSuccess) e = cudaMemcpy(D + o_pi, img.data(), img.size(), cudaMemcpyHostToDevice);
     } else {
         t.a.g = g[0];

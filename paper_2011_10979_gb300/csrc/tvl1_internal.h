@@ -59,7 +59,6 @@ struct __align__(16) PairIter {
     const float *ms_max;
     const int *done;
     float *tmp;  // the pair's FP32 scratch planes (pDR engine)
-    const void *maps;  // tensor maps of the staged tile kernel: per buffer, flow, dual and data planes
     const float *I0, *I1;  // the level's images
     float *I1x, *I1y;      // the derivatives of I1
     int *timeout;          // set when a bounded wait left the pair unfinished
@@ -136,6 +135,7 @@ struct TileArgs {
     long long wait_ns = WAIT_NS;  // bound of every device-side wait
     int withhold = -1;    // self-test: the tile whose copies are never started
     int *tiny;            // set when a tile needed the quotients' form for any numerator
+    const CUtensorMap *table;  // work-lists: per pair and state buffer the maps of flow, dual and data planes
     CUtensorMap maps[4];  // staged form, single pair: flow, dual and data planes, Xbar (pDR)
 };
 

@@ -202,7 +202,6 @@ cudaError_t run_group(std::vector<StepPair *> &G, const of_params *p, StepTables
         pl[k] = k;
         const int t0 = t;
         if (tile) {
-            P.maps = T.dev + o_tm + 6 * sizeof(CUtensorMap) * k;
             for (int b = 0; b < 2; ++b) {
                 CUtensorMap m[3];  // aligned as the encoder asks for
                 if (!tile_encode_maps(m, P.buf[b], P.Ix, P.Iy, g, prec, pflow, has_w)) return cudaErrorUnknown;
@@ -262,6 +261,7 @@ cudaError_t run_group(std::vector<StepPair *> &G, const of_params *p, StepTables
             ta.a = a;
             tile_set_plan(ta, tp, step);
             ta.vec = 1;
+            ta.table = (const CUtensorMap *)(T.dev + o_tm);
             launch_admm_tile(ta, prec, pflow, s);
         } else {
             a.tiles = dtr;
