@@ -192,7 +192,7 @@ def run_level(args):
     engine, strip height --rows-per-warp (ADMM only; unset: the built-in rule, which on the
     streaming engine runs these levels three iterations per launch on the tile kernel, as ALG1
     does).  A pinned height runs the row-streaming kernel, whose 40x30 level shows the latency of
-    one warp's row steps; with --method pdr the 640x480 level runs the one-launch pDR tile kernel."""
+    one warp's row steps; with --method pdr the 640x480 level runs the register tile kernel."""
     import torch
     dev = torch.device("cuda", 0)
     torch.cuda.set_device(dev)
@@ -374,9 +374,9 @@ def batch_pairs(n):
 def batch_measure(flow, torch, dev, n=256, prec=None, fp32_flow=1, steps=2, engine=None, rows_per_warp=-1):
     """Uneven-size batch: n distinct pairs, each with its own seed, sizes drawn uniformly from
     {96x64, 320x240, 640x480, 1024x436, 1242x375}, affine+box motion up to 15 px, BF16 storage,
-    FP32 last warp, 5 levels x 10 warps x 100 iterations, solved with of_solve_batch (one
-    work-list launch per inner iteration for all pairs).  The streaming kernel's strip height is
-    autotuned per level on the (untimed) first solve unless rows_per_warp sets it."""
+    FP32 last warp, 5 levels x 10 warps x 100 iterations, solved with of_solve_batch (launches over
+    a work-list of all pairs).  The kernel and, on the row-streaming one, its strip height are autotuned
+    per level on the (untimed) first solve unless rows_per_warp sets the height."""
     prec = flow.OF_PREC_BF16 if prec is None else prec
     pairs = batch_pairs(n)
     I0 = [torch.from_numpy(p.I0).to(dev) for p in pairs]
@@ -594,8 +594,9 @@ def kernel_roofline(flow, torch, dev, pr, reps=20):
     CUDA graph.  On the streaming engine that level runs three inner iterations per launch
     (k_admm_tile).  Two graph-launched single-level solves of the bench pair, with 220 and 20 inner
     iterations, are timed with CUDA events on their stream; the difference / 200 is one iteration
-    (with its share of graph launch gaps), three of them one launch.  Algorithmic traffic: 13
-    planes read + 10 written, FP32 = 92 B per pixel-iteration, 276 B per pixel and launch."""
+    (with its share of graph launch gaps), three of them one launch.  Algorithmic traffic of a
+    launch: 13 planes read + 10 written, FP32 = 92 B per pixel (the state between its iterations
+    stays in registers)."""
     peaks = {}
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
@@ -623,11 +624,11 @@ def kernel_roofline(flow, torch, dev, pr, reps=20):
         t[iters] = e0.elapsed_time(e1) / reps / 1e3
     ctx.close()
     per = (t[220] - t[20]) / 200.0 * ITERS_PER_LAUNCH   # one launch = three iterations
-    bytes_per_launch = ITERS_PER_LAUNCH * 92.0 * H * W
+    bytes_per_launch = 92.0 * H * W
     achieved = bytes_per_launch / per / 1e9
     # the level's working set stays in L2: its bandwidth for a working set of the same size
     # (half read, half written, streamed 400 times in one launch)
-    l2 = flow.of_l2_bandwidth(int(bytes_per_launch / ITERS_PER_LAUNCH), 400)
+    l2 = flow.of_l2_bandwidth(int(bytes_per_launch), 400)
     return {"kernel": "k_admm_tile<float,float,1,0,12,4,DIRECT> (640x480 level, three iterations per launch)",
             "bound": "hbm", "achieved": achieved,
             "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_source": src,
@@ -635,10 +636,8 @@ def kernel_roofline(flow, torch, dev, pr, reps=20):
             "us_per_iteration": per * 1e6 / ITERS_PER_LAUNCH, "algorithmic_bytes_per_launch": bytes_per_launch,
             "timing": "graph-launched single-level solves, (t(220 iters) - t(20 iters)) / 200 x 3 per launch",
             "l2_peak": l2, "frac_of_l2": achieved / l2,
-            "state_bytes_per_launch": bytes_per_launch / ITERS_PER_LAUNCH,
-            "frac_of_state_bytes": achieved / ITERS_PER_LAUNCH / peak,
-            "note": "frac counts every iteration's algorithmic bytes, of which a launch of three iterations moves one "
-                    "iteration's (frac_of_state_bytes), the rest staying in registers; "
+            "gbs_counting_every_iteration": ITERS_PER_LAUNCH * achieved,
+            "note": "a launch reads and writes the state once for three iterations, which frac counts; "
                     "the 640x480 level's 28 MB state stays in the 129 MB L2 between iterations; l2_peak is the "
                     "library's L2 streaming probe over a 28 MB read+write working set"}
 

@@ -28,7 +28,7 @@
 // Bound by latency and issue with three warps per SM quarter (some 240 clocks per row and warp), beside
 // 4 to 6 us per launch for instruction fetch and the state's loads and stores.  Measured per iteration,
 // and in brackets with the frame in shared memory and scalar instructions, which this replaced:
-// 640x480 2.83 us (4.51), 320x240 1.30 (1.87), 160x120 1.09 (1.32), 3840x2160 75 (114).
+// 640x480 2.65 us (4.54), 320x240 1.22 (1.87), 160x120 1.07 (1.32), 3840x2160 76 (115).
 #pragma once
 #include <math.h>
 

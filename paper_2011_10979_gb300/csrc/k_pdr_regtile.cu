@@ -4,8 +4,8 @@
 
 namespace tvl1 {
 
-// Microseconds of a launch of k iterations, fitted to launches of one round: 640x480, one iteration, 10.8 us;
-// 320x240, five, 21.6.
+// Microseconds of a launch of k iterations, fitted to launches of one round before the divisions left the usual body
+// (640x480, one iteration, 10.8 us; 320x240, five, 21.6; now 9.0 and 19.4, both a tenth or so less).
 float pdr_regtile_us(const TilePlan &p, int k) {
     const int rounds = (p.gx * p.gy + TILE_SMS - 1) / TILE_SMS;
     return 0.4f + rounds * (7.7f + 2.7f * k);

@@ -26,13 +26,13 @@
 // flat 3.41 (6.81, 3.84), a textured box on an empty background 3.35 (7.28, 3.86).
 //
 // What bounds it: with one iteration per launch, the state's traffic through L2 (184 KB in and 147 KB out
-// per SM: some 8 us of a launch's 10.8 at 640x480), and per iteration issue and latency with three warps
-// per SM quarter (some 330 instructions per row of a warp; 2.7 us).  A tile on the image's border costs
+// per SM) and the fetch of straight-line code, most of a launch's 9.0 us at 640x480, and per iteration issue and
+// latency with three warps per SM quarter (some 330 instructions per row of a warp).  A tile on the image's border costs
 // no more than the others, since a launch of one round is as slow as its slowest tile: pixels outside
 // have a zero reciprocal, which keeps X zero there, and ybar is zero across the border (masks and
-// branches instead: 11.8 us at 640x480).  Pairs of rows in packed arithmetic took more moves than it saved.
-// Measured per iteration, in brackets k_pdr_tile: 240x180 4.2 us (5.6), 320x240 4.3 (5.8), 640x480 10.8
-// (13.4), 1024x436 12.3 (19.3), 3840x2160 199 (333).
+// branches instead: 1.0 us more at 640x480).  Pairs of rows in packed arithmetic took more moves than it saved.
+// Measured per iteration, in brackets k_pdr_tile: 240x180 3.8 us (5.6), 320x240 3.9 (5.8), 640x480 9.0
+// (13.4), 1024x436 10.5 (19.3), 3840x2160 188 (335).
 #pragma once
 #include <cuda.h>
 #include <math.h>

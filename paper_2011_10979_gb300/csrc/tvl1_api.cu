@@ -327,7 +327,7 @@ std::vector<int> pdr_launches(int ni, int iters, bool tested, bool last_warp) {
 
 // Whether a single pair's streamed pDR level runs on the register tile kernel (k_pdr_regtile.cuh) rather than on the
 // one-iteration tile kernel of k_pdr.cu.  Levels from 40,000 pixels (measured per iteration, register tiles
-// against it: 4.5 / 4.4 us at 213x160, 4.2 / 5.6 at 240x180, 4.3 / 5.8 at 320x240), with the stopping test, whose
+// against it: 4.5 / 4.4 us at 213x160, 3.8 / 5.6 at 240x180, 3.9 / 5.8 at 320x240), with the stopping test, whose
 // tested iterations are launches of their own, from 60,000 but for strips (7.0 / 6.5 at 201x200), where the
 // estimated time is the smaller: the one-iteration kernel takes some 6.2 us per wave of 32 x 32 tiles over the SMs, less on strips that
 // leave most of a tile's rows outside the image (20000x2: 15.4 / 13.2 us; 32768x8: 23.7 / 20.9; 5000x8: 4.8 / 7.0),
