@@ -64,12 +64,15 @@ typedef enum { OF_PREC_FP32 = 0, OF_PREC_FP16 = 1, OF_PREC_BF16 = 2 } of_precisi
 typedef enum {
     OF_ENGINE_FUSED = 0,    /* default: small levels (those the level-resident launch runs faster)
                                run all inner iterations of a warp in one level-resident launch of
-                               a thread-block cluster; the others one fused streaming kernel per
-                               inner iteration.  Both give bitwise the same flow. */
+                               a thread-block cluster; the others fused kernels that run several
+                               inner iterations per launch, or one.  All give bitwise the same
+                               flow. */
     OF_ENGINE_PLAIN = 1,    /* one kernel per operator, FP32 only: the plain reference GPU path */
-    OF_ENGINE_STREAM = 2,   /* the fused streaming kernel on every level */
+    OF_ENGINE_STREAM = 2,   /* those fused kernels on every level, at a fixed three iterations per
+                               launch where they run several (no level-resident launch) */
     OF_ENGINE_RESIDENT = 3, /* the level-resident launch on every level that fits one cluster's
-                               shared memory, the streaming kernel on the others */
+                               shared memory, the fused kernels of one iteration per launch on
+                               the others */
     OF_ENGINE_PERSISTENT = 4 /* ADMM methods: levels that the default engine does not run
                                level-resident run every inner iteration of a warp in one
                                persistent launch over all pairs of the level, whose warps
@@ -193,7 +196,9 @@ long long of_solve_kernel_count(of_ctx *ctx, int H, int W, const of_params *para
  * per-iteration kernels) in a solve of n pairs of sizes H[k] x W[k] (n = 1: of_solve; n > 1:
  * of_solve_batch) with these parameters: rows[l] for l in [0, params->levels) is the height used on
  * pyramid level l, 0 where no pair of that level runs on those kernels (a level-resident or
- * persistent launch, pDR's one-launch tile kernel, the plain engine, or a level below out_level).  With params->rows_per_warp = -1 it runs the autotuner first if this layout is not
+ * persistent launch, pDR's tile kernels, the plain engine, or a level below out_level); a level on a
+ * tile kernel of several iterations per launch reports the height that the built-in rule would take
+ * otherwise.  With params->rows_per_warp = -1 it runs the autotuner first if this layout is not
  * tuned on the context yet (allocating the arena and launching kernels; the device is
  * synchronised).  `rows` is caller-owned host memory of params->levels ints.  OF_EINVAL for bad
  * arguments, OF_ENOMEM / OF_ECUDA as for of_solve_batch. */
@@ -303,9 +308,9 @@ typedef struct {
 /* `iters` inner iterations of rpADMMI / rpADMMII (params->method 0 or 1) at a fixed
  * linearisation (Sec. 3.1.1), in place on `f`.  a_tilde > 0 is used as given.  The stopping
  * rule params->tol applies.  res2: optional host pointer, receives ||A s + B y||^2 after the
- * last iteration (synchronises).  Uses params->engine: PLAIN, or the fused streaming kernel
- * (FUSED and STREAM alike: this call has no level-resident form); the fused kernel
- * needs `scratch`, a device buffer of >= of_fields_bytes(H, pitch) bytes (NULL for PLAIN). */
+ * last iteration (synchronises).  Uses params->engine: PLAIN, or the fused kernels
+ * (FUSED and STREAM alike: this call has no level-resident form); planes that the method does not
+ * use are left alone.  The fused kernels need `scratch`, a device buffer of >= of_fields_bytes(H, pitch) bytes (NULL for PLAIN). */
 of_status of_admm_iterate(of_fields f, const float *Ix, const float *Iy, const float *It, int H,
                           int W, int pitch, float a_tilde, const of_params *params, int iters,
                           void *scratch, double *res2, void *stream);
